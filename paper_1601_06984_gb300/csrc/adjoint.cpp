@@ -474,7 +474,7 @@ lbm_status lbm_adjoint(lbm_ctx* c, int64_t n, int32_t K, int32_t objective, void
       m.elem = c->at<int32_t>(c->ld[lc].src_elem);
       m.Ntot = (int64_t)N;
       m.nsrc = c->ld[lc].nsrc;
-      m.omega = Hc.omega;
+      m.rx = make_relax(c->Q, Hc.omega);
       m.rho_off = c->rho_off;
       m.src = snap(sa);
       m.mom = W + L.recA[lc];

@@ -469,13 +469,13 @@ __global__ void __launch_bounds__(256, LBM_ADJ_MINB(S, LBM_ADJ_SC_MINB, 2)) k_ad
 // pdfs' adjoints back into those slots; interior bricks have no boundary
 // links.  Grid: ceil(nB / 4) blocks of 256, block b adding its sums to running
 // row b.
-static_assert(LBM_BR_BLOCK / 64 == LBM_BRICKS_PER_BLOCK, "host sizes the running rows by this many bricks per block");
+constexpr int kAdjBrBlock = 64 * LBM_BRICKS_PER_BLOCK;  // the host sizes the running rows by this many bricks per block
 template <int Q, class S>
-__global__ void __launch_bounds__(LBM_BR_BLOCK, LBM_ADJ_MINB(S, LBM_ADJ_BRICK_MINB, 2)) k_adj_sc_brick(const AdjSCArgs a) {
+__global__ void __launch_bounds__(kAdjBrBlock, LBM_ADJ_MINB(S, LBM_ADJ_BRICK_MINB, 2)) k_adj_sc_brick(const AdjSCArgs a) {
   using R = typename Sto<S>::R;
   using LT = Lat<Q>;
   constexpr int D = LT::D;
-  constexpr int BPB = LBM_BR_BLOCK / 64;
+  constexpr int BPB = LBM_BRICKS_PER_BLOCK;
   constexpr int NW = Q / 2;  // (Q-1)/2 words of two 16-bit entries
   const int l = threadIdx.x & 63, lane = threadIdx.x & 31;
   // the brick index is uniform over each warp, so the shuffles run with whole warps
@@ -952,7 +952,7 @@ struct AdjLaunch {
   static void sc_brick(int Q, const AdjSCArgs& a, cudaStream_t st) {
     if (a.nB <= 0) return;
     const unsigned g = (unsigned)((a.nB + LBM_BRICKS_PER_BLOCK - 1) / LBM_BRICKS_PER_BLOCK);
-    with_q(Q, [&](auto q) { k_adj_sc_brick<decltype(q)::value, S><<<g, LBM_BR_BLOCK, 0, st>>>(a); });
+    with_q(Q, [&](auto q) { k_adj_sc_brick<decltype(q)::value, S><<<g, kAdjBrBlock, 0, st>>>(a); });
   }
   static void outlet(int Q, const AdjOutletArgs& a, cudaStream_t st) {
     // the normal-link pass writes one row of omega partials per block, so it

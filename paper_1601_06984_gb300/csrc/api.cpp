@@ -100,7 +100,7 @@ void lbm_ctx::fill_gff(int li) {
   a.dst = cur(li);
   a.Ntot = M.Ntot;
   a.omega_c = H.omega;
-  a.omega_f = Hf.omega;
+  a.rx_f = make_relax(Q, Hf.omega);
   a.rho_off = rho_off;
   // fine -> coarse lattice units: u_c = (dt_c / dt_f) / 2 u_f, the density
   // deviation with the square of that factor (1 in acoustic scaling)
@@ -109,6 +109,7 @@ void lbm_ctx::fill_gff(int li) {
   a.r_scale = a.u_scale * a.u_scale;
   a.r_shift = (1.0 - a.r_scale) * (p.rho0 - rho_off);
   a.odd_ratio = odd_fneq_ratio(p.time_mode, true);
+  a.scale = (1.0 - H.omega) * a.tratio * Hf.omega / H.omega / (1 << d);
   timed_launch(li, TK_GFF, [&] { ops->fill_gff(Q, a, st); });
   ++launches;
 }
@@ -132,7 +133,7 @@ void lbm_ctx::source_moments(int li, size_t mom_off, size_t prev_off, cudaStream
   a.prev = prev_off ? at(prev_off) : nullptr;
   a.Ntot = M.Ntot;
   a.nsrc = n;
-  a.omega = M.lv[li].omega;
+  a.rx = make_relax(Q, M.lv[li].omega);
   a.rho_off = rho_off;
   timed_launch(li, TK_MOM, [&] { ops->source_moments(Q, a, s); }, s);
   ++launches;
@@ -165,6 +166,7 @@ void lbm_ctx::fill_gfc(int lf, bool two_times, bool all_layers, cudaStream_t s, 
   a.r_scale = a.u_scale * a.u_scale;
   a.r_shift = (1.0 - a.r_scale) * (p.rho0 - rho_off);
   a.odd_ratio = odd_fneq_ratio(p.time_mode, false);
+  a.scale = (1.0 - a.omega_f) * a.omega_c / (a.tratio * a.omega_f);
   timed_launch(lf, TK_GFC, [&] { ops->fill_gfc(Q, a, s); }, s);
   ++launches;
 }
@@ -206,7 +208,7 @@ void lbm_ctx::stream_collide(int li, cudaStream_t s0) {
   b.Ntot = M.Ntot;
   b.begin = H.base + H.oF;
   b.nB = H.nB;
-  b.omega = H.omega;
+  b.rx = make_relax(Q, H.omega);
   b.rho_off = rho_off;
   b.nbr = at<uint32_t>(oNbr);
   b.side = at(oSide);
@@ -247,7 +249,7 @@ void lbm_ctx::stream_collide(int li, cudaStream_t s0) {
     a.hole_at = a.end;
     a.hole_len = 0;
   }
-  a.omega = H.omega;
+  a.rx = b.rx;
   a.rho_off = rho_off;
   std::memcpy(a.inlet, b.inlet, sizeof(a.inlet));
   a.so = so;

@@ -237,6 +237,174 @@ __device__ __forceinline__ void post_moments(const R* g, R omega, R rho_off, con
   }
 }
 
+// ----------------------------------------------------------------- FP64 arithmetic
+// GB300 issues an FP64 instruction of a warp over about 19 cycles of its SM,
+// so the FP64 kernels are bound by the number of FP64 instructions, and these
+// forms of the moments, the collision and post_moments are written for fewest
+// of them: c.j instead of c.u (one reciprocal, no velocity), every uniform
+// factor a constant operand (Relax), each pair of opposite velocities as two
+// fused multiply-adds on its two values, signs flipped on the integer pipe.
+// With one-warp blocks (kScBlock), per coarse step of two-level flows: forced
+// D3Q19, 1.5e5 elements, 293 -> 211 us; D2Q9, 1,800 elements, 67 -> 47 us.
+template <int Q>
+__host__ __device__ constexpr int wclass(int i) {
+  return Lat<Q>::c(i, 0) * Lat<Q>::c(i, 0) + Lat<Q>::c(i, 1) * Lat<Q>::c(i, 1) + Lat<Q>::c(i, 2) * Lat<Q>::c(i, 2);
+}
+
+// x with its sign flipped when `neg`
+__device__ __forceinline__ double flip(double x, bool neg) {
+  return __hiloint2double(__double2hiint(x) ^ (neg ? (int)0x80000000 : 0), __double2loint(x));
+}
+
+// sum of the pdfs and first moment: the x moment shares its two half sums
+// with the total, the other axes take the differences of opposite pdfs
+template <int Q>
+__device__ __forceinline__ void raw_moments64(const double* g, double& rp, double* j) {
+  using LT = Lat<Q>;
+  double sp = 0, sm = 0, s0 = g[0];
+#pragma unroll
+  for (int i = 1; i < Q; ++i) {
+    if (LT::c(i, 0) > 0) sp += g[i];
+    else if (LT::c(i, 0) < 0) sm += g[i];
+    else s0 += g[i];
+  }
+  rp = (sp + sm) + s0;
+  j[0] = sp - sm;
+  j[1] = j[2] = 0;
+#pragma unroll
+  for (int i = 1; i < Q; i += 2) {
+    if (LT::c(i, 1) == 0 && LT::c(i, 2) == 0) continue;
+    const double m = g[i] - g[i + 1];
+#pragma unroll
+    for (int a = 1; a < LT::D; ++a) {
+      if (LT::c(i, a) > 0) j[a] += m;
+      if (LT::c(i, a) < 0) j[a] -= m;
+    }
+  }
+}
+
+// c_i . v
+template <int Q>
+__device__ __forceinline__ double cdot(int i, const double* v) {
+  using LT = Lat<Q>;
+  double s = 0;
+#pragma unroll
+  for (int a = 0; a < LT::D; ++a) {
+    if (LT::c(i, a) > 0) s += v[a];
+    if (LT::c(i, a) < 0) s -= v[a];
+  }
+  return s;
+}
+
+// BGK collision of one element in place (bgk_collide): with J = rho u,
+//   g_i := (1 - omega) g_i + omega w [rp - 3/2 J.J / rho + 9/2 (c.J)^2 / rho + 3 c.J] + Guo
+template <int Q, bool FORCE>
+__device__ __forceinline__ void bgk_collide64(double (&g)[Q], const Relax& rx, double rho_off, const double* F) {
+  using LT = Lat<Q>;
+  constexpr int D = LT::D, NC = Q == 27 ? 4 : 3;
+  double rp, J[3];
+  raw_moments64<Q>(g, rp, J);
+  if (FORCE) {
+#pragma unroll
+    for (int a = 0; a < D; ++a) J[a] = fma(0.5, F[a], J[a]);
+  }
+  const double inv = 1.0 / (rho_off + rp);
+  double jj = 0, jF = 0;
+#pragma unroll
+  for (int a = 0; a < D; ++a) {
+    jj = fma(J[a], J[a], jj);
+    if (FORCE) jF = fma(J[a], F[a], jF);
+  }
+  const double base = fma(-1.5 * inv, jj, rp);
+  const double uF = FORCE ? jF * inv : 0.0;
+  double b[NC], kq[NC], kf[NC];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) {
+    b[c] = FORCE ? fma(rx.eq[c], base, -rx.force[c] * uF) : rx.eq[c] * base;
+    kq[c] = c ? rx.quad[c] * inv : 0.0;
+    kf[c] = FORCE && c ? 3.0 * rx.force[c] * inv : 0.0;
+  }
+  g[0] = fma(rx.keep, g[0], b[0]);
+#pragma unroll
+  for (int i = 1; i < Q; i += 2) {
+    const int c = wclass<Q>(i);
+    const double cJ = cdot<Q>(i, J);
+    if (FORCE) {
+      const double cF = cdot<Q>(i, F);
+      const double ev = fma(cJ, fma(kq[c], cJ, kf[c] * cF), b[c]);
+      const double od = fma(rx.lin[c], cJ, rx.force[c] * cF);
+      g[i] = fma(rx.keep, g[i], ev + od);
+      g[i + 1] = fma(rx.keep, g[i + 1], ev - od);
+    } else {
+      const double ev = fma(kq[c] * cJ, cJ, b[c]);
+      g[i] = fma(rx.keep, g[i], fma(rx.lin[c], cJ, ev));
+      g[i + 1] = fma(rx.keep, g[i + 1], fma(-rx.lin[c], cJ, ev));
+    }
+  }
+}
+
+// post_moments with the strain rate
+template <int Q, bool FORCE>
+__device__ __forceinline__ void post_moments64(const double* g, const Relax& rx, double rho_off, const double* F,
+                                               double& rp, double* u, double* fneq, double* S) {
+  using LT = Lat<Q>;
+  constexpr int D = LT::D, NS = LT::NS, NC = Q == 27 ? 4 : 3;
+  double J[3];
+  raw_moments64<Q>(g, rp, J);
+  if (FORCE) {
+#pragma unroll
+    for (int a = 0; a < D; ++a) J[a] = fma(-0.5, F[a], J[a]);
+  }
+  const double inv = 1.0 / (rho_off + rp);
+  double jj = 0, uF = 0;
+  u[0] = u[1] = u[2] = 0;
+#pragma unroll
+  for (int a = 0; a < D; ++a) {
+    u[a] = J[a] * inv;
+    jj = fma(J[a], u[a], jj);
+    if (FORCE) uF = fma(u[a], F[a], uF);
+  }
+  const double base = fma(-1.5, jj, rp);
+  double b[NC], kq[NC], kf[NC];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) {
+    b[c] = FORCE ? fma(rx.nforce[c], uF, -rx.neq[c] * base) : -rx.neq[c] * base;
+    kq[c] = c ? -rx.nquad[c] * inv : 0.0;
+    kf[c] = FORCE && c ? -3.0 * rx.nforce[c] * inv : 0.0;
+  }
+  fneq[0] = fma(rx.r1w, g[0], b[0]);
+#pragma unroll
+  for (int s = 0; s < NS; ++s) S[s] = 0;
+#pragma unroll
+  for (int i = 1; i < Q; i += 2) {
+    const int c = wclass<Q>(i);
+    const double cJ = cdot<Q>(i, J);
+    if (FORCE) {
+      const double cF = cdot<Q>(i, F);
+      const double ev = fma(cJ, fma(kq[c], cJ, kf[c] * cF), b[c]);
+      const double od = fma(rx.nlin[c], cJ, rx.nforce[c] * cF);
+      fneq[i] = fma(rx.r1w, g[i], ev - od);
+      fneq[i + 1] = fma(rx.r1w, g[i + 1], ev + od);
+    } else {
+      const double ev = fma(kq[c] * cJ, cJ, b[c]);
+      fneq[i] = fma(rx.r1w, g[i], fma(-rx.nlin[c], cJ, ev));
+      fneq[i + 1] = fma(rx.r1w, g[i + 1], fma(rx.nlin[c], cJ, ev));
+    }
+    const double ps = fneq[i] + fneq[i + 1];
+#pragma unroll
+    for (int a = 0; a < D; ++a)
+#pragma unroll
+      for (int e = a; e < D; ++e) {
+        const int cc = LT::c(i, a) * LT::c(i, e);
+        if (cc > 0) S[sidx<D>(a, e)] += ps;
+        if (cc < 0) S[sidx<D>(a, e)] -= ps;
+      }
+  }
+  const double pre = rx.strain * inv;
+#pragma unroll
+  for (int s = 0; s < NS; ++s) S[s] *= pre;
+}
+
 // ----------------------------------------------------------------- GFC source records
 // Record of one source (compute type, mom_stride(Q) values, 16-byte aligned
 // groups): f^neq[Q] padded to a multiple of 4, then rho - rho_off, u[D], S[nS],
@@ -278,14 +446,15 @@ __device__ __forceinline__ void st4(double* p, const double* v) {
 // Interpolation step 1 (Sec. 2.2) for one source: its record from its stored
 // (post-collision) pdfs g.
 template <int Q, class R, bool FORCE>
-__device__ __forceinline__ void source_record(const R (&g)[Q], R omega, R rho_off, const R* F,
+__device__ __forceinline__ void source_record(const R (&g)[Q], const Relax& rx, R rho_off, const R* F,
                                               R (&rec)[RecLayout<Q>::STRIDE]) {
   using RL = RecLayout<Q>;
   constexpr int D = Lat<Q>::D, NS = Lat<Q>::NS;
 #pragma unroll
   for (int f = 0; f < RL::STRIDE; ++f) rec[f] = R(0);
   R rp, u[3], fneq[Q], Sv[NS];
-  post_moments<Q, R, true, FORCE>(g, omega, rho_off, F, rp, u, fneq, Sv);
+  if constexpr (sizeof(R) == 8) post_moments64<Q, FORCE>(g, rx, rho_off, F, rp, u, fneq, Sv);
+  else post_moments<Q, R, true, FORCE>(g, R(rx.omega), rho_off, F, rp, u, fneq, Sv);
 #pragma unroll
   for (int q = 0; q < Q; ++q) rec[RL::FN + q] = fneq[q];
   rec[RL::RP] = rp;
@@ -321,7 +490,7 @@ __device__ __forceinline__ void store_record(R* __restrict__ out, const R (&rec)
 // slots: one broadcast load for a warp of consecutive elements.
 template <int Q, class S, bool FORCE>
 __device__ __forceinline__ void source_out(const SourceOut& so, int64_t e, const typename Sto<S>::R (&g)[Q],
-                                           typename Sto<S>::R omega, typename Sto<S>::R rho_off,
+                                           const Relax& rx, typename Sto<S>::R rho_off,
                                            const typename Sto<S>::R* F) {
   using R = typename Sto<S>::R;
   using RL = RecLayout<Q>;
@@ -336,19 +505,15 @@ __device__ __forceinline__ void source_out(const SourceOut& so, int64_t e, const
     gs[q] = Sto<S>::ld(&v);
   }
   R rec[RL::STRIDE];
-  source_record<Q, R, FORCE>(gs, omega, rho_off, F, rec);
+  source_record<Q, R, FORCE>(gs, rx, rho_off, F, rec);
   store_record<Q, R>(static_cast<R*>(so.rec_out) + k * RL::STRIDE, rec);
 }
 
 // ----------------------------------------------------------------- stream + collide
 // Tuning knobs of the hot kernel (compile-time; the defaults are the measured
-// best on GB300).  LBM_SC_EPT: elements per thread; LBM_SC_BLOCK: threads per
-// block; LBM_SC_MINB: minimum resident blocks per SM for __launch_bounds__;
-// LBM_SC_STREAM: streaming (evict-first) hints on the use-once neighbour
-// indices and on the stores.
-#ifndef LBM_SC_EPT
-#define LBM_SC_EPT 1
-#endif
+// best on GB300).  LBM_SC_BLOCK: threads per block; LBM_SC_MINB: minimum
+// resident blocks per SM for __launch_bounds__; LBM_SC_STREAM: streaming
+// (evict-first) hints on the use-once neighbour indices and on the stores.
 #ifndef LBM_SC_BLOCK
 #define LBM_SC_BLOCK 256
 #endif
@@ -358,6 +523,15 @@ __device__ __forceinline__ void source_out(const SourceOut& so, int64_t e, const
 #ifndef LBM_SC_STREAM
 #define LBM_SC_STREAM 1
 #endif
+// FP64 storage: one warp per block.  A warp holds its SM's FP64 pipe for about
+// 120 x 19 cycles, so a launch takes as long as the SM with the most warps,
+// and small blocks spread a small level over all SMs (D2Q9, 1,800 elements:
+// 7 blocks of 256 on 7 SMs before).  Registers are not capped: 12 to 24 warps
+// per SM keep the pipe busy, and the caps of 64 and 80 registers spilled.
+template <class S>
+constexpr int kScBlock = sizeof(S) == 8 ? 32 : LBM_SC_BLOCK;
+template <int Q, class S>
+constexpr int kScMinb = sizeof(S) == 8 ? (Q == 27 ? 12 : Q == 19 ? 16 : 24) : LBM_SC_MINB;
 
 __device__ __forceinline__ uint32_t ld_once(const uint32_t* p) {
 #if LBM_SC_STREAM
@@ -392,9 +566,14 @@ __device__ __forceinline__ void st_once(__nv_bfloat16* p, __nv_bfloat16 v) {
 // symmetry of each velocity pair (i, opp(i)): c.u and c.F change sign, so the
 // even part of f^eq (and of the forcing term) is shared and the odd part flips.
 template <int Q, class R, bool FORCE>
-__device__ __forceinline__ void bgk_collide(R (&g)[Q], R om, R rho_off, const R* F) {
+__device__ __forceinline__ void bgk_collide(R (&g)[Q], const Relax& rx, R rho_off, const R* F) {
   using LT = Lat<Q>;
   constexpr int D = LT::D;
+  if constexpr (sizeof(R) == 8) {
+    bgk_collide64<Q, FORCE>(g, rx, rho_off, F);
+    return;
+  }
+  const R om = R(rx.omega);
   R rp, j[3];
   raw_moments<Q, R>(g, rp, j);
   const R rho = rho_off + rp;
@@ -452,73 +631,51 @@ __device__ __forceinline__ void bgk_collide(R (&g)[Q], R om, R rho_off, const R*
 // a plain pull read the element's own opposite slot, which is the bounce-back
 // value), and patches the rare inlet / outlet values afterwards, so that up to
 // 2(Q-1) independent loads per element are in flight.
-template <int Q, class S, bool FORCE, int EPT, bool MOMS>
-__global__ void __launch_bounds__(LBM_SC_BLOCK, LBM_SC_MINB) k_stream_collide(const StreamCollideArgs a) {
+template <int Q, class S, bool FORCE, bool MOMS>
+__global__ void __launch_bounds__(kScBlock<S>, kScMinb<Q, S>) k_stream_collide(const StreamCollideArgs a) {
   using R = typename Sto<S>::R;
   using LT = Lat<Q>;
   constexpr int D = LT::D;
-  const int64_t l0 = a.begin + (int64_t)blockIdx.x * (LBM_SC_BLOCK * EPT) + threadIdx.x;
+  // linear position -> element, stepping over the interior bricks
+  const int64_t lin = a.begin + (int64_t)blockIdx.x * kScBlock<S> + threadIdx.x;
+  if (lin >= a.end) return;
+  const int64_t e = lin + (lin >= a.hole_at ? a.hole_len : 0);
   const S* __restrict__ src = static_cast<const S*>(a.src);
   S* __restrict__ dst = static_cast<S*>(a.dst);
   const uint32_t* __restrict__ nbr = a.nbr;
   const size_t N = (size_t)a.Ntot;
-  // linear position -> element, stepping over the interior bricks; linear
-  // positions at or past a.end are idle
-  int64_t el[EPT];
+  uint32_t nb[Q - 1];
 #pragma unroll
-  for (int k = 0; k < EPT; ++k) {
-    const int64_t lin = l0 + k * LBM_SC_BLOCK;
-    el[k] = lin >= a.end ? -1 : lin + (lin >= a.hole_at ? a.hole_len : 0);
+  for (int i = 1; i < Q; ++i) nb[i - 1] = ld_once(nbr + (size_t)(i - 1) * N + e);
+  R g[Q];
+  g[0] = Sto<S>::ld(src + e);
+#pragma unroll
+  for (int i = 1; i < Q; ++i) {
+    const uint32_t n = nb[i - 1];
+    const size_t idx = n < NB_FLAG30 ? (size_t)i * N + n : (size_t)opp(i) * N + (size_t)e;
+    g[i] = Sto<S>::ld(src + idx);
   }
-  uint32_t nb[EPT][Q - 1];
 #pragma unroll
-  for (int k = 0; k < EPT; ++k) {
-    const int64_t e = el[k];
-    if (e >= 0) {
-#pragma unroll
-      for (int i = 1; i < Q; ++i) nb[k][i - 1] = ld_once(nbr + (size_t)(i - 1) * N + e);
-    }
-  }
-  R g[EPT][Q];
-#pragma unroll
-  for (int k = 0; k < EPT; ++k) {
-    const int64_t e = el[k];
-    if (e >= 0) {
-      g[k][0] = Sto<S>::ld(src + e);
-#pragma unroll
-      for (int i = 1; i < Q; ++i) {
-        const uint32_t n = nb[k][i - 1];
-        const size_t idx = n < NB_FLAG30 ? (size_t)i * N + n : (size_t)opp(i) * N + (size_t)e;
-        g[k][i] = Sto<S>::ld(src + idx);
+  for (int i = 1; i < Q; ++i) {
+    const uint32_t n = nb[i - 1];
+    if (n >= NB_FLAG30) {
+      if (n & NB_BOUNCE) {
+        if (n & NB_FLAG30) g[i] += R(a.inlet[i]) * (a.inlet_s ? R(a.inlet_s[n & NB_INDEX]) : R(1));
+      } else {
+        g[i] = static_cast<const R*>(a.side)[n & NB_INDEX];
       }
     }
   }
+  R F[3] = {R(0), R(0), R(0)};
+  if (FORCE) {
+    const R* __restrict__ fp = static_cast<const R*>(a.force);
 #pragma unroll
-  for (int k = 0; k < EPT; ++k) {
-    const int64_t e = el[k];
-    if (e < 0) continue;
-#pragma unroll
-    for (int i = 1; i < Q; ++i) {
-      const uint32_t n = nb[k][i - 1];
-      if (n >= NB_FLAG30) {
-        if (n & NB_BOUNCE) {
-          if (n & NB_FLAG30) g[k][i] += R(a.inlet[i]) * (a.inlet_s ? R(a.inlet_s[n & NB_INDEX]) : R(1));
-        } else {
-          g[k][i] = static_cast<const R*>(a.side)[n & NB_INDEX];
-        }
-      }
-    }
-    R F[3] = {R(0), R(0), R(0)};
-    if (FORCE) {
-      const R* __restrict__ fp = static_cast<const R*>(a.force);
-#pragma unroll
-      for (int b = 0; b < D; ++b) F[b] = fp[(size_t)b * N + e];
-    }
-    bgk_collide<Q, R, FORCE>(g[k], R(a.omega), R(a.rho_off), F);
-#pragma unroll
-    for (int i = 0; i < Q; ++i) st_once(dst + (size_t)i * N + e, Sto<S>::cv(g[k][i]));
-    if (MOMS) source_out<Q, S, FORCE>(a.so, e, g[k], R(a.omega), R(a.rho_off), F);
+    for (int b = 0; b < D; ++b) F[b] = fp[(size_t)b * N + e];
   }
+  bgk_collide<Q, R, FORCE>(g, a.rx, R(a.rho_off), F);
+#pragma unroll
+  for (int i = 0; i < Q; ++i) st_once(dst + (size_t)i * N + e, Sto<S>::cv(g[i]));
+  if (MOMS) source_out<Q, S, FORCE>(a.so, e, g, a.rx, R(a.rho_off), F);
 }
 
 // Stream-collide of interior bricks: the same pull and BGK collision as
@@ -536,7 +693,7 @@ __global__ void __launch_bounds__(LBM_SC_BLOCK, LBM_SC_MINB) k_stream_collide(co
 #define LBM_BR_BLOCK 256
 #endif
 #ifndef LBM_BR_MINB
-#define LBM_BR_MINB 4
+#define LBM_BR_MINB (4 * 256 / LBM_BR_BLOCK)
 #endif
 //
 // Boundary bricks (BND): a complete brick whose neighbour brick behind some
@@ -546,28 +703,34 @@ __global__ void __launch_bounds__(LBM_SC_BLOCK, LBM_SC_MINB) k_stream_collide(co
 // Every link is first resolved to one 32-bit offset, so the gathers need no
 // branch.  Five blocks per SM (48 registers, no spills) for D3Q19 and D2Q9
 // with 4-byte or narrower storage (measured: 4.66 against 4.38 TB/s at four);
-// three where more registers are needed (D3Q27, FP64).
+// three where more registers are needed (D3Q27).
 #ifndef LBM_BR_BND_MINB_NARROW
 #define LBM_BR_BND_MINB_NARROW 5
 #endif
-#define LBM_BR_BND_MINB(Q, S) ((Q) > 19 || sizeof(S) > 4 ? 3 : LBM_BR_BND_MINB_NARROW)
+#define LBM_BR_BND_MINB(Q, S) ((Q) > 19 ? 3 * 256 / LBM_BR_BLOCK : LBM_BR_BND_MINB_NARROW * 256 / LBM_BR_BLOCK)
 // Interior bricks: BF16 storage moves half the bytes per element, so it needs
 // more elements in flight; five blocks per SM (48 registers, no spills) for
 // D3Q19 / D2Q9 BF16, measured faster than four or six.
-#define LBM_BR_INT_MINB(Q, S) ((Q) <= 19 && sizeof(S) == 2 ? 5 : LBM_BR_MINB)
-#define LBM_BR_MOMS_MINB(Q, S) ((Q) <= 19 && sizeof(S) <= 4 ? 5 : LBM_BR_MINB)
+#define LBM_BR_INT_MINB(Q, S) ((Q) <= 19 && sizeof(S) == 2 ? 5 * 256 / LBM_BR_BLOCK : LBM_BR_MINB)
+#define LBM_BR_MOMS_MINB(Q, S) ((Q) <= 19 ? 5 * 256 / LBM_BR_BLOCK : LBM_BR_MINB)
+
+template <class S>
+constexpr int kBrBlock = sizeof(S) == 8 ? 32 : LBM_BR_BLOCK;  // FP64: one warp, as kScBlock
+template <int Q, class S, bool BND, bool MOMS>
+constexpr int kBrMinb = sizeof(S) == 8 ? kScMinb<Q, S>
+                                       : BND ? LBM_BR_BND_MINB(Q, S) : MOMS ? LBM_BR_MOMS_MINB(Q, S) : LBM_BR_INT_MINB(Q, S);
 
 template <int Q, class S, bool FORCE, bool BND, bool MOMS>
-__global__ void __launch_bounds__(LBM_BR_BLOCK, BND ? LBM_BR_BND_MINB(Q, S) : (MOMS ? LBM_BR_MOMS_MINB(Q, S) : LBM_BR_INT_MINB(Q, S))) k_stream_collide_brick(const BrickArgs a) {
+__global__ void __launch_bounds__(kBrBlock<S>, kBrMinb<Q, S, BND, MOMS>) k_stream_collide_brick(const BrickArgs a) {
   using R = typename Sto<S>::R;
   using LT = Lat<Q>;
   constexpr int D = LT::D;
-  constexpr int BPB = LBM_BR_BLOCK / 64;
   constexpr int NW = Q / 2;  // (Q-1)/2 words of two 16-bit entries
-  const int l = threadIdx.x & 63, lane = threadIdx.x & 31;
+  const int64_t t = (int64_t)blockIdx.x * kBrBlock<S> + threadIdx.x;
+  const int l = (int)t & 63, lane = threadIdx.x & 31;
   // the brick index is uniform over each warp (64 threads per brick), so the
   // exit below and the shuffles run with whole warps
-  const int64_t b = (int64_t)blockIdx.x * BPB + (threadIdx.x >> 6);
+  const int64_t b = t >> 6;
   if (b >= a.nB) return;
   uint32_t tw[NW];
 #pragma unroll
@@ -647,10 +810,10 @@ __global__ void __launch_bounds__(LBM_BR_BLOCK, BND ? LBM_BR_BND_MINB(Q, S) : (M
 #pragma unroll
     for (int c = 0; c < D; ++c) F[c] = fp[c * N];
   }
-  bgk_collide<Q, R, FORCE>(g, R(a.omega), R(a.rho_off), F);
+  bgk_collide<Q, R, FORCE>(g, a.rx, R(a.rho_off), F);
 #pragma unroll
   for (int i = 0; i < Q; ++i) st_once(dst + i * N, Sto<S>::cv(g[i]));
-  if (MOMS) source_out<Q, S, FORCE>(a.so, first + l, g, R(a.omega), R(a.rho_off), F);
+  if (MOMS) source_out<Q, S, FORCE>(a.so, first + l, g, a.rx, R(a.rho_off), F);
 }
 
 // BF16 interior bricks, two neighbouring elements per thread: lane m of the
@@ -730,8 +893,8 @@ __global__ void __launch_bounds__(LBM_BR_PAIR_BLOCK, LBM_BR_PAIR_MINB(Q)) k_stre
       F1[c] = f.y;
     }
   }
-  bgk_collide<Q, R, FORCE>(g0, R(a.omega), R(a.rho_off), F0);
-  bgk_collide<Q, R, FORCE>(g1, R(a.omega), R(a.rho_off), F1);
+  bgk_collide<Q, R, FORCE>(g0, a.rx, R(a.rho_off), F0);
+  bgk_collide<Q, R, FORCE>(g1, a.rx, R(a.rho_off), F1);
 #pragma unroll
   for (int i = 0; i < Q; ++i) {
     const __nv_bfloat162 p = __floats2bfloat162_rn(g0[i], g1[i]);
@@ -821,19 +984,15 @@ __global__ void k_outlet(const OutletArgs a) {
 // stream-collide writes the records of the sources it updates (source_out);
 // this kernel takes the GhostFromFiner sources after their fill and every
 // source when the records have to be rebuilt from a new state.
-// Launch bounds of the ghost kernels: LBM_*_MINB sets a minimum of resident
-// blocks per SM; unset (0), only the block size is given, which lets the
+// The ghost kernels' launch bounds give the block size only, which lets the
 // compiler use fewer registers than an explicit minimum of one block.
 #ifndef LBM_MOM_BLOCK
 #define LBM_MOM_BLOCK 128
 #endif
-#if defined(LBM_MOM_MINB) && LBM_MOM_MINB > 0
-#define LBM_MOM_BOUNDS __launch_bounds__(LBM_MOM_BLOCK, LBM_MOM_MINB)
-#else
-#define LBM_MOM_BOUNDS __launch_bounds__(LBM_MOM_BLOCK)
-#endif
+template <class S>
+constexpr int kMomBlock = sizeof(S) == 8 ? 32 : LBM_MOM_BLOCK;  // FP64: one warp, as kScBlock
 template <int Q, class S, bool FORCE>
-__global__ void LBM_MOM_BOUNDS k_source_moments(const MomentsArgs a) {
+__global__ void __launch_bounds__(kMomBlock<S>) k_source_moments(const MomentsArgs a) {
   using R = typename Sto<S>::R;
   using RL = RecLayout<Q>;
   constexpr int D = Lat<Q>::D;
@@ -851,7 +1010,7 @@ __global__ void LBM_MOM_BOUNDS k_source_moments(const MomentsArgs a) {
 #pragma unroll
     for (int b = 0; b < D; ++b) F[b] = static_cast<const R*>(a.force)[(size_t)b * N + e];
   R rec[RL::STRIDE];
-  source_record<Q, R, FORCE>(g, R(a.omega), R(a.rho_off), F, rec);
+  source_record<Q, R, FORCE>(g, a.rx, R(a.rho_off), F, rec);
   if (a.prev) mean_record<Q, R>(static_cast<const R*>(a.prev) + (size_t)r * RL::STRIDE, rec);
   store_record<Q, R>(static_cast<R*>(a.mom) + (size_t)r * RL::STRIDE, rec);
 }
@@ -955,12 +1114,19 @@ __device__ __forceinline__ void gfc_ghost(const GfcArgs& a, const typename Sto<S
       if (f < RL::END) ld4(rec[s] + f, h + (f - RL::RP));
     rps[s] = h[0];
 #pragma unroll
-    for (int b = 0; b < D; ++b) ul[s][b] = sg[b] * h[RL::U - RL::RP + b];
+    for (int b = 0; b < D; ++b) {
+      const R v = h[RL::U - RL::RP + b];
+      if constexpr (sizeof(R) == 8) ul[s][b] = flip(v, !((oct >> b) & 1));
+      else ul[s][b] = sg[b] * v;
+    }
 #pragma unroll
     for (int b = 0; b < D; ++b)
 #pragma unroll
-      for (int c = b; c < D; ++c)
-        Sl[s][sidx<D>(b, c)] = sg[b] * sg[c] * h[RL::SS - RL::RP + sidx<D>(b, c)];
+      for (int c = b; c < D; ++c) {
+        const R v = h[RL::SS - RL::RP + sidx<D>(b, c)];
+        if constexpr (sizeof(R) == 8) Sl[s][sidx<D>(b, c)] = b == c ? v : flip(v, ((oct >> b) ^ (oct >> c)) & 1);
+        else Sl[s][sidx<D>(b, c)] = sg[b] * sg[c] * v;
+      }
   }
   R uloc[3];
   compact_uloc<Q, R>(ul, Sl, uloc);
@@ -979,7 +1145,7 @@ __device__ __forceinline__ void gfc_ghost(const GfcArgs& a, const typename Sto<S
   const R rp = R(a.r_scale) * (lw0 * rps[0] + lw1 * rps[1] + lw2 * rps[2] + lw3 * rps[3]) + R(a.r_shift);
   const R rho = R(a.rho_off) + rp;
   const R wf = R(a.omega_f);
-  const R scale = (R(1) - wf) * R(a.omega_c) / (R(a.tratio) * wf);
+  const R scale = sizeof(R) == 8 ? R(a.scale) : (R(1) - wf) * R(a.omega_c) / (R(a.tratio) * wf);
   S* __restrict__ dst = static_cast<S*>(a.dst);
   const size_t N = (size_t)a.Ntot;
   const int64_t e = a.dest0 + k;
@@ -1010,8 +1176,16 @@ __device__ __forceinline__ void gfc_ghost(const GfcArgs& a, const typename Sto<S
       if (LT::c(i, b) < 0) cu -= u[b];
     }
     const R w = R(LT::w(i));
-    const R even = w * (base + R(4.5) * rho * cu * cu);
-    const R odd = w * R(3) * rho * cu;
+    R even, odd;
+    if constexpr (sizeof(R) == 8) {
+      // w base and w rho are shared by all directions of a weight
+      const double wr = w * rho, t = wr * cu;
+      odd = 3.0 * t;
+      even = fma(4.5 * t, cu, w * base);
+    } else {
+      even = w * (base + R(4.5) * rho * cu * cu);
+      odd = w * R(3) * rho * cu;
+    }
     R fa = fn[i], fb = fn[i + 1];
     if (odd_rescale) {
       const R fe = R(0.5) * (fa + fb), fo = R(0.5) * (fa - fb) * ro;
@@ -1027,20 +1201,17 @@ __device__ __forceinline__ void gfc_ghost(const GfcArgs& a, const typename Sto<S
 #ifndef LBM_GFC_BLOCK
 #define LBM_GFC_BLOCK 64
 #endif
-#if defined(LBM_GFC_MINB) && LBM_GFC_MINB > 0
-#define LBM_GFC_BOUNDS __launch_bounds__(LBM_GFC_BLOCK, LBM_GFC_MINB)
-#else
-#define LBM_GFC_BOUNDS __launch_bounds__(LBM_GFC_BLOCK)
-#endif
+template <class S>
+constexpr int kGfcBlock = sizeof(S) == 8 ? 32 : LBM_GFC_BLOCK;  // FP64: one warp, as kScBlock
 template <int Q, class S, bool TWO>
-__global__ void LBM_GFC_BOUNDS k_fill_gfc(const GfcArgs a) {
+__global__ void __launch_bounds__(kGfcBlock<S>) k_fill_gfc(const GfcArgs a) {
   using R = typename Sto<S>::R;
   using LT = Lat<Q>;
   using RL = RecLayout<Q>;
   using GG = GfcGroup<LT::D>;
   constexpr int G = GG::G, NSLOT = GG::NSLOT;
   constexpr int PSTR = RL::STRIDE + 4;  // padded record: sibling lanes' reads fall in distinct banks
-  constexpr int NGRP = LBM_GFC_BLOCK / G;
+  constexpr int NGRP = kGfcBlock<S> / G;
   __shared__ __align__(16) R stage[NGRP * NSLOT * PSTR];
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int oct = threadIdx.x & (G - 1);  // octant of the ghost
@@ -1091,13 +1262,13 @@ __global__ void LBM_GFC_BOUNDS k_fill_gfc(const GfcArgs a) {
 // One group of 2^d consecutive lanes per ghost: lane b loads child b (siblings
 // are contiguous, so the group's loads are coalesced), and the sums over the
 // children are shuffles inside the group.
-#if defined(LBM_GFF_MINB) && LBM_GFF_MINB > 0
-#define LBM_GFF_BOUNDS __launch_bounds__(256, LBM_GFF_MINB)
-#else
-#define LBM_GFF_BOUNDS __launch_bounds__(256)
+#ifndef LBM_GFF_BLOCK
+#define LBM_GFF_BLOCK 256
 #endif
+template <class S>
+constexpr int kGffBlock = sizeof(S) == 8 ? 32 : LBM_GFF_BLOCK;  // FP64: one warp, as kScBlock
 template <int Q, class S, bool FORCE>
-__global__ void LBM_GFF_BOUNDS k_fill_gff(const GffArgs a) {
+__global__ void __launch_bounds__(kGffBlock<S>) k_fill_gff(const GffArgs a) {
   using R = typename Sto<S>::R;
   using LT = Lat<Q>;
   constexpr int D = LT::D, NS = LT::NS, NCH = 1 << D;
@@ -1107,7 +1278,7 @@ __global__ void LBM_GFF_BOUNDS k_fill_gff(const GffArgs a) {
   const bool active = k < a.ng;
   const S* __restrict__ src = static_cast<const S*>(a.src_fine);
   const size_t N = (size_t)a.Ntot;
-  const R wf = R(a.omega_f), rho_off = R(a.rho_off);
+  const R wf = R(a.rx_f.omega), rho_off = R(a.rho_off);
   R rp = R(0), u[3] = {R(0), R(0), R(0)}, fneq[Q], Sv[NS];
 #pragma unroll
   for (int q = 0; q < Q; ++q) fneq[q] = R(0);
@@ -1122,7 +1293,8 @@ __global__ void LBM_GFF_BOUNDS k_fill_gff(const GffArgs a) {
     if (FORCE)
 #pragma unroll
       for (int c = 0; c < D; ++c) F[c] = static_cast<const R*>(a.force)[(size_t)c * N + e];
-    post_moments<Q, R, true, FORCE>(g, wf, rho_off, F, rp, u, fneq, Sv);
+    if constexpr (sizeof(R) == 8) post_moments64<Q, FORCE>(g, a.rx_f, rho_off, F, rp, u, fneq, Sv);
+    else post_moments<Q, R, true, FORCE>(g, wf, rho_off, F, rp, u, fneq, Sv);
     if (a.odd_ratio != 1.0) {
       // diffusive scaling: f^neq's odd part takes an extra factor (the sum
       // over the children is linear, so each child's share is rescaled)
@@ -1147,16 +1319,30 @@ __global__ void LBM_GFF_BOUNDS k_fill_gff(const GffArgs a) {
   const R inv_u = inv * R(a.u_scale);
   const R dfac = R(a.tratio) * R(D == 3 ? 0.5 : 1.0);
   R rpm = rp * inv, uP[3] = {R(0), R(0), R(0)};
+  if constexpr (sizeof(R) == 8) {
+    double tr = 0;
 #pragma unroll
-  for (int aa = 0; aa < D; ++aa) {
-    const R sa = ((b >> aa) & 1) ? R(1) : R(-1);
-    R lap = R(0);
+    for (int c = 0; c < D; ++c) tr += Sv[c];
 #pragma unroll
-    for (int c = 0; c < D; ++c) {
-      const R sc = ((b >> c) & 1) ? R(1) : R(-1);
-      lap += dfac * (R(2) * sc * Sv[sidx<D>(aa, c)] - sa * Sv[sidx<D>(c, c)]);
+    for (int aa = 0; aa < D; ++aa) {
+      double s2 = 0;
+#pragma unroll
+      for (int c = 0; c < D; ++c) s2 += flip(Sv[sidx<D>(aa, c)], !((b >> c) & 1));
+      const double lap = fma(2.0, s2, flip(tr, (b >> aa) & 1));
+      uP[aa] = fma(-dfac / 32.0, lap, u[aa] * inv_u);
     }
-    uP[aa] = u[aa] * inv_u - lap * R(1.0 / 32.0);
+  } else {
+#pragma unroll
+    for (int aa = 0; aa < D; ++aa) {
+      const R sa = ((b >> aa) & 1) ? R(1) : R(-1);
+      R lap = R(0);
+#pragma unroll
+      for (int c = 0; c < D; ++c) {
+        const R sc = ((b >> c) & 1) ? R(1) : R(-1);
+        lap += dfac * (R(2) * sc * Sv[sidx<D>(aa, c)] - sa * Sv[sidx<D>(c, c)]);
+      }
+      uP[aa] = u[aa] * inv_u - lap * R(1.0 / 32.0);
+    }
   }
 #pragma unroll
   for (int o = 1; o < NCH; o <<= 1) {
@@ -1192,7 +1378,7 @@ __global__ void LBM_GFF_BOUNDS k_fill_gff(const GffArgs a) {
   const R wc = R(a.omega_c);
   rpm = R(a.r_scale) * rpm + R(a.r_shift);  // to coarse units (unchanged in acoustic scaling)
   const R rho = rho_off + rpm;
-  const R scale = (R(1) - wc) * R(a.tratio) * wf / wc * inv;
+  const R scale = sizeof(R) == 8 ? R(a.scale) : (R(1) - wc) * R(a.tratio) * wf / wc * inv;
   S* __restrict__ dst = static_cast<S*>(a.dst);
   const int64_t e = k < a.n_inner ? a.dest0 + k : a.dest_outer + (k - a.n_inner);
   // the group's lanes share the Q stores: lane b the directions j 2^d + b,
@@ -1492,7 +1678,7 @@ template <class S>
 struct Launch {
   static void stream_collide_brick(int Q, bool force, bool boundary, const BrickArgs& a, cudaStream_t st) {
     if (a.nB <= 0) return;
-    const unsigned g = blocks_for(a.nB, LBM_BR_BLOCK / 64);
+    const unsigned g = blocks_for(64 * a.nB, kBrBlock<S>);
     with_q(Q, [&](auto q) {
       constexpr int QQ = decltype(q)::value;
       const bool moms = a.so.mask != nullptr;
@@ -1509,7 +1695,7 @@ struct Launch {
       }
       auto go = [&](auto F, auto B, auto M) {
         k_stream_collide_brick<QQ, S, decltype(F)::value, decltype(B)::value, decltype(M)::value>
-            <<<g, LBM_BR_BLOCK, 0, st>>>(a);
+            <<<g, kBrBlock<S>, 0, st>>>(a);
       };
       using T = std::true_type;
       using U = std::false_type;
@@ -1525,50 +1711,49 @@ struct Launch {
   static void stream_collide(int Q, bool force, const StreamCollideArgs& a, cudaStream_t st) {
     const int64_t n = a.end - a.begin;
     if (n <= 0) return;
-    constexpr int EPT = LBM_SC_EPT;
-    const unsigned g = blocks_for(n, LBM_SC_BLOCK * EPT);
+    const unsigned g = blocks_for(n, kScBlock<S>);
     with_q(Q, [&](auto q) {
       constexpr int QQ = decltype(q)::value;
       const bool moms = a.so.mask != nullptr;
       if (force) {
-        if (moms) k_stream_collide<QQ, S, true, EPT, true><<<g, LBM_SC_BLOCK, 0, st>>>(a);
-        else k_stream_collide<QQ, S, true, EPT, false><<<g, LBM_SC_BLOCK, 0, st>>>(a);
+        if (moms) k_stream_collide<QQ, S, true, true><<<g, kScBlock<S>, 0, st>>>(a);
+        else k_stream_collide<QQ, S, true, false><<<g, kScBlock<S>, 0, st>>>(a);
       } else {
-        if (moms) k_stream_collide<QQ, S, false, EPT, true><<<g, LBM_SC_BLOCK, 0, st>>>(a);
-        else k_stream_collide<QQ, S, false, EPT, false><<<g, LBM_SC_BLOCK, 0, st>>>(a);
+        if (moms) k_stream_collide<QQ, S, false, true><<<g, kScBlock<S>, 0, st>>>(a);
+        else k_stream_collide<QQ, S, false, false><<<g, kScBlock<S>, 0, st>>>(a);
       }
     });
   }
   static void outlet(int Q, const OutletArgs& a, cudaStream_t st) {
     const int64_t n = a.end - a.begin;
     if (n <= 0) return;
-    with_q(Q, [&](auto q) { k_outlet<decltype(q)::value, S><<<blocks_for(n, 128), 128, 0, st>>>(a); });
+    with_q(Q, [&](auto q) { k_outlet<decltype(q)::value, S><<<blocks_for(n, kMomBlock<S>), kMomBlock<S>, 0, st>>>(a); });
   }
   static void source_moments(int Q, const MomentsArgs& a, cudaStream_t st) {
     if (a.nsrc <= 0) return;
     with_q(Q, [&](auto q) {
       constexpr int QQ = decltype(q)::value;
-      const unsigned g = blocks_for(a.nsrc, LBM_MOM_BLOCK);
-      if (a.force) k_source_moments<QQ, S, true><<<g, LBM_MOM_BLOCK, 0, st>>>(a);
-      else k_source_moments<QQ, S, false><<<g, LBM_MOM_BLOCK, 0, st>>>(a);
+      const unsigned g = blocks_for(a.nsrc, kMomBlock<S>);
+      if (a.force) k_source_moments<QQ, S, true><<<g, kMomBlock<S>, 0, st>>>(a);
+      else k_source_moments<QQ, S, false><<<g, kMomBlock<S>, 0, st>>>(a);
     });
   }
   static void fill_gfc(int Q, const GfcArgs& a, cudaStream_t st) {
     if (a.ng <= 0) return;
     with_q(Q, [&](auto q) {
       constexpr int QQ = decltype(q)::value;
-      const unsigned g = blocks_for(a.ng, LBM_GFC_BLOCK);
-      if (a.mom2) k_fill_gfc<QQ, S, true><<<g, LBM_GFC_BLOCK, 0, st>>>(a);
-      else k_fill_gfc<QQ, S, false><<<g, LBM_GFC_BLOCK, 0, st>>>(a);
+      const unsigned g = blocks_for(a.ng, kGfcBlock<S>);
+      if (a.mom2) k_fill_gfc<QQ, S, true><<<g, kGfcBlock<S>, 0, st>>>(a);
+      else k_fill_gfc<QQ, S, false><<<g, kGfcBlock<S>, 0, st>>>(a);
     });
   }
   static void fill_gff(int Q, const GffArgs& a, cudaStream_t st) {
     if (a.ng <= 0) return;
     with_q(Q, [&](auto q) {
       constexpr int QQ = decltype(q)::value;
-      const unsigned g = blocks_for(a.ng * (1 << Lat<QQ>::D), 256);
-      if (a.force) k_fill_gff<QQ, S, true><<<g, 256, 0, st>>>(a);
-      else k_fill_gff<QQ, S, false><<<g, 256, 0, st>>>(a);
+      const unsigned g = blocks_for(a.ng * (1 << Lat<QQ>::D), kGffBlock<S>);
+      if (a.force) k_fill_gff<QQ, S, true><<<g, kGffBlock<S>, 0, st>>>(a);
+      else k_fill_gff<QQ, S, false><<<g, kGffBlock<S>, 0, st>>>(a);
     });
   }
   static void fill_rest(int Q, const FillArgs& a, cudaStream_t st) {

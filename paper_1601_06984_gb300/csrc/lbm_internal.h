@@ -76,6 +76,42 @@ inline double odd_fneq_ratio(int mode, bool to_coarse) {
 // the same flow's lattice velocity on level index li over that on the coarsest level
 inline double level_velocity_ratio(int li, int mode) { return mode == LBM_TIME_DIFFUSIVE ? std::ldexp(1.0, -li) : 1.0; }
 
+// Relaxation constants of a level for the FP64 kernels, whose pipe is GB300's
+// narrowest unit (1.7 multiply-adds per clock and SM): every factor that is
+// the same for all elements is formed here once, and the kernels read it as a
+// constant operand.  Arrays are indexed by |c_i|^2.
+struct Relax {
+  double omega;
+  double keep;                     // 1 - omega
+  double eq[4], quad[4], lin[4];   // omega w {1, 9/2, 3}
+  double force[4];                 // 3 w (1 - omega / 2)
+  double r1w;                      // 1 / (1 - omega)
+  double neq[4], nquad[4], nlin[4], nforce[4];  // w {1, 9/2, 3}, 3 w (1 - omega / 2), each times r1w
+  double strain;                   // -3 omega / 2
+};
+inline Relax make_relax(int Q, double omega) {
+  int c[kQmax][3];
+  double w[kQmax];
+  host_lattice(Q, c, w);
+  Relax r{};
+  r.omega = omega;
+  r.keep = 1.0 - omega;
+  r.r1w = 1.0 / (1.0 - omega);
+  r.strain = -1.5 * omega;
+  for (int i = 0; i < Q; ++i) {
+    const int n = c[i][0] * c[i][0] + c[i][1] * c[i][1] + c[i][2] * c[i][2];
+    r.eq[n] = omega * w[i];
+    r.quad[n] = 4.5 * r.eq[n];
+    r.lin[n] = 3.0 * r.eq[n];
+    r.force[n] = 3.0 * w[i] * (1.0 - 0.5 * omega);
+    r.neq[n] = w[i] * r.r1w;
+    r.nquad[n] = 4.5 * r.neq[n];
+    r.nlin[n] = 3.0 * r.neq[n];
+    r.nforce[n] = r.force[n] * r.r1w;
+  }
+  return r;
+}
+
 struct HostLevel {
   int L = 0;
   double omega = 1.0;
@@ -175,7 +211,8 @@ struct StreamCollideArgs {
   const double* inlet_s;  // inlet profile factor per inlet link
   int64_t Ntot, begin, end;  // linear range; element = lin + (lin >= hole_at ? hole_len : 0)
   int64_t hole_at, hole_len;  // interior bricks skipped by this kernel (0 length: none)
-  double omega, rho_off;
+  Relax rx;
+  double rho_off;
   double inlet[kQmax];  // 6 w_i rho0 (c_i . u_in)
   SourceOut so;
 };
@@ -190,7 +227,8 @@ struct BrickArgs {
   const int32_t* nb;    // [nB][27] rows (offsets from the brick's first element, or kBrickMissing)
   const uint16_t* tab;  // [Q-1][64]
   int64_t Ntot, begin, nB;
-  double omega, rho_off;
+  Relax rx;
+  double rho_off;
   // boundary bricks: links through a missing neighbour brick use the element's
   // neighbour-list code (pull, bounce-back, inlet, boundary value)
   const uint32_t* nbr;
@@ -224,7 +262,8 @@ struct MomentsArgs {
   const void* prev;  // if set: mom = (prev + moments now) / 2 (mean of two time levels)
   const int32_t* rec;  // record index of elem[k] (null: k)
   int64_t Ntot, nsrc;
-  double omega, rho_off;
+  Relax rx;
+  double rho_off;
 };
 
 struct GfcArgs {
@@ -237,6 +276,7 @@ struct GfcArgs {
   void* dst;
   int64_t Ntot;
   double omega_c, omega_f, rho_off;
+  double scale;          // (1 - omega_f) omega_c / (tratio omega_f) (FP64 kernels)
   int skip_outer;        // leave the outer-layer ghosts (oct & kGfcOuter) unwritten
   // unit conversion coarse -> fine: dt_c / dt_f, u_f = u_scale u_c and the
   // density deviation rho'_f = r_scale rho'_c + r_shift (relative to rho_off);
@@ -252,7 +292,9 @@ struct GffArgs {
   int64_t dest0, dest_outer;
   void* dst;             // pdfs holding the coarse ghosts
   int64_t Ntot;
-  double omega_c, omega_f, rho_off;
+  Relax rx_f;            // of the children's level
+  double omega_c, rho_off;
+  double scale;          // factor of the children's f^neq sum in the stored ghost (FP64 kernels)
   // unit conversion fine -> coarse: dt_c / dt_f, u_c = u_scale u_f and the
   // density deviation rho'_c = r_scale rho'_f + r_shift (relative to rho_off);
   // odd_ratio: the extra factor of f^neq's odd part (odd_fneq_ratio)
