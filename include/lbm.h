@@ -219,11 +219,10 @@ lbm_status lbm_set_force(lbm_ctx* ctx, const double* F);
  * graph captured on first use, a remaining single step a one-step graph (one
  * of each per A/B parity state; dropped by lbm_set_params and lbm_bind), on
  * the bound stream; in timing mode 1 every step is launched kernel by kernel
- * (the adjoint's recomputed steps too).  Both paths
- * issue the same kernels; in the graphs the three stream-collide kernels of a
- * level (interior bricks, boundary bricks, neighbour list: disjoint elements,
- * the same source state) run as parallel branches, joined before the next op,
- * which leaves every result bitwise the same.  With params.check_every = M
+ * (the adjoint's recomputed steps too).  Both paths do the same ops with the
+ * same kernels; in the graphs one launch takes all levels that advance at the
+ * same instant, and the interior bricks run beside the other elements, which
+ * leaves every result bitwise the same.  With params.check_every = M
  * the mass is checked after every M-th coarse step (see lbm_params); a failed
  * check returns LBM_ERR_NUMERIC right after that step, with the state left as
  * it was then (the context stays usable, e.g. for lbm_set_state). */
@@ -365,7 +364,10 @@ lbm_status lbm_adjoint(lbm_ctx* ctx, int64_t n_coarse, int32_t K, int32_t object
                        uint64_t bytes, double* J, double* dJ_dF, double* dJ_domega, double* dJ_duin,
                        double* dJ_df0);
 
-/* Launches of library kernels enqueued by this context since it was bound. */
+/* Level kernels enqueued by this context since it was bound: every kernel of
+ * every level (fills, source records, boundary values, stream-collide per kind
+ * of element) counts once, whether it has a launch of its own, as in timing
+ * mode 1, or shares one with other levels, as in the captured steps. */
 lbm_status lbm_kernel_launches(const lbm_ctx* ctx, int64_t* count);
 
 /* Device timing of the step's kernels with CUDA events on the bound stream.
@@ -374,11 +376,14 @@ lbm_status lbm_kernel_launches(const lbm_ctx* ctx, int64_t* count);
  *          launched kernel by kernel, not replayed from graphs.
  *  mode 2: lbm_step keeps replaying its captured graphs, which then
  *          also record events around the finest level's stream-collide
- *          launches (kinds 0-2) and around their whole group (kind 7: in the
- *          graphs a level's three stream-collide kernels run as parallel
- *          branches, so their span is the level's stream-collide time);
+ *          launches (kinds 0, 2) and around their whole group (kind 7: they
+ *          run as parallel branches, so their span is the level's
+ *          stream-collide time);
  *          lbm_timing_read returns those of the most recent replay (its two
- *          coarse steps), if not read before.
+ *          coarse steps), if not read before.  Recorded at the instants when
+ *          only the finest level advances (the others share their launches
+ *          with it); kind 2 is then the launch of the boundary bricks and the
+ *          neighbour-list elements.
  * Changing between mode 2 and the others drops the captured graphs.
  * lbm_timing_read synchronises the stream and returns, in row 8 L + k for level
  * index L (coarsest 0) and kernel kind k, the number of timed launches and
@@ -386,7 +391,8 @@ lbm_status lbm_kernel_launches(const lbm_ctx* ctx, int64_t* count);
  * record.  Enabling clears it too.  Kinds: 0 stream-collide of the interior
  * bricks, 1 stream-collide through the neighbour list, 2 stream-collide of the
  * boundary bricks, 3 GhostFromFiner (L: the coarse level holding the ghosts),
- * 4 source moments (L: the coarse level), 5 GhostFromCoarser (L: the fine
+ * 4 source moments where a kernel of their own forms them (L: the coarse
+ * level), 5 GhostFromCoarser (L: the fine
  * level holding the ghosts), 6 outlet values, 7 the span of a level's
  * stream-collide kernels (mode 2 only).  Other modes: LBM_ERR_ARG. */
 lbm_status lbm_timing_enable(lbm_ctx* ctx, int32_t mode);

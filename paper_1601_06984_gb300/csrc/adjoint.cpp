@@ -475,7 +475,9 @@ lbm_status lbm_adjoint(lbm_ctx* c, int64_t n, int32_t K, int32_t objective, void
       m.Ntot = (int64_t)N;
       m.nsrc = c->ld[lc].nsrc;
       m.rx = make_relax(c->Q, Hc.omega);
+      m.rx32 = make_relax32(Hc.omega);
       m.rho_off = c->rho_off;
+      m.rho_off32 = (float)c->rho_off;
       m.src = snap(sa);
       m.mom = W + L.recA[lc];
       m.prev = nullptr;
@@ -495,23 +497,8 @@ lbm_status lbm_adjoint(lbm_ctx* c, int64_t n, int32_t K, int32_t objective, void
         const int p = t.parity[li];
         const bool outlet = H.out_end > H.out_begin;
         if (outlet) {
-          OutletArgs o{};
-          o.src = snap(t.snap);
-          o.side = W + L.side_fwd;
-          o.elem = c->at<int32_t>(c->oOutElem);
-          o.a = c->at<int32_t>(c->oOutA);
-          o.b = c->at<int32_t>(c->oOutB);
-          o.dir = c->at<int8_t>(c->oOutDir);
-          o.kind = c->at<int8_t>(c->oOutKind);
-          o.force = force;
-          o.Ntot = (int64_t)N;
-          o.begin = H.out_begin;
-          o.end = H.out_end;
-          o.omega = H.omega;
-          o.rho_off = c->rho_off;
-          o.rho0 = c->p.rho0;
-          o.zero_gradient = c->p.outlet == LBM_OUTLET_ZERO_GRADIENT;
-          o.q = c->at<double>(c->oOutQ);
+          OutletArgs o = c->outlet_args(W + L.side_fwd);
+          c->add_outlet(o, li, snap(t.snap));
           c->ops->outlet(c->Q, o, st);
         }
         AdjSCArgs a{};

@@ -837,7 +837,7 @@ __global__ void __launch_bounds__(256, LBM_ADJ_MINB(S, LBM_ADJ_GFF_MINB, 1)) k_a
 #pragma unroll
       for (int q = 0; q < Q; ++q) g[q] = Sto<S>::ld(x + (size_t)q * N + ec);
       load_force<S, R>(a.c.force, a.c.Ntot, ec, F, D);
-      post_moments<Q, R, true>(g, wf, rho_off, F, rp, u, fneq, Sv);
+      post_moments<Q, R, true>(g, wf, R(1) / (R(1) - wf), rho_off, F, rp, u, fneq, Sv);
     }
     R dS[3][NS];
 #pragma unroll

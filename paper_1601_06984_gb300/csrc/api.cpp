@@ -82,41 +82,74 @@ void lbm_ctx::layout() {
   oPartial = take((size_t)nlev * kReduceBlocks * 8 * 8);
   oRed = take(8 * 8);
   bytes = o;
+  n_filled = 1;
+  for (int li = 0; li < nlev; ++li)
+    if (m.lv[li].nF > 0) n_filled = li + 1;
+  outlet_reads_ghosts = false;
+  for (const auto* v : {&m.out_elem, &m.out_a, &m.out_b})
+    for (int32_t e : *v)
+      if (e >= 0 && m.kind[e] != K_FLUID) outlet_reads_ghosts = true;
 }
 
 // ---------------------------------------------------------------- driver
-void lbm_ctx::fill_gff(int li) {
+// unit conversion into the ghosts' level: fine -> coarse u_c = (dt_c / dt_f) / 2
+// u_f, the density deviation with the square of that factor (1 in acoustic
+// scaling); coarse -> fine the inverse
+template <class Args>
+void lbm_ctx::ghost_units(Args& a, bool to_coarse) const {
+  const double m = time_ratio(p.time_mode), us = to_coarse ? m / 2.0 : 2.0 / m;
+  const double odd = odd_fneq_ratio(p.time_mode, to_coarse), rs = us * us, shift = (1.0 - rs) * (p.rho0 - rho_off);
+  a.u64 = {rho_off, m, us, rs, shift, odd};
+  a.u32 = {(float)rho_off, (float)m, (float)us, (float)rs, (float)shift, (float)odd};
+  a.odd_rescale = odd != 1.0;
+  a.Ntot = M.Ntot;
+}
+
+GffArgs lbm_ctx::gff_args() const {
+  GffArgs a{};
+  ghost_units(a, true);
+  a.force = force_ptr();
+  a.sources = source_table();
+  return a;
+}
+
+void lbm_ctx::add_gff(GffArgs& a, int li) const {
   const HostLevel& H = M.lv[li];
   const HostLevel& Hf = M.lv[li + 1];
   if (H.nG1 + H.nG2 == 0) return;
-  GffArgs a{};
-  a.src_fine = cur(li + 1);
-  a.force = force_ptr();
-  a.child0 = at<int32_t>(ld[li].gff_child0);
-  a.ng = H.nG1 + H.nG2;
-  a.n_inner = H.nG1;
-  a.dest0 = H.base + H.oG1;
-  a.dest_outer = H.base + H.oG2;
-  a.dst = cur(li);
-  a.Ntot = M.Ntot;
-  a.omega_c = H.omega;
-  a.rx_f = make_relax(Q, Hf.omega);
-  a.rho_off = rho_off;
-  // fine -> coarse lattice units: u_c = (dt_c / dt_f) / 2 u_f, the density
-  // deviation with the square of that factor (1 in acoustic scaling)
-  a.tratio = time_ratio(p.time_mode);
-  a.u_scale = a.tratio / 2.0;
-  a.r_scale = a.u_scale * a.u_scale;
-  a.r_shift = (1.0 - a.r_scale) * (p.rho0 - rho_off);
-  a.odd_ratio = odd_fneq_ratio(p.time_mode, true);
-  a.scale = (1.0 - H.omega) * a.tratio * Hf.omega / H.omega / (1 << d);
+  const int k = a.nseg++;
+  GffLevel& L = a.lev[k];
+  L.src_fine = cur(li + 1);
+  L.child0 = at<int32_t>(ld[li].gff_child0);
+  L.ng = (int32_t)(H.nG1 + H.nG2);
+  L.n_inner = (int32_t)H.nG1;
+  L.dest0 = (int32_t)(H.base + H.oG1);
+  L.dest_outer = (int32_t)(H.base + H.oG2);
+  L.dst = cur(li);
+  L.rec_out = ld[li].n_gsrc > 0 ? at(ld[li].momA[parity[li]]) : nullptr;
+  L.rx_f = make_relax32(Hf.omega);
+  a.rx_c[k] = make_relax32(H.omega);
+  a.rx_c64[k] = make_relax(Q, H.omega);
+  a.rx_f64[k] = make_relax(Q, Hf.omega);
+  const double m = time_ratio(p.time_mode);
+  a.scale[k] = (1.0 - H.omega) * m * Hf.omega / H.omega / (1 << d);
+  const float wc = (float)H.omega, wf = (float)Hf.omega;  // the FP32 kernels' factor, in their arithmetic
+  L.scale32 = (1.0f - wc) * (float)m * wf / wc * (1.0f / (float)(1 << d));
+}
+
+void lbm_ctx::fill_gff(int li) {
+  GffArgs a = gff_args();
+  add_gff(a, li);
+  if (!a.nseg) return;
   timed_launch(li, TK_GFF, [&] { ops->fill_gff(Q, a, st); });
   ++launches;
 }
 
-void lbm_ctx::source_moments(int li, size_t mom_off, size_t prev_off, cudaStream_t s, int subset) {
+SourceTable lbm_ctx::source_table() const { return {at<uint32_t>(oSrcMask), at<int32_t>(oSrcFirst)}; }
+
+void lbm_ctx::source_moments(int li, size_t mom_off, cudaStream_t s, int subset) {
   const LevelDev& L = ld[li];
-  const int64_t n = subset == SRC_ALL ? L.nsrc : subset == SRC_GFF ? L.n_gsrc : L.n_gsrc - L.n_gsrc_inner;
+  const int64_t n = subset == SRC_ALL ? L.nsrc : L.n_gsrc - L.n_gsrc_inner;
   if (n == 0) return;
   if (!s) s = st;
   MomentsArgs a{};
@@ -125,167 +158,261 @@ void lbm_ctx::source_moments(int li, size_t mom_off, size_t prev_off, cudaStream
   if (subset == SRC_ALL) {
     a.elem = at<int32_t>(L.src_elem);
   } else {
-    const int64_t skip = subset == SRC_GFF ? 0 : L.n_gsrc_inner;
-    a.elem = at<int32_t>(L.gsrc_elem) + skip;
-    a.rec = at<int32_t>(L.gsrc_rec) + skip;
+    a.elem = at<int32_t>(L.gsrc_elem) + L.n_gsrc_inner;
+    a.rec = at<int32_t>(L.gsrc_rec) + L.n_gsrc_inner;
   }
   a.mom = at(mom_off);
-  a.prev = prev_off ? at(prev_off) : nullptr;
   a.Ntot = M.Ntot;
   a.nsrc = n;
   a.rx = make_relax(Q, M.lv[li].omega);
+  a.rx32 = make_relax32(M.lv[li].omega);
   a.rho_off = rho_off;
+  a.rho_off32 = (float)rho_off;
   timed_launch(li, TK_MOM, [&] { ops->source_moments(Q, a, s); }, s);
   ++launches;
 }
 
-void lbm_ctx::fill_gfc(int lf, bool two_times, bool all_layers, cudaStream_t s, bool next_buffer) {
+GfcArgs lbm_ctx::gfc_args() const {
+  GfcArgs a{};
+  ghost_units(a, false);
+  return a;
+}
+
+void lbm_ctx::add_gfc(GfcArgs& a, int lf, bool two_times, bool all_layers) const {
   const HostLevel& H = M.lv[lf];
   if (H.nC == 0) return;
-  if (!s) s = st;
   const int lc = lf - 1;
-  GfcArgs a{};
+  GfcLevel& L = a.lev[a.nseg++];
   // at t + 1/2 (after the coarse stream-collide): the means of the records
   // at t and t + 1, which the two buffers hold
-  a.mom = at(ld[lc].momA[parity[lc] ^ (two_times ? 1 : 0)]);
-  a.mom2 = two_times ? at(ld[lc].momA[parity[lc]]) : nullptr;
-  a.nsrc = ld[lc].nsrc;
-  a.gsrc = at<int32_t>(ld[lf].gfc_src);
-  a.oct = at<uint8_t>(ld[lf].gfc_oct);
-  a.ng = H.nC;
-  a.dest0 = H.base + H.oC;
-  a.dst = next_buffer ? nxt(lf) : cur(lf);
-  a.Ntot = M.Ntot;
-  a.omega_c = M.lv[lc].omega;
-  a.omega_f = H.omega;
-  a.rho_off = rho_off;
-  a.skip_outer = !all_layers && p.time_mode == LBM_TIME_LINEAR;
-  // coarse -> fine lattice units, the inverse of the GhostFromFiner conversion
-  a.tratio = time_ratio(p.time_mode);
-  a.u_scale = 2.0 / a.tratio;
-  a.r_scale = a.u_scale * a.u_scale;
-  a.r_shift = (1.0 - a.r_scale) * (p.rho0 - rho_off);
-  a.odd_ratio = odd_fneq_ratio(p.time_mode, false);
-  a.scale = (1.0 - a.omega_f) * a.omega_c / (a.tratio * a.omega_f);
-  timed_launch(lf, TK_GFC, [&] { ops->fill_gfc(Q, a, s); }, s);
+  L.mom = at(ld[lc].momA[parity[lc] ^ (two_times ? 1 : 0)]);
+  L.mom2 = two_times ? at(ld[lc].momA[parity[lc]]) : nullptr;
+  L.gsrc = at<int32_t>(ld[lf].gfc_src);
+  L.oct = at<uint8_t>(ld[lf].gfc_oct);
+  L.ng = (int32_t)H.nC;
+  L.dest0 = (int32_t)(H.base + H.oC);
+  L.dst = cur(lf);
+  L.skip_outer = !all_layers && p.time_mode == LBM_TIME_LINEAR;
+  const double wc = M.lv[lc].omega, wf = H.omega, m = time_ratio(p.time_mode);
+  L.scale = (1.0 - wf) * wc / (m * wf);
+  const float wcf = (float)wc, wff = (float)wf;  // the FP32 kernels' factor, in their arithmetic
+  L.scale32 = (1.0f - wff) * wcf / ((float)m * wff);
+}
+
+void lbm_ctx::fill_gfc(int lf, bool two_times, bool all_layers) {
+  GfcArgs a = gfc_args();
+  add_gfc(a, lf, two_times, all_layers);
+  if (!a.nseg) return;
+  timed_launch(lf, TK_GFC, [&] { ops->fill_gfc(Q, a, st); });
   ++launches;
 }
 
-void lbm_ctx::stream_collide(int li, cudaStream_t s0) {
-  if (!s0) s0 = st;
+OutletArgs lbm_ctx::outlet_args(const void* side) const {
+  OutletArgs o{};
+  o.side = const_cast<void*>(side);
+  o.elem = at<int32_t>(oOutElem);
+  o.a = at<int32_t>(oOutA);
+  o.b = at<int32_t>(oOutB);
+  o.dir = at<int8_t>(oOutDir);
+  o.kind = at<int8_t>(oOutKind);
+  o.force = force_ptr();
+  o.Ntot = M.Ntot;
+  o.rho_off = rho_off;
+  o.rho0 = p.rho0;
+  o.zero_gradient = p.outlet == LBM_OUTLET_ZERO_GRADIENT;
+  o.q = at<double>(oOutQ);
+  return o;
+}
+
+void lbm_ctx::add_outlet(OutletArgs& o, int li, const void* src) const {
   const HostLevel& H = M.lv[li];
-  if (H.out_end > H.out_begin) {
-    OutletArgs o{};
-    o.src = cur(li);
-    o.side = at(oSide);
-    o.elem = at<int32_t>(oOutElem);
-    o.a = at<int32_t>(oOutA);
-    o.b = at<int32_t>(oOutB);
-    o.dir = at<int8_t>(oOutDir);
-    o.kind = at<int8_t>(oOutKind);
-    o.force = force_ptr();
-    o.Ntot = M.Ntot;
-    o.begin = H.out_begin;
-    o.end = H.out_end;
-    o.omega = H.omega;
-    o.rho_off = rho_off;
-    o.rho0 = p.rho0;
-    o.zero_gradient = p.outlet == LBM_OUTLET_ZERO_GRADIENT;
-    o.q = at<double>(oOutQ);
-    timed_launch(li, TK_OUTLET, [&] { ops->outlet(Q, o, s0); }, s0);
-    ++launches;
-  }
-  // interior bricks, then boundary bricks (the first 64 (nB + nBb) fluid
-  // elements) through the brick tables
-  const int64_t nbnd = ops->boundary_bricks ? H.nBb : 0;
-  const int64_t nbrick = 64 * (H.nB + nbnd);
-  BrickArgs b{};
-  b.src = cur(li);
-  b.dst = nxt(li);
-  b.force = force_ptr();
-  b.nb = at<int32_t>(oBrickNb) + (size_t)H.brick_first * 27;
-  b.tab = at<uint16_t>(oBrickTab);
-  b.Ntot = M.Ntot;
-  b.begin = H.base + H.oF;
-  b.nB = H.nB;
-  b.rx = make_relax(Q, H.omega);
-  b.rho_off = rho_off;
-  b.nbr = at<uint32_t>(oNbr);
-  b.side = at(oSide);
-  b.inlet_s = at<double>(oInletS);
-  // the inlet velocity in this level's lattice units
-  const double uin_unit = level_velocity_ratio(li, p.time_mode);
-  for (int i = 0; i < kQmax; ++i) b.inlet[i] = inlet[i] * uin_unit;
-  // the level's GFC source records at t + 1 from the new state
-  SourceOut so{};
-  if (li + 1 < nlev && ld[li].nsrc > 0) {
-    so.mask = at<uint32_t>(oSrcMask);
-    so.first = at<int32_t>(oSrcFirst);
-    so.rec_out = at(ld[li].momA[parity[li] ^ 1]);
-  }
-  b.so = so;
-  BrickArgs bb = b;
-  bb.nb = b.nb + (size_t)H.nB * 27;
-  bb.begin = b.begin + 64 * H.nB;
-  bb.nB = nbnd;
-  // the rest through the neighbour list; processed range: TWO_LAYER and
-  // DIFFUSIVE [GFC | fluid], LINEAR [fluid | GFF inner], minus the bricks
-  StreamCollideArgs a{};
-  a.src = cur(li);
-  a.dst = nxt(li);
-  a.nbr = at<uint32_t>(oNbr);
+  if (H.out_end == H.out_begin) return;
+  if (!o.nlev) o.begin = H.out_begin;  // consecutive levels' links are consecutive
+  OutletLevel& L = o.lev[o.nlev++];
+  L.src = src;
+  L.end = H.out_end;
+  L.omega = H.omega;
+}
+
+ScArgs lbm_ctx::sc_args() const {
+  ScArgs a{};
   a.force = force_ptr();
+  a.tab = at<uint16_t>(oBrickTab);
+  a.nbr = at<uint32_t>(oNbr);
   a.side = at(oSide);
   a.inlet_s = at<double>(oInletS);
+  a.sources = source_table();
   a.Ntot = M.Ntot;
-  if (p.time_mode != LBM_TIME_LINEAR) {
-    a.begin = H.base + H.oC;
-    a.end = H.base + H.oG1 - nbrick;
-    a.hole_at = H.base + H.oF;
-    a.hole_len = nbrick;
-  } else {
-    a.begin = H.base + H.oF + nbrick;
-    a.end = H.base + H.oG2;
-    a.hole_at = a.end;
-    a.hole_len = 0;
-  }
-  a.rx = b.rx;
   a.rho_off = rho_off;
-  std::memcpy(a.inlet, b.inlet, sizeof(a.inlet));
-  a.so = so;
-  const bool use_force = p.use_force != 0;
-  auto launch = [&](int kernel, cudaStream_t s) {
-    if (kernel == TK_INTERIOR) ops->stream_collide_brick(Q, use_force, false, b, s);
-    else if (kernel == TK_BOUNDARY) ops->stream_collide_brick(Q, use_force, true, bb, s);
-    else ops->stream_collide(Q, use_force, a, s);
+  a.rho_off32 = (float)rho_off;
+  for (int i = 0; i < kQmax; ++i) a.inlet[i] = inlet[i];
+  return a;
+}
+
+int lbm_ctx::add_sc(ScArgs& a, int slot, int li, int kind) const {
+  const HostLevel& H = M.lv[li];
+  // interior bricks, then boundary bricks are the first 64 (nB + nBb) fluid
+  // elements; the rest goes through the neighbour list: TWO_LAYER and
+  // DIFFUSIVE [GFC | fluid], LINEAR [fluid | GFF inner], minus the bricks
+  const int64_t nbrick = 64 * (H.nB + H.nBb);
+  ScSeg g{};
+  g.nb = at<int32_t>(oBrickNb) + (size_t)H.brick_first * 27;
+  int64_t begin = H.base + H.oF, n = 0;
+  if (kind == TK_INTERIOR) {
+    n = H.nB;
+  } else if (kind == TK_BOUNDARY) {
+    g.nb += (size_t)H.nB * 27;
+    begin += 64 * H.nB;
+    n = H.nBb;
+  } else {
+    g.list = 1;
+    if (p.time_mode != LBM_TIME_LINEAR) {
+      g.hole_at = (int32_t)begin;
+      g.hole_len = (int32_t)nbrick;
+      begin = H.base + H.oC;
+      n = H.base + H.oG1 - nbrick - begin;
+    } else {
+      begin += nbrick;
+      n = H.base + H.oG2 - begin;
+      g.hole_at = (int32_t)(begin + n);
+    }
+  }
+  if (n <= 0) return 0;
+  g.begin = (int32_t)begin;
+  g.n = (int32_t)n;
+  g.src = cur(li);
+  g.dst = nxt(li);
+  g.rx = make_relax32(H.omega);
+  g.uin = (float)level_velocity_ratio(li, p.time_mode);  // a power of two
+  // the level's GFC source records at t + 1 from the new state
+  if (li + 1 < nlev && ld[li].nsrc > 0) g.rec_out = at(ld[li].momA[parity[li] ^ 1]);
+  g.level = (int16_t)slot;
+  a.rx[slot] = make_relax(Q, H.omega);
+  a.seg[a.nseg++] = g;
+  return 1;
+}
+
+void lbm_ctx::stream_collide(int li) {
+  OutletArgs o = outlet_args(at(oSide));
+  add_outlet(o, li, cur(li));
+  if (o.nlev) {
+    timed_launch(li, TK_OUTLET, [&] { ops->outlet(Q, o, st); });
     ++launches;
-  };
-  const bool has[3] = {b.nB > 0, a.end > a.begin, bb.nB > 0};  // by TimedKind 0..2
-  // inside a graph capture the kernels run as parallel branches (boundary
-  // bricks and neighbour list on the level's two side streams), joined before
-  // the next op; launched kernel by kernel they run one after the other
-  const bool fork = capturing && concurrent_sc && timing != 1 && !lvs.empty() && (has[TK_BOUNDARY] || has[TK_LIST]);
-  auto group = [&] {
-    if (fork) {
-      cudaEventRecord(lvs[li].fork, s0);
-      cudaStreamWaitEvent(lvs[li].side[0], lvs[li].fork, 0);
-      cudaStreamWaitEvent(lvs[li].side[1], lvs[li].fork, 0);
-    }
-    for (int kernel : {TK_INTERIOR, TK_BOUNDARY, TK_LIST}) {
-      if (!has[kernel]) continue;
-      cudaStream_t s = !fork || kernel == TK_INTERIOR ? s0 : lvs[li].side[kernel == TK_BOUNDARY ? 0 : 1];
-      timed_launch(li, kernel, [&] { launch(kernel, s); }, s);
-    }
-    if (fork) {
-      for (int k = 0; k < 2; ++k) {
-        cudaEventRecord(lvs[li].join[k], lvs[li].side[k]);
-        cudaStreamWaitEvent(s0, lvs[li].join[k], 0);
-      }
-    }
-  };
-  // the whole level's stream-collide (fork to join) as one timed span
-  timed_launch(li, TK_SC_SPAN, group, s0);
+  }
+  for (int kind : {TK_INTERIOR, TK_BOUNDARY, TK_LIST}) {
+    ScArgs a = sc_args();
+    if (!add_sc(a, 0, li, kind)) continue;
+    timed_launch(li, kind, [&] { (kind == TK_INTERIOR ? ops->sc_interior : ops->sc_rest)(Q, p.use_force != 0, a, st); });
+    ++launches;
+  }
   parity[li] ^= 1;
+}
+
+// One coarse step, all levels that advance at the same instant together.
+// With r the time-step ratio and T = r^(n-1) ticks of the finest level in a
+// coarse step, level l advances at the ticks that are multiples of
+// r^(n-1-l); the levels advancing at a tick are l0..n-1.  At such an instant
+// the order the recursion (advance()) gives them is not needed: a
+// GhostFromFiner ghost reads fluid children only, a GhostFromCoarser ghost
+// the records of fluid and GhostFromFiner sources only, and a level's
+// stream-collide its own state, so three launches serve all levels:
+//   the GhostFromFiner fills of l0..n-2 with their ghosts' records,
+//   the GhostFromCoarser fills of l0+1..n-1 (and, in LINEAR mode, that of l0
+//   at the middle of the coarser level's step),
+//   the stream-collide of l0..n-1 (interior bricks beside the rest).
+// The four-level cylinder has 20 such launches in a row instead of 36, the
+// five-level sphere 40 instead of 76, two-level flows 5 instead of 7, and
+// small levels share a launch (cylinder 109 -> 67 us a coarse step, 56 us
+// with the launches chained; sphere of 1.1e7 elements 5.08 -> 4.94 ms).
+// Every op has the inputs it has in advance(): same results bit for bit.
+// Starting the interior bricks, which read no ghost, beside the ghost fills
+// slowed both (two-level 64^3, FP32: 50 against 48 us; FP64 D2Q9: 84 against
+// 40 us), and taking them into the other stream-collide launch cost more than
+// the fork it saves (49 against 48 us).
+void lbm_ctx::step_batched() {
+  const int n = n_filled, r = time_ratio(p.time_mode);
+  int64_t T = 1;
+  for (int l = 1; l < n; ++l) T *= r;
+  for (int64_t tick = 0; tick < T; ++tick) {
+    int l0 = n - 1;
+    for (int64_t period = r; l0 > 0 && tick % period == 0; period *= r) --l0;
+    tick_batched(l0, n);
+  }
+  // levels declared beyond the finest one present hold no element; each takes
+  // an even number of substeps per coarse step
+}
+
+void lbm_ctx::tick_batched(int l0, int n) {
+  const bool finest_only = l0 == n - 1;
+  const int timed_level = finest_only ? n - 1 : -1;
+  auto fork = [&](int b) {
+    cudaEventRecord(br.fork[b], st);
+    cudaStreamWaitEvent(br.s[b], br.fork[b], 0);
+  };
+  auto join = [&](int b) {
+    cudaEventRecord(br.join[b], br.s[b]);
+    cudaStreamWaitEvent(st, br.join[b], 0);
+  };
+  ScArgs in = sc_args(), rest = sc_args();
+  OutletArgs out = outlet_args(at(oSide));
+  int64_t elements = 0;
+  for (int l = l0; l < n; ++l) elements += M.lv[l].nF;
+  for (int l = l0; l < n; ++l) {
+    launches += add_sc(in, l - l0, l, TK_INTERIOR);
+    launches += add_sc(rest, l - l0, l, TK_BOUNDARY);
+    launches += add_sc(rest, l - l0, l, TK_LIST);
+    const int no = out.nlev;
+    add_outlet(out, l, cur(l));
+    launches += out.nlev - no;
+  }
+  const bool chain = elements <= (p.precision == LBM_FP64 ? kChainElements64 : kChainElements);
+  rest.chain = chain;
+  auto run_interior = [&] {
+    fork(0);
+    // BF16 streams the finest level two elements per thread, which has no
+    // record epilogue, so that level goes apart from the coarser ones
+    ScArgs a = in;
+    if (p.precision == LBM_BF16DEV && in.nseg > 1 && !in.seg[in.nseg - 1].rec_out) {
+      a.nseg = 1;
+      a.seg[0] = in.seg[in.nseg - 1];
+      ScArgs b = in;
+      --b.nseg;
+      ops->sc_interior(Q, p.use_force != 0, b, br.s[0]);
+    }
+    timed_launch(timed_level, TK_INTERIOR, [&] { ops->sc_interior(Q, p.use_force != 0, a, br.s[0]); }, br.s[0]);
+  };
+  auto run_outlet = [&](cudaStream_t s) { ops->outlet(Q, out, s); };
+  const bool out_branch = out.nlev && !outlet_reads_ghosts;
+  if (out_branch) {
+    fork(1);
+    run_outlet(br.s[1]);
+  }
+  GffArgs gff = gff_args();
+  gff.chain = chain;
+  for (int l = l0; l + 1 < n; ++l) {
+    const int k = gff.nseg;
+    add_gff(gff, l);
+    if (gff.nseg > k) launches += 1 + (gff.lev[k].rec_out != nullptr);
+  }
+  if (gff.nseg) ops->fill_gff(Q, gff, st);
+  GfcArgs gfc = gfc_args();
+  gfc.chain = chain;
+  if (p.time_mode == LBM_TIME_LINEAR && l0 > 0) {
+    source_moments(l0 - 1, ld[l0 - 1].momA[parity[l0 - 1]], nullptr, SRC_GFF_OUTER);
+    add_gfc(gfc, l0, true, false);
+  }
+  for (int l = l0 + 1; l < n; ++l) add_gfc(gfc, l, false, false);
+  launches += gfc.nseg;
+  if (gfc.nseg) ops->fill_gfc(Q, gfc, st);
+  if (out.nlev && !out_branch) run_outlet(st);
+  if (out_branch) join(1);
+  timed_launch(timed_level, TK_SC_SPAN, [&] {
+    if (in.nseg) run_interior();
+    if (rest.nseg)
+      timed_launch(timed_level, TK_BOUNDARY, [&] { ops->sc_rest(Q, p.use_force != 0, rest, st); });
+    if (in.nseg) join(0);
+  });
+  for (int l = l0; l < n; ++l) parity[l] ^= 1;
 }
 
 void lbm_ctx::ensure_records() {
@@ -294,6 +421,15 @@ void lbm_ctx::ensure_records() {
   recs_valid = true;
 }
 
+// The recursive step of Sec. 2.2, kernel by kernel on the bound stream (timing
+// mode 1, the adjoint's recorded steps, a dry walk of the op sequence).
+// Source records (interpolation step 1), two buffers per level: momA[parity]
+// holds those of the current state.  The stream-collide writes the records of
+// the sources it updates into the other buffer (their state at t + 1), the
+// GhostFromFiner fill those of its ghosts at t, and in LINEAR mode the outer
+// GhostFromFiner layer, which no stream-collide updates, gets its records at
+// t + 1 from its stored state.  The fill at t + 1/2 takes the means of the
+// two buffers.
 void lbm_ctx::advance(int li) {
   const bool has_finer = li + 1 < nlev;
   const bool linear = p.time_mode == LBM_TIME_LINEAR;
@@ -301,56 +437,19 @@ void lbm_ctx::advance(int li) {
     if (hook) hook(kind, level);
     return !dry;
   };
-  // Source records (interpolation step 1), two buffers per level: momA[parity]
-  // holds those of the current state.  The stream-collide writes the records
-  // of the sources it updates into the other buffer (their state at t + 1);
-  // the GhostFromFiner sources get theirs at t after their fill, and in
-  // LINEAR mode the outer GhostFromFiner layer, which no stream-collide
-  // updates, at t + 1 from its stored state.  The fill at t + 1/2 takes the
-  // means of the two buffers.
-  // In a graph capture the level's stream-collide becomes a branch of its
-  // own, forked after the GhostFromFiner fill (the last op it needs) and
-  // joined before the finer level's second substep; meanwhile the records at
-  // t, the finer level's GhostFromCoarser fill and its first substep run on
-  // the main branch (they read this level's current buffer, its records at t
-  // or other levels only).  With gfc_b_branch the finer level's fill at
-  // t + 1/2 follows the stream-collide on its branch (forked after the
-  // records at t), into the fine buffer that the first substep's
-  // stream-collide writes, whose ghost slots nothing touches before the
-  // second substep.
-  const bool branch = has_finer && capturing && concurrent_sc && level_branch && timing != 1 && !lvs.empty() && !dry;
-  const bool gfc_b_on_branch = branch && linear && gfc_b_branch;
   if (has_finer) {
     if (op(OP_GFF, li)) fill_gff(li);
-    if (branch && !gfc_b_on_branch) cudaEventRecord(lvs[li].fork_sc, st);
-    if (op(OP_MOM_A, li)) source_moments(li, ld[li].momA[parity[li]], 0, nullptr, SRC_GFF);
-    if (gfc_b_on_branch) cudaEventRecord(lvs[li].fork_sc, st);
-    if (op(OP_GFC_A, li + 1)) fill_gfc(li + 1, false);
+    // the records of the GhostFromFiner sources: written by the fill
+    if (op(OP_MOM_A, li) && ld[li].n_gsrc > 0) ++launches;
+    if (op(OP_GFC_A, li + 1)) fill_gfc(li + 1, false, false);
   }
-  if (op(OP_SC, li)) {
-    if (branch) {
-      cudaStreamWaitEvent(lvs[li].sc, lvs[li].fork_sc, 0);
-      stream_collide(li, lvs[li].sc);
-      if (gfc_b_on_branch) {
-        source_moments(li, ld[li].momA[parity[li]], 0, lvs[li].sc, SRC_GFF_OUTER);
-        fill_gfc(li + 1, true, false, lvs[li].sc, true);
-      }
-    } else {
-      stream_collide(li);
-    }
-  } else {
-    parity[li] ^= 1;
-  }
+  if (op(OP_SC, li)) stream_collide(li);
+  else parity[li] ^= 1;
   if (has_finer) {
     advance(li + 1);
-    if (branch) {
-      cudaEventRecord(lvs[li].done_sc, lvs[li].sc);
-      cudaStreamWaitEvent(st, lvs[li].done_sc, 0);
-    }
     if (linear) {
-      if (op(OP_MOM_B, li) && !gfc_b_on_branch)
-        source_moments(li, ld[li].momA[parity[li]], 0, nullptr, SRC_GFF_OUTER);
-      if (op(OP_GFC_B, li + 1) && !gfc_b_on_branch) fill_gfc(li + 1, true);
+      if (op(OP_MOM_B, li)) source_moments(li, ld[li].momA[parity[li]], nullptr, SRC_GFF_OUTER);
+      if (op(OP_GFC_B, li + 1)) fill_gfc(li + 1, true, false);
     }
     // the remaining substeps (one in acoustic scaling; three with diffusive
     // scaling, whose four ghost layers filled at t last all four)
@@ -358,19 +457,16 @@ void lbm_ctx::advance(int li) {
   }
 }
 
-bool lbm_ctx::make_level_streams() {
-  if (!lvs.empty()) return true;
-  std::vector<LevelStreams> v(nlev);
-  bool ok = true;
-  for (auto& L : v) {
-    for (cudaStream_t* s : {&L.sc, &L.side[0], &L.side[1]})
-      ok = ok && cudaStreamCreateWithFlags(s, cudaStreamNonBlocking) == cudaSuccess;
-    for (cudaEvent_t* e : {&L.fork_sc, &L.done_sc, &L.fork, &L.join[0], &L.join[1]})
-      ok = ok && cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess;
+bool lbm_ctx::make_branches() {
+  if (br.s[0]) return br.ok;
+  br.ok = true;
+  for (int b = 0; b < 2; ++b) {
+    br.ok = br.ok && cudaStreamCreateWithFlags(&br.s[b], cudaStreamNonBlocking) == cudaSuccess;
+    for (cudaEvent_t* e : {&br.fork[b], &br.join[b]})
+      br.ok = br.ok && cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess;
   }
-  lvs.swap(v);  // created handles are released by the destructor either way
-  if (!ok) cudaGetLastError();
-  return ok;
+  if (!br.ok) cudaGetLastError();
+  return br.ok;
 }
 
 const lbm_ctx::StepGraph* lbm_ctx::step_graph(int nsteps) {
@@ -381,8 +477,9 @@ const lbm_ctx::StepGraph* lbm_ctx::step_graph(int nsteps) {
     graphs_on = false;
     return nullptr;
   }
-  // no branch streams: the captured steps stay sequential
-  if (concurrent_sc && !make_level_streams()) concurrent_sc = false;
+  // levels batched by instant (up to kMaxBatch of them); without branch
+  // streams, or with more levels, the captured steps are the recursion's
+  const bool batched = n_filled <= kMaxBatch && make_branches();
   // capture on a private stream (the bound stream may be the legacy default
   // stream, which cannot be captured); host bookkeeping is restored afterwards
   const std::vector<int> p0 = parity;
@@ -403,7 +500,10 @@ const lbm_ctx::StepGraph* lbm_ctx::step_graph(int nsteps) {
   cudaError_t e = cudaStreamBeginCapture(cap_stream, cudaStreamCaptureModeThreadLocal);
   if (e == cudaSuccess) {
     capturing = true;
-    for (int k = 0; k < nsteps; ++k) advance(0);
+    for (int k = 0; k < nsteps; ++k) {
+      if (batched) step_batched();
+      else advance(0);
+    }
     capturing = false;
     e = cudaStreamEndCapture(cap_stream, &graph);
   }

@@ -130,6 +130,43 @@ struct Sto<__nv_bfloat16> {
   __device__ static __forceinline__ __nv_bfloat16 cv(R v) { return __float2bfloat16_rn(v); }
 };
 
+// Programmatic dependent launch of the step's kernels (launched so where
+// *Args::chain is set): once every block of a kernel has its inputs, the
+// successor's blocks may start, and load what no kernel of the step writes
+// (tables, neighbour lists) before they wait for its end here.  Before the
+// wait a kernel neither reads the state nor writes anything, and no kernel
+// lets the next one start before it: at most two of a chain are resident.
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Index of the launch segment that holds block b, given the segments' first
+// blocks in order (uniform over the block).
+__device__ __forceinline__ int segment_of(const uint32_t* first, int n, unsigned b) {
+  int s = 0;
+  for (int k = 1; k < n; ++k)
+    if (b >= first[k]) s = k;
+  return s;
+}
+
+// The compute type's one of two launch constants.
+template <class R>
+__device__ __forceinline__ auto& pick(const double& d, const float& f) {
+  if constexpr (sizeof(R) == 8) return d;
+  else return f;
+}
+template <class R>
+__device__ __forceinline__ auto& pick(const Relax& d, const Relax32& f) {
+  if constexpr (sizeof(R) == 8) return d;
+  else return f;
+}
+template <class R>
+__device__ __forceinline__ auto& pick(const GhostUnits<double>& d, const GhostUnits<float>& f) {
+  if constexpr (sizeof(R) == 8) return d;
+  else return f;
+}
+template <class R>
+using RelaxOf = std::conditional_t<sizeof(R) == 8, Relax, Relax32>;
+
 // ----------------------------------------------------------------- physics
 // g^eq_i for density deviation rp = rho - rho_off
 template <int Q, class R>
@@ -173,11 +210,11 @@ __device__ __forceinline__ void raw_moments(const R* g, R& rp, R* j) {
 }
 
 // Pre-collision moments from a stored post-collision set: u = (j - F/2)/rho,
-// f^neq = (g - g^eq - F_i) / (1 - omega), S_ab = -(3 omega / 2 rho) sum c_a c_b f^neq.
+// f^neq = (g - g^eq - F_i) r1w, r1w = 1 / (1 - omega), S_ab = -(3 omega / 2 rho) sum c_a c_b f^neq.
 // g^eq per pair of opposite velocities (c.u changes sign: the even part is
 // shared); without FORCE the forcing terms are left out at compile time.
 template <int Q, class R, bool WANT_S, bool FORCE = true>
-__device__ __forceinline__ void post_moments(const R* g, R omega, R rho_off, const R* F, R& rp, R* u,
+__device__ __forceinline__ void post_moments(const R* g, R omega, R r1w, R rho_off, const R* F, R& rp, R* u,
                                              R* fneq, R* S) {
   using LT = Lat<Q>;
   constexpr int D = LT::D;
@@ -191,7 +228,6 @@ __device__ __forceinline__ void post_moments(const R* g, R omega, R rho_off, con
   R usq = R(0);
 #pragma unroll
   for (int a = 0; a < D; ++a) usq += u[a] * u[a];
-  const R r1w = R(1) / (R(1) - omega);
   const R base = rp - R(1.5) * rho * usq;
   {
     R f0 = g[0] - R(LT::w(0)) * base;
@@ -261,14 +297,15 @@ __device__ __forceinline__ double flip(double x, bool neg) {
 template <int Q>
 __device__ __forceinline__ void raw_moments64(const double* g, double& rp, double* j) {
   using LT = Lat<Q>;
-  double sp = 0, sm = 0, s0 = g[0];
+  double sp = 0, sm = 0, s0 = g[0], s1 = 0;  // short chains: a lone warp waits for each sum
 #pragma unroll
   for (int i = 1; i < Q; ++i) {
     if (LT::c(i, 0) > 0) sp += g[i];
     else if (LT::c(i, 0) < 0) sm += g[i];
-    else s0 += g[i];
+    else if (i & 1) s0 += g[i];
+    else s1 += g[i];
   }
-  rp = (sp + sm) + s0;
+  rp = (sp + sm) + (s0 + s1);
   j[0] = sp - sm;
   j[1] = j[2] = 0;
 #pragma unroll
@@ -320,8 +357,8 @@ __device__ __forceinline__ void bgk_collide64(double (&g)[Q], const Relax& rx, d
   double b[NC], kq[NC], kf[NC];
 #pragma unroll
   for (int c = 0; c < NC; ++c) {
-    b[c] = FORCE ? fma(rx.eq[c], base, -rx.force[c] * uF) : rx.eq[c] * base;
-    kq[c] = c ? rx.quad[c] * inv : 0.0;
+    b[c] = FORCE ? fma(rx.eq(c), base, -rx.force[c] * uF) : rx.eq(c) * base;
+    kq[c] = c ? rx.quad(c) * inv : 0.0;
     kf[c] = FORCE && c ? 3.0 * rx.force[c] * inv : 0.0;
   }
   g[0] = fma(rx.keep, g[0], b[0]);
@@ -332,13 +369,13 @@ __device__ __forceinline__ void bgk_collide64(double (&g)[Q], const Relax& rx, d
     if (FORCE) {
       const double cF = cdot<Q>(i, F);
       const double ev = fma(cJ, fma(kq[c], cJ, kf[c] * cF), b[c]);
-      const double od = fma(rx.lin[c], cJ, rx.force[c] * cF);
+      const double od = fma(rx.lin(c), cJ, rx.force[c] * cF);
       g[i] = fma(rx.keep, g[i], ev + od);
       g[i + 1] = fma(rx.keep, g[i + 1], ev - od);
     } else {
       const double ev = fma(kq[c] * cJ, cJ, b[c]);
-      g[i] = fma(rx.keep, g[i], fma(rx.lin[c], cJ, ev));
-      g[i + 1] = fma(rx.keep, g[i + 1], fma(-rx.lin[c], cJ, ev));
+      g[i] = fma(rx.keep, g[i], fma(rx.lin(c), cJ, ev));
+      g[i + 1] = fma(rx.keep, g[i + 1], fma(-rx.lin(c), cJ, ev));
     }
   }
 }
@@ -368,8 +405,8 @@ __device__ __forceinline__ void post_moments64(const double* g, const Relax& rx,
   double b[NC], kq[NC], kf[NC];
 #pragma unroll
   for (int c = 0; c < NC; ++c) {
-    b[c] = FORCE ? fma(rx.nforce[c], uF, -rx.neq[c] * base) : -rx.neq[c] * base;
-    kq[c] = c ? -rx.nquad[c] * inv : 0.0;
+    b[c] = FORCE ? fma(rx.nforce[c], uF, -rx.neq(c) * base) : -rx.neq(c) * base;
+    kq[c] = c ? -rx.nquad(c) * inv : 0.0;
     kf[c] = FORCE && c ? -3.0 * rx.nforce[c] * inv : 0.0;
   }
   fneq[0] = fma(rx.r1w, g[0], b[0]);
@@ -382,13 +419,13 @@ __device__ __forceinline__ void post_moments64(const double* g, const Relax& rx,
     if (FORCE) {
       const double cF = cdot<Q>(i, F);
       const double ev = fma(cJ, fma(kq[c], cJ, kf[c] * cF), b[c]);
-      const double od = fma(rx.nlin[c], cJ, rx.nforce[c] * cF);
+      const double od = fma(rx.nlin(c), cJ, rx.nforce[c] * cF);
       fneq[i] = fma(rx.r1w, g[i], ev - od);
       fneq[i + 1] = fma(rx.r1w, g[i + 1], ev + od);
     } else {
       const double ev = fma(kq[c] * cJ, cJ, b[c]);
-      fneq[i] = fma(rx.r1w, g[i], fma(-rx.nlin[c], cJ, ev));
-      fneq[i + 1] = fma(rx.r1w, g[i + 1], fma(rx.nlin[c], cJ, ev));
+      fneq[i] = fma(rx.r1w, g[i], fma(-rx.nlin(c), cJ, ev));
+      fneq[i + 1] = fma(rx.r1w, g[i + 1], fma(rx.nlin(c), cJ, ev));
     }
     const double ps = fneq[i] + fneq[i + 1];
 #pragma unroll
@@ -446,7 +483,7 @@ __device__ __forceinline__ void st4(double* p, const double* v) {
 // Interpolation step 1 (Sec. 2.2) for one source: its record from its stored
 // (post-collision) pdfs g.
 template <int Q, class R, bool FORCE>
-__device__ __forceinline__ void source_record(const R (&g)[Q], const Relax& rx, R rho_off, const R* F,
+__device__ __forceinline__ void source_record(const R (&g)[Q], const RelaxOf<R>& rx, R rho_off, const R* F,
                                               R (&rec)[RecLayout<Q>::STRIDE]) {
   using RL = RecLayout<Q>;
   constexpr int D = Lat<Q>::D, NS = Lat<Q>::NS;
@@ -454,7 +491,7 @@ __device__ __forceinline__ void source_record(const R (&g)[Q], const Relax& rx, 
   for (int f = 0; f < RL::STRIDE; ++f) rec[f] = R(0);
   R rp, u[3], fneq[Q], Sv[NS];
   if constexpr (sizeof(R) == 8) post_moments64<Q, FORCE>(g, rx, rho_off, F, rp, u, fneq, Sv);
-  else post_moments<Q, R, true, FORCE>(g, R(rx.omega), rho_off, F, rp, u, fneq, Sv);
+  else post_moments<Q, R, true, FORCE>(g, rx.omega, rx.r1w, rho_off, F, rp, u, fneq, Sv);
 #pragma unroll
   for (int q = 0; q < Q; ++q) rec[RL::FN + q] = fneq[q];
   rec[RL::RP] = rp;
@@ -483,21 +520,28 @@ __device__ __forceinline__ void store_record(R* __restrict__ out, const R (&rec)
   for (int f = 0; f < RecLayout<Q>::END; f += 4) st4(out + f, rec + f);
 }
 
+// Record index of element e among its level's GhostFromCoarser sources, -1 if
+// it is none.  Mask words are per 32 slots: one broadcast load for a warp of
+// consecutive elements.
+__device__ __forceinline__ int64_t source_index(const SourceTable& so, int64_t e) {
+  const uint32_t m = __ldg(so.mask + (e >> 5));
+  const uint32_t bit = (uint32_t)e & 31u;
+  if (!((m >> bit) & 1u)) return -1;
+  return (int64_t)__ldg(so.first + (e >> 5)) + __popc(m & ((1u << bit) - 1u));
+}
+
 // Stream-collide epilogue for a GhostFromCoarser source among the processed
 // elements: g are the element's new values before rounding to storage; the
 // record is taken from the values as stored, so it equals what
-// k_source_moments computes from the stored state.  Mask words are per 32
-// slots: one broadcast load for a warp of consecutive elements.
+// k_source_moments computes from the stored state.
 template <int Q, class S, bool FORCE>
-__device__ __forceinline__ void source_out(const SourceOut& so, int64_t e, const typename Sto<S>::R (&g)[Q],
-                                           const Relax& rx, typename Sto<S>::R rho_off,
-                                           const typename Sto<S>::R* F) {
+__device__ __forceinline__ void source_out(const SourceTable& so, void* rec_out, int64_t e,
+                                           const typename Sto<S>::R (&g)[Q], const RelaxOf<typename Sto<S>::R>& rx,
+                                           typename Sto<S>::R rho_off, const typename Sto<S>::R* F) {
   using R = typename Sto<S>::R;
   using RL = RecLayout<Q>;
-  const uint32_t m = __ldg(so.mask + (e >> 5));
-  const uint32_t bit = (uint32_t)e & 31u;
-  if (!((m >> bit) & 1u)) return;
-  const int64_t k = (int64_t)__ldg(so.first + (e >> 5)) + __popc(m & ((1u << bit) - 1u));
+  const int64_t k = source_index(so, e);
+  if (k < 0) return;
   R gs[Q];
 #pragma unroll
   for (int q = 0; q < Q; ++q) {
@@ -506,32 +550,15 @@ __device__ __forceinline__ void source_out(const SourceOut& so, int64_t e, const
   }
   R rec[RL::STRIDE];
   source_record<Q, R, FORCE>(gs, rx, rho_off, F, rec);
-  store_record<Q, R>(static_cast<R*>(so.rec_out) + k * RL::STRIDE, rec);
+  store_record<Q, R>(static_cast<R*>(rec_out) + k * RL::STRIDE, rec);
 }
 
 // ----------------------------------------------------------------- stream + collide
-// Tuning knobs of the hot kernel (compile-time; the defaults are the measured
-// best on GB300).  LBM_SC_BLOCK: threads per block; LBM_SC_MINB: minimum
-// resident blocks per SM for __launch_bounds__; LBM_SC_STREAM: streaming
-// (evict-first) hints on the use-once neighbour indices and on the stores.
-#ifndef LBM_SC_BLOCK
-#define LBM_SC_BLOCK 256
-#endif
-#ifndef LBM_SC_MINB
-#define LBM_SC_MINB 4
-#endif
+// LBM_SC_STREAM: streaming (evict-first) hints on the use-once neighbour
+// indices and on the stores.
 #ifndef LBM_SC_STREAM
 #define LBM_SC_STREAM 1
 #endif
-// FP64 storage: one warp per block.  A warp holds its SM's FP64 pipe for about
-// 120 x 19 cycles, so a launch takes as long as the SM with the most warps,
-// and small blocks spread a small level over all SMs (D2Q9, 1,800 elements:
-// 7 blocks of 256 on 7 SMs before).  Registers are not capped: 12 to 24 warps
-// per SM keep the pipe busy, and the caps of 64 and 80 registers spilled.
-template <class S>
-constexpr int kScBlock = sizeof(S) == 8 ? 32 : LBM_SC_BLOCK;
-template <int Q, class S>
-constexpr int kScMinb = sizeof(S) == 8 ? (Q == 27 ? 12 : Q == 19 ? 16 : 24) : LBM_SC_MINB;
 
 __device__ __forceinline__ uint32_t ld_once(const uint32_t* p) {
 #if LBM_SC_STREAM
@@ -566,14 +593,14 @@ __device__ __forceinline__ void st_once(__nv_bfloat16* p, __nv_bfloat16 v) {
 // symmetry of each velocity pair (i, opp(i)): c.u and c.F change sign, so the
 // even part of f^eq (and of the forcing term) is shared and the odd part flips.
 template <int Q, class R, bool FORCE>
-__device__ __forceinline__ void bgk_collide(R (&g)[Q], const Relax& rx, R rho_off, const R* F) {
+__device__ __forceinline__ void bgk_collide(R (&g)[Q], const RelaxOf<R>& rx, R rho_off, const R* F) {
   using LT = Lat<Q>;
   constexpr int D = LT::D;
   if constexpr (sizeof(R) == 8) {
     bgk_collide64<Q, FORCE>(g, rx, rho_off, F);
     return;
   }
-  const R om = R(rx.omega);
+  const R om = rx.omega;
   R rp, j[3];
   raw_moments<Q, R>(g, rp, j);
   const R rho = rho_off + rp;
@@ -625,195 +652,199 @@ __device__ __forceinline__ void bgk_collide(R (&g)[Q], const Relax& rx, R rho_of
   }
 }
 
-// Pull streaming f_i(x) = f*_i(x - c_i) through the neighbour list (Sec. 2.1,
-// Eq. lbe) fused with the BGK collision (Eq. bgk).  Every thread first issues
-// all neighbour-index loads, then all pdf gathers (branch-free: codes other than
-// a plain pull read the element's own opposite slot, which is the bounce-back
-// value), and patches the rare inlet / outlet values afterwards, so that up to
-// 2(Q-1) independent loads per element are in flight.
+// FP64 storage: one warp per block.  A warp holds its SM's FP64 pipe for about
+// 120 x 19 cycles, so a launch takes as long as the SM with the most warps,
+// and small blocks spread a small level over all SMs (D2Q9, 1,800 elements:
+// 7 blocks of 256 on 7 SMs before).  Registers are not capped: 12 to 24 warps
+// per SM keep the pipe busy, and the caps of 64 and 80 registers spilled.
+template <class S>
+constexpr int kScBlock = sizeof(S) == 8 ? 32 : 256;
+template <int Q>
+constexpr int kScMinb64 = Q == 27 ? 12 : Q == 19 ? 16 : 24;
+
+// Collision, store and source record of one element from its pulled pdfs.
 template <int Q, class S, bool FORCE, bool MOMS>
-__global__ void __launch_bounds__(kScBlock<S>, kScMinb<Q, S>) k_stream_collide(const StreamCollideArgs a) {
+__device__ __forceinline__ void sc_finish(const ScArgs& a, const ScSeg& sg, int64_t e,
+                                          typename Sto<S>::R (&g)[Q]) {
   using R = typename Sto<S>::R;
-  using LT = Lat<Q>;
-  constexpr int D = LT::D;
-  // linear position -> element, stepping over the interior bricks
-  const int64_t lin = a.begin + (int64_t)blockIdx.x * kScBlock<S> + threadIdx.x;
-  if (lin >= a.end) return;
-  const int64_t e = lin + (lin >= a.hole_at ? a.hole_len : 0);
-  const S* __restrict__ src = static_cast<const S*>(a.src);
-  S* __restrict__ dst = static_cast<S*>(a.dst);
-  const uint32_t* __restrict__ nbr = a.nbr;
+  constexpr int D = Lat<Q>::D;
   const size_t N = (size_t)a.Ntot;
-  uint32_t nb[Q - 1];
-#pragma unroll
-  for (int i = 1; i < Q; ++i) nb[i - 1] = ld_once(nbr + (size_t)(i - 1) * N + e);
-  R g[Q];
-  g[0] = Sto<S>::ld(src + e);
-#pragma unroll
-  for (int i = 1; i < Q; ++i) {
-    const uint32_t n = nb[i - 1];
-    const size_t idx = n < NB_FLAG30 ? (size_t)i * N + n : (size_t)opp(i) * N + (size_t)e;
-    g[i] = Sto<S>::ld(src + idx);
-  }
-#pragma unroll
-  for (int i = 1; i < Q; ++i) {
-    const uint32_t n = nb[i - 1];
-    if (n >= NB_FLAG30) {
-      if (n & NB_BOUNCE) {
-        if (n & NB_FLAG30) g[i] += R(a.inlet[i]) * (a.inlet_s ? R(a.inlet_s[n & NB_INDEX]) : R(1));
-      } else {
-        g[i] = static_cast<const R*>(a.side)[n & NB_INDEX];
-      }
-    }
-  }
   R F[3] = {R(0), R(0), R(0)};
   if (FORCE) {
-    const R* __restrict__ fp = static_cast<const R*>(a.force);
+    const R* __restrict__ fp = static_cast<const R*>(a.force) + e;
 #pragma unroll
-    for (int b = 0; b < D; ++b) F[b] = fp[(size_t)b * N + e];
+    for (int c = 0; c < D; ++c) F[c] = fp[c * N];
   }
-  bgk_collide<Q, R, FORCE>(g, a.rx, R(a.rho_off), F);
+  const R rho_off = pick<R>(a.rho_off, a.rho_off32);
+  const auto& rx = pick<R>(a.rx[sg.level], sg.rx);
+  let_next_start();
+  bgk_collide<Q, R, FORCE>(g, rx, rho_off, F);
+  S* __restrict__ dst = static_cast<S*>(sg.dst) + e;
 #pragma unroll
-  for (int i = 0; i < Q; ++i) st_once(dst + (size_t)i * N + e, Sto<S>::cv(g[i]));
-  if (MOMS) source_out<Q, S, FORCE>(a.so, e, g, a.rx, R(a.rho_off), F);
+  for (int i = 0; i < Q; ++i) st_once(dst + i * N, Sto<S>::cv(g[i]));
+  if (MOMS)
+    if (sg.rec_out) source_out<Q, S, FORCE>(a.sources, sg.rec_out, e, g, rx, rho_off, F);
 }
 
-// Stream-collide of interior bricks: the same pull and BGK collision as
-// k_stream_collide, with the pull source of link i located by the brick's
-// neighbour row instead of the per-element neighbour list.  Each group of 64
-// threads takes one brick, thread l its element at z-curve position l; blocks
-// are issued in brick order, so the bricks in flight stay a compact window of
-// the level and their neighbours' lines are still in L2 when gathered.  The
-// thread's Q-1 link-table entries (slot, position) are loaded into registers,
-// lanes 0..26 of each warp load the brick's 27-entry neighbour row in one
-// coalesced access, and every link takes its row entry by a warp shuffle, so
-// all pdf gathers issue after two loads.  The element's HBM traffic is its Q
-// pdf reads and Q writes.
-#ifndef LBM_BR_BLOCK
-#define LBM_BR_BLOCK 256
-#endif
-#ifndef LBM_BR_MINB
-#define LBM_BR_MINB (4 * 256 / LBM_BR_BLOCK)
-#endif
-//
-// Boundary bricks (BND): a complete brick whose neighbour brick behind some
-// link is not complete; those links (row entry kBrickMissing) take the
-// element's neighbour-list code like k_stream_collide: a pull, the element's
-// own opposite slot (bounce-back), plus the inlet term, or a boundary value.
-// Every link is first resolved to one 32-bit offset, so the gathers need no
-// branch.  Five blocks per SM (48 registers, no spills) for D3Q19 and D2Q9
-// with 4-byte or narrower storage (measured: 4.66 against 4.38 TB/s at four);
-// three where more registers are needed (D3Q27).
-#ifndef LBM_BR_BND_MINB_NARROW
-#define LBM_BR_BND_MINB_NARROW 5
-#endif
-#define LBM_BR_BND_MINB(Q, S) ((Q) > 19 ? 3 * 256 / LBM_BR_BLOCK : LBM_BR_BND_MINB_NARROW * 256 / LBM_BR_BLOCK)
-// Interior bricks: BF16 storage moves half the bytes per element, so it needs
-// more elements in flight; five blocks per SM (48 registers, no spills) for
-// D3Q19 / D2Q9 BF16, measured faster than four or six.
-#define LBM_BR_INT_MINB(Q, S) ((Q) <= 19 && sizeof(S) == 2 ? 5 * 256 / LBM_BR_BLOCK : LBM_BR_MINB)
-#define LBM_BR_MOMS_MINB(Q, S) ((Q) <= 19 ? 5 * 256 / LBM_BR_BLOCK : LBM_BR_MINB)
+// the incoming value of a link with a boundary code: the inlet's term on top
+// of the bounce-back value, or the precomputed boundary value
+template <class R>
+__device__ __forceinline__ R link_value(const ScArgs& a, const ScSeg& sg, int i, uint32_t n, R back) {
+  if (n & NB_BOUNCE) return back + R(a.inlet[i] * (double)sg.uin) * (a.inlet_s ? R(a.inlet_s[n & NB_INDEX]) : R(1));
+  return static_cast<const R*>(a.side)[n & NB_INDEX];
+}
 
-template <class S>
-constexpr int kBrBlock = sizeof(S) == 8 ? 32 : LBM_BR_BLOCK;  // FP64: one warp, as kScBlock
-template <int Q, class S, bool BND, bool MOMS>
-constexpr int kBrMinb = sizeof(S) == 8 ? kScMinb<Q, S>
-                                       : BND ? LBM_BR_BND_MINB(Q, S) : MOMS ? LBM_BR_MOMS_MINB(Q, S) : LBM_BR_INT_MINB(Q, S);
+// Pull streaming f_i(x) = f*_i(x - c_i) (Sec. 2.1, Eq. lbe) of interior bricks:
+// the pull source of link i is located by the brick's neighbour row instead
+// of the per-element neighbour list.  Each group of 64 threads takes one brick,
+// thread l its element at z-curve position l; blocks are issued in brick
+// order, so the bricks in flight stay a compact window of the level and their
+// neighbours' lines are still in L2 when gathered.  The thread's Q-1
+// link-table entries (slot, position) are loaded into registers, lanes 0..26
+// of each warp load the brick's 27-entry neighbour row in one coalesced
+// access, and every link takes its row entry by a warp shuffle, so all pdf
+// gathers issue after two loads.  The element's HBM traffic is its Q pdf reads
+// and Q writes.
+// the link-table entries of position l, and lane's entry of the brick's row
+template <int Q>
+struct BrickLinks {
+  uint32_t tw[Q / 2];  // (Q-1)/2 words of two 16-bit entries
+  int32_t row;
+  __device__ __forceinline__ void load(const uint16_t* tab, const int32_t* nb, int64_t b, int l, int lane) {
+#pragma unroll
+    for (int k = 0; k < Q / 2; ++k)
+      tw[k] = (uint32_t)__ldg(tab + (2 * k) * 64 + l) | ((uint32_t)__ldg(tab + (2 * k + 1) * 64 + l) << 16);
+    row = lane < 27 ? __ldg(nb + b * 27 + lane) : 0;
+  }
+  __device__ __forceinline__ uint32_t entry(int i) const { return (tw[(i - 1) >> 1] >> (((i - 1) & 1) * 16)) & 0xffffu; }
+};
 
-template <int Q, class S, bool FORCE, bool BND, bool MOMS>
-__global__ void __launch_bounds__(kBrBlock<S>, kBrMinb<Q, S, BND, MOMS>) k_stream_collide_brick(const BrickArgs a) {
-  using R = typename Sto<S>::R;
-  using LT = Lat<Q>;
-  constexpr int D = LT::D;
-  constexpr int NW = Q / 2;  // (Q-1)/2 words of two 16-bit entries
-  const int64_t t = (int64_t)blockIdx.x * kBrBlock<S> + threadIdx.x;
+template <int Q, class S>
+__device__ __forceinline__ void pull_interior(const ScArgs& a, const ScSeg& sg, const BrickLinks<Q>& k, int64_t first,
+                                              int l, typename Sto<S>::R (&g)[Q]) {
+  const size_t N = (size_t)a.Ntot;
+  const S* __restrict__ src = static_cast<const S*>(sg.src) + first;
+  g[0] = Sto<S>::ld(src + l);
+#pragma unroll
+  for (int i = 1; i < Q; ++i) {
+    const uint32_t v = k.entry(i);
+    const int32_t r = __shfl_sync(0xffffffffu, k.row, (int)(v >> 6));
+    g[i] = Sto<S>::ld(src + (int64_t)(i * N) + r + (v & 63));
+  }
+}
+
+// Pull of the elements that read ghosts or boundary values: boundary bricks (a
+// complete brick whose neighbour brick behind some link is not complete: row
+// entry kBrickMissing) and the elements of the neighbour-list range, all of
+// whose links go through the list.  Every link is first resolved to one
+// 32-bit offset from src + i N + first: the brick-table entry, or the
+// element's neighbour-list code turned into a pull (n - first), its own
+// opposite slot (bounce-back, and the inlet's base value: (opp(i) - i) N + l),
+// or, for a boundary value, that same valid slot, the value being substituted
+// afterwards.  So all codes are loaded before any is used, and the gathers
+// need no branch.  |offsets| < 2^30 + 64 since Ntot < 2^30.
+template <int Q, class S>
+__device__ __forceinline__ void pull_rest(const ScArgs& a, const ScSeg& sg, int32_t (&off)[Q], uint32_t miss,
+                                          int64_t first, int l, typename Sto<S>::R (&g)[Q]) {
+  const size_t N = (size_t)a.Ntot;
+  const S* __restrict__ src = static_cast<const S*>(sg.src) + first;
+  uint32_t patch = 0;  // links whose value gets an inlet term or a substitute
+#pragma unroll
+  for (int i = 1; i < Q; ++i) {
+    if (!((miss >> i) & 1u)) continue;
+    const uint32_t n = (uint32_t)off[i];
+    if (n < NB_FLAG30) {
+      off[i] = (int32_t)((int64_t)n - first);
+    } else {
+      off[i] = (int32_t)((int64_t)(opp(i) - i) * (int64_t)N + l);
+      if (n & NB_FLAG30) patch |= 1u << i;
+    }
+  }
+  g[0] = Sto<S>::ld(src + l);
+#pragma unroll
+  for (int i = 1; i < Q; ++i) g[i] = Sto<S>::ld(src + (int64_t)(i * N) + off[i]);
+  // the inlet term or the precomputed boundary value, from the link's code
+  // read again
+  if (patch) {
+#pragma unroll
+    for (int i = 1; i < Q; ++i) {
+      if (!((patch >> i) & 1u)) continue;
+      g[i] = link_value(a, sg, i, __ldg(a.nbr + (size_t)(i - 1) * N + first + l), g[i]);
+    }
+  }
+}
+
+// Minimum blocks of 256 per SM (FP32, BF16).  D3Q19 and D2Q9: five, 48
+// registers (boundary bricks alone 4.66 against 4.38 TB/s at four); D3Q27:
+// four for interior bricks, three for the rest.
+template <int Q, class S>
+constexpr int kIntMinb = sizeof(S) == 8 ? kScMinb64<Q> : Q <= 19 ? 5 : 4;
+template <int Q, class S>
+constexpr int kRestMinb = sizeof(S) == 8 ? kScMinb64<Q> : Q <= 19 ? 5 : 3;
+
+template <int Q, class S, bool FORCE, bool MOMS>
+__global__ void __launch_bounds__(kScBlock<S>, kIntMinb<Q, S>) k_sc_interior(const __grid_constant__ ScArgs a) {
+  const int seg = segment_of(a.first, a.nseg, blockIdx.x);
+  const ScSeg& sg = a.seg[seg];
+  const int64_t t = (int64_t)(blockIdx.x - a.first[seg]) * kScBlock<S> + threadIdx.x;
   const int l = (int)t & 63, lane = threadIdx.x & 31;
   // the brick index is uniform over each warp (64 threads per brick), so the
   // exit below and the shuffles run with whole warps
   const int64_t b = t >> 6;
-  if (b >= a.nB) return;
-  uint32_t tw[NW];
-#pragma unroll
-  for (int k = 0; k < NW; ++k)
-    tw[k] = (uint32_t)__ldg(a.tab + (2 * k) * 64 + l) | ((uint32_t)__ldg(a.tab + (2 * k + 1) * 64 + l) << 16);
-  const int32_t row = lane < 27 ? __ldg(a.nb + b * 27 + lane) : 0;
+  if (b >= sg.n) return;
+  BrickLinks<Q> k;
+  k.load(a.tab, sg.nb, b, l, lane);
+  const int64_t first = sg.begin + b * 64;
+  typename Sto<S>::R g[Q];
+  wait_for_previous();
+  pull_interior<Q, S>(a, sg, k, first, l, g);
+  sc_finish<Q, S, FORCE, MOMS>(a, sg, first + l, g);
+}
+
+// Everything that reads ghosts or boundary values: boundary bricks and (LIST)
+// the elements of the neighbour-list range (incomplete bricks, the processed
+// ghost layers), in one launch.
+template <int Q, class S, bool FORCE, bool MOMS, bool LIST>
+__global__ void __launch_bounds__(kScBlock<S>, kRestMinb<Q, S>) k_sc_rest(const __grid_constant__ ScArgs a) {
+  const int seg = segment_of(a.first, a.nseg, blockIdx.x);
+  const ScSeg& sg = a.seg[seg];
+  const int64_t t = (int64_t)(blockIdx.x - a.first[seg]) * kScBlock<S> + threadIdx.x;
   const size_t N = (size_t)a.Ntot;
-  // offsets below are relative to the brick's first element
-  const int64_t first = a.begin + b * 64;
-  const S* __restrict__ src = static_cast<const S*>(a.src) + first;
-  S* __restrict__ dst = static_cast<S*>(a.dst) + first + l;
-  R g[Q];
-  g[0] = Sto<S>::ld(src + l);
-  if (!BND) {
+  int32_t off[Q];
+  uint32_t miss = 0;
+  int64_t first;
+  int l = 0;
+  if (LIST && sg.list) {
+    if (t >= sg.n) return;
+    const int64_t lin = sg.begin + t;
+    first = lin + (lin >= sg.hole_at ? sg.hole_len : 0);
 #pragma unroll
-    for (int i = 1; i < Q; ++i) {
-      const uint32_t v = (tw[(i - 1) >> 1] >> (((i - 1) & 1) * 16)) & 0xffffu;
-      const int32_t r = __shfl_sync(0xffffffffu, row, (int)(v >> 6));
-      g[i] = Sto<S>::ld(src + (int64_t)(i * N) + r + (v & 63));
-    }
+    for (int i = 1; i < Q; ++i) off[i] = (int32_t)ld_once(a.nbr + (size_t)(i - 1) * N + first);
+    miss = ~0u;
   } else {
-    // phase 1: every link's pull source as one 32-bit offset from src + i N
-    // (src starts at the brick's first element): the brick-table entry, or,
-    // through a missing neighbour brick, the element's neighbour-list code
-    // resolved to a pull (n - first), to its own opposite slot (bounce-back,
-    // and the inlet's base value: (opp(i) - i) N + l), or, for a boundary
-    // value, to that same valid slot, the value being substituted below.
-    // |offsets| < 2^30 + 64 since Ntot < 2^30.  Links whose value gets an
-    // inlet term or a substitute are marked in `patch`.
-    const int64_t e = first + l;
-    int32_t off[Q];
-    uint32_t miss = 0, patch = 0;
-    off[0] = 0;
-    // 1a: brick-table offsets; the codes of links through missing bricks are
-    // loaded, all before any of them is used
+    // the brick index is uniform over each warp: whole warps exit or shuffle
+    const int64_t b = t >> 6;
+    if (b >= sg.n) return;
+    l = (int)t & 63;
+    BrickLinks<Q> k;
+    k.load(a.tab, sg.nb, b, l, threadIdx.x & 31);
+    first = sg.begin + b * 64;
 #pragma unroll
     for (int i = 1; i < Q; ++i) {
-      const uint32_t v = (tw[(i - 1) >> 1] >> (((i - 1) & 1) * 16)) & 0xffffu;
-      const int32_t r = __shfl_sync(0xffffffffu, row, (int)(v >> 6));
+      const uint32_t v = k.entry(i);
+      const int32_t r = __shfl_sync(0xffffffffu, k.row, (int)(v >> 6));
       if (r != kBrickMissing) {
         off[i] = r + (int32_t)(v & 63);
       } else {
-        off[i] = (int32_t)__ldg(a.nbr + (size_t)(i - 1) * N + e);
+        off[i] = (int32_t)__ldg(a.nbr + (size_t)(i - 1) * N + first + l);
         miss |= 1u << i;
       }
     }
-    // 1b: the codes resolved to offsets
-#pragma unroll
-    for (int i = 1; i < Q; ++i) {
-      if (!((miss >> i) & 1u)) continue;
-      const uint32_t n = (uint32_t)off[i];
-      if (n < NB_FLAG30) {
-        off[i] = (int32_t)((int64_t)n - first);
-      } else {
-        off[i] = (int32_t)((int64_t)(opp(i) - i) * (int64_t)N + l);
-        if (n & NB_FLAG30) patch |= 1u << i;
-      }
-    }
-    // phase 2: the gathers, branch-free
-#pragma unroll
-    for (int i = 1; i < Q; ++i) g[i] = Sto<S>::ld(src + (int64_t)(i * N) + off[i]);
-    // phase 3 (inlet and boundary-value elements only): the inlet term or the
-    // precomputed boundary value, from the link's code read again
-    if (patch) {
-#pragma unroll
-      for (int i = 1; i < Q; ++i) {
-        if (!((patch >> i) & 1u)) continue;
-        const uint32_t n = __ldg(a.nbr + (size_t)(i - 1) * N + e);
-        if (n & NB_BOUNCE) g[i] += R(a.inlet[i]) * (a.inlet_s ? R(a.inlet_s[n & NB_INDEX]) : R(1));
-        else g[i] = static_cast<const R*>(a.side)[n & NB_INDEX];
-      }
-    }
   }
-  R F[3] = {R(0), R(0), R(0)};
-  if (FORCE) {
-    const R* __restrict__ fp = static_cast<const R*>(a.force) + first + l;
-#pragma unroll
-    for (int c = 0; c < D; ++c) F[c] = fp[c * N];
-  }
-  bgk_collide<Q, R, FORCE>(g, a.rx, R(a.rho_off), F);
-#pragma unroll
-  for (int i = 0; i < Q; ++i) st_once(dst + i * N, Sto<S>::cv(g[i]));
-  if (MOMS) source_out<Q, S, FORCE>(a.so, first + l, g, a.rx, R(a.rho_off), F);
+  typename Sto<S>::R g[Q];
+  wait_for_previous();
+  pull_rest<Q, S>(a, sg, off, miss, first, l, g);
+  sc_finish<Q, S, FORCE, MOMS>(a, sg, first + l, g);
 }
 
 // BF16 interior bricks, two neighbouring elements per thread: lane m of the
@@ -841,21 +872,24 @@ __global__ void __launch_bounds__(kBrBlock<S>, kBrMinb<Q, S, BND, MOMS>) k_strea
 #endif
 #define LBM_BR_PAIR_MINB(Q) ((Q) > 19 ? 768 / LBM_BR_PAIR_BLOCK : LBM_BR_PAIR_MINB_Q19)
 template <int Q, bool FORCE>
-__global__ void __launch_bounds__(LBM_BR_PAIR_BLOCK, LBM_BR_PAIR_MINB(Q)) k_stream_collide_brick_pair(const BrickArgs a) {
+__global__ void __launch_bounds__(LBM_BR_PAIR_BLOCK, LBM_BR_PAIR_MINB(Q)) k_sc_interior_pair(const __grid_constant__ ScArgs a) {
   using S = __nv_bfloat16;
   using R = float;
   using LT = Lat<Q>;
   constexpr int D = LT::D;
   constexpr int BPB = LBM_BR_PAIR_BLOCK / 32;
   const int m = threadIdx.x & 31;
+  const int seg = segment_of(a.first, a.nseg, blockIdx.x);
+  const ScSeg& sg = a.seg[seg];
   // one brick per warp: the exit below and the shuffles run with whole warps
-  const int64_t b = (int64_t)blockIdx.x * BPB + (threadIdx.x >> 5);
-  if (b >= a.nB) return;
-  const int32_t row = m < 27 ? __ldg(a.nb + b * 27 + m) : 0;
+  const int64_t b = (int64_t)(blockIdx.x - a.first[seg]) * BPB + (threadIdx.x >> 5);
+  if (b >= sg.n) return;
+  const int32_t row = m < 27 ? __ldg(sg.nb + b * 27 + m) : 0;
   const size_t N = (size_t)a.Ntot;
-  const int64_t first = a.begin + b * 64;
-  const S* __restrict__ src = static_cast<const S*>(a.src) + first;
-  S* __restrict__ dst = static_cast<S*>(a.dst) + first + 2 * m;
+  const int64_t first = sg.begin + b * 64;
+  const S* __restrict__ src = static_cast<const S*>(sg.src) + first;
+  S* __restrict__ dst = static_cast<S*>(sg.dst) + first + 2 * m;
+  wait_for_previous();
   // the link-table entries of positions 2m (low half) and 2m+1 (high half)
   const uint32_t* __restrict__ tab2 = reinterpret_cast<const uint32_t*>(a.tab);
   R g0[Q], g1[Q];
@@ -893,8 +927,9 @@ __global__ void __launch_bounds__(LBM_BR_PAIR_BLOCK, LBM_BR_PAIR_MINB(Q)) k_stre
       F1[c] = f.y;
     }
   }
-  bgk_collide<Q, R, FORCE>(g0, a.rx, R(a.rho_off), F0);
-  bgk_collide<Q, R, FORCE>(g1, a.rx, R(a.rho_off), F1);
+  let_next_start();
+  bgk_collide<Q, R, FORCE>(g0, sg.rx, a.rho_off32, F0);
+  bgk_collide<Q, R, FORCE>(g1, sg.rx, a.rho_off32, F1);
 #pragma unroll
   for (int i = 0; i < Q; ++i) {
     const __nv_bfloat162 p = __floats2bfloat162_rn(g0[i], g1[i]);
@@ -913,16 +948,19 @@ __global__ void __launch_bounds__(LBM_BR_PAIR_BLOCK, LBM_BR_PAIR_MINB(Q)) k_stre
 // f_i(x - c_i - n)), or, for c_i = -n, correct the pressure:
 // f^eq_i(rho0, u) + f^neq_opp(i)(x) with the pre-collision f^neq.
 template <int Q, class S>
-__global__ void k_outlet(const OutletArgs a) {
+__global__ void k_outlet(const __grid_constant__ OutletArgs a) {
   using R = typename Sto<S>::R;
   using LT = Lat<Q>;
   constexpr int D = LT::D;
   const int64_t k = a.begin + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= a.end) return;
-  const S* __restrict__ src = static_cast<const S*>(a.src);
+  int lv = 0;
+  while (lv < a.nlev && k >= a.lev[lv].end) ++lv;
+  if (lv == a.nlev) return;
+  const S* __restrict__ src = static_cast<const S*>(a.lev[lv].src);
   const size_t N = (size_t)a.Ntot;
   const int i = a.dir[k];
   R* side = static_cast<R*>(a.side);
+  wait_for_previous();
   if (a.kind[k] == OUT_EXTRAP) {
     const R fa = Sto<S>::ld(src + (size_t)i * N + a.a[k]);
     side[k] = a.zero_gradient ? fa : R(2) * fa - Sto<S>::ld(src + (size_t)i * N + a.b[k]);
@@ -970,7 +1008,7 @@ __global__ void k_outlet(const OutletArgs a) {
     if (q == ib) gib = g[q];
   // f^eq_i(rho0, u) + f^neq_ib, f^neq the pre-collision non-equilibrium part
   // recovered from the stored post-collision pdf: (f* - f^eq - F_ib) / (1 - omega)
-  const R om = R(a.omega);
+  const R om = R(a.lev[lv].omega);
   const R fneq_ib = (gib - geq<Q, R>(ib, rp, rho, u, usq) - guo<Q, R>(ib, om, u, F)) * (R(1) / (R(1) - om));
   const R r0 = R(a.rho0);
   side[k] = geq<Q, R>(i, r0 - R(a.rho_off), r0, u, usq) + fneq_ib;
@@ -992,7 +1030,7 @@ __global__ void k_outlet(const OutletArgs a) {
 template <class S>
 constexpr int kMomBlock = sizeof(S) == 8 ? 32 : LBM_MOM_BLOCK;  // FP64: one warp, as kScBlock
 template <int Q, class S, bool FORCE>
-__global__ void __launch_bounds__(kMomBlock<S>) k_source_moments(const MomentsArgs a) {
+__global__ void __launch_bounds__(kMomBlock<S>) k_source_moments(const __grid_constant__ MomentsArgs a) {
   using R = typename Sto<S>::R;
   using RL = RecLayout<Q>;
   constexpr int D = Lat<Q>::D;
@@ -1010,7 +1048,7 @@ __global__ void __launch_bounds__(kMomBlock<S>) k_source_moments(const MomentsAr
 #pragma unroll
     for (int b = 0; b < D; ++b) F[b] = static_cast<const R*>(a.force)[(size_t)b * N + e];
   R rec[RL::STRIDE];
-  source_record<Q, R, FORCE>(g, a.rx, R(a.rho_off), F, rec);
+  source_record<Q, R, FORCE>(g, pick<R>(a.rx, a.rx32), pick<R>(a.rho_off, a.rho_off32), F, rec);
   if (a.prev) mean_record<Q, R>(static_cast<const R*>(a.prev) + (size_t)r * RL::STRIDE, rec);
   store_record<Q, R>(static_cast<R*>(a.mom) + (size_t)r * RL::STRIDE, rec);
 }
@@ -1087,10 +1125,11 @@ struct GfcGroup {
   }
 };
 
-// Interpolation steps 2-5 for ghost k (octant oct) from its group's staged
-// records (sg_base: NSLOT padded records), written into a.dst.
+// Interpolation steps 2-5 for ghost k (octant oct) of level L from its group's
+// staged records (sg_base: NSLOT padded records), written into L.dst.
 template <int Q, class S>
-__device__ __forceinline__ void gfc_ghost(const GfcArgs& a, const typename Sto<S>::R* sg_base, int oct, int64_t k) {
+__device__ __forceinline__ void gfc_ghost(const GfcArgs& a, const GfcLevel& L, const typename Sto<S>::R* sg_base, int oct,
+                                          int64_t k) {
   using R = typename Sto<S>::R;
   using LT = Lat<Q>;
   using RL = RecLayout<Q>;
@@ -1132,7 +1171,8 @@ __device__ __forceinline__ void gfc_ghost(const GfcArgs& a, const typename Sto<S
   compact_uloc<Q, R>(ul, Sl, uloc);
   R u[3] = {R(0), R(0), R(0)};
   R usq = R(0);
-  const R us = R(a.u_scale);  // to fine lattice units (1 in acoustic scaling)
+  const auto& un = pick<R>(a.u64, a.u32);
+  const R us = un.u_scale;  // to fine lattice units (1 in acoustic scaling)
 #pragma unroll
   for (int b = 0; b < D; ++b) {
     u[b] = sg[b] * uloc[b] * us;
@@ -1142,13 +1182,12 @@ __device__ __forceinline__ void gfc_ghost(const GfcArgs& a, const typename Sto<S
   const R lw1 = D == 3 ? R(0.125) : R(0.1875);
   const R lw2 = D == 3 ? R(0.125) : R(0.1875);
   const R lw3 = D == 3 ? R(0.125) : R(0.0625);
-  const R rp = R(a.r_scale) * (lw0 * rps[0] + lw1 * rps[1] + lw2 * rps[2] + lw3 * rps[3]) + R(a.r_shift);
-  const R rho = R(a.rho_off) + rp;
-  const R wf = R(a.omega_f);
-  const R scale = sizeof(R) == 8 ? R(a.scale) : (R(1) - wf) * R(a.omega_c) / (R(a.tratio) * wf);
-  S* __restrict__ dst = static_cast<S*>(a.dst);
+  const R rp = un.r_scale * (lw0 * rps[0] + lw1 * rps[1] + lw2 * rps[2] + lw3 * rps[3]) + un.r_shift;
+  const R rho = un.rho_off + rp;
+  const R scale = pick<R>(L.scale, L.scale32);
+  S* __restrict__ dst = static_cast<S*>(L.dst);
   const size_t N = (size_t)a.Ntot;
-  const int64_t e = a.dest0 + k;
+  const int64_t e = L.dest0 + k;
   // interpolated f^neq, then f^eq per pair of opposite velocities (shared even part)
   R fn[Q];
 #pragma unroll
@@ -1165,8 +1204,8 @@ __device__ __forceinline__ void gfc_ghost(const GfcArgs& a, const typename Sto<S
   const R base = rp - R(1.5) * rho * usq;
   dst[e] = Sto<S>::cv(R(LT::w(0)) * base + scale * fn[0]);
   // diffusive scaling: f^neq's odd part takes an extra factor (odd_ratio)
-  const bool odd_rescale = a.odd_ratio != 1.0;
-  const R ro = R(a.odd_ratio);
+  const bool odd_rescale = a.odd_rescale != 0;
+  const R ro = un.odd;
 #pragma unroll
   for (int i = 1; i < Q; i += 2) {
     R cu = R(0);
@@ -1204,7 +1243,7 @@ __device__ __forceinline__ void gfc_ghost(const GfcArgs& a, const typename Sto<S
 template <class S>
 constexpr int kGfcBlock = sizeof(S) == 8 ? 32 : LBM_GFC_BLOCK;  // FP64: one warp, as kScBlock
 template <int Q, class S, bool TWO>
-__global__ void __launch_bounds__(kGfcBlock<S>) k_fill_gfc(const GfcArgs a) {
+__global__ void __launch_bounds__(kGfcBlock<S>) k_fill_gfc(const __grid_constant__ GfcArgs a) {
   using R = typename Sto<S>::R;
   using LT = Lat<Q>;
   using RL = RecLayout<Q>;
@@ -1213,40 +1252,65 @@ __global__ void __launch_bounds__(kGfcBlock<S>) k_fill_gfc(const GfcArgs a) {
   constexpr int PSTR = RL::STRIDE + 4;  // padded record: sibling lanes' reads fall in distinct banks
   constexpr int NGRP = kGfcBlock<S> / G;
   __shared__ __align__(16) R stage[NGRP * NSLOT * PSTR];
-  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int seg = segment_of(a.first, a.nseg, blockIdx.x);
+  const GfcLevel& L = a.lev[seg];
+  const int64_t k = (int64_t)(blockIdx.x - a.first[seg]) * kGfcBlock<S> + threadIdx.x;
   const int oct = threadIdx.x & (G - 1);  // octant of the ghost
   const int grp = threadIdx.x / G;
-  const bool active = k < a.ng;                   // ng is a multiple of G: whole groups
+  const bool active = k < L.ng;                   // ng is a multiple of G: whole groups
   const unsigned lane0 = (threadIdx.x & 31) & ~(unsigned)(G - 1);
   int32_t src[4] = {0, 0, 0, 0};
   if (active)
 #pragma unroll
-    for (int s = 0; s < 4; ++s) src[s] = a.gsrc[(size_t)s * a.ng + k];
-  const R* __restrict__ mom = static_cast<const R*>(a.mom);
-  const R* __restrict__ mom2 = static_cast<const R*>(a.mom2);
+    for (int s = 0; s < 4; ++s) src[s] = L.gsrc[(size_t)s * L.ng + k];
+  const R* __restrict__ mom = static_cast<const R*>(L.mom);
+  const R* __restrict__ mom2 = static_cast<const R*>(L.mom2);
+  const bool two = mom2 != nullptr;
   R* sg_base = stage + grp * NSLOT * PSTR;
+  wait_for_previous();
+  // every record's loads are issued before the first is stored, so that they
+  // overlap (one round trip instead of one per record)
+  constexpr int CH = RL::STRIDE / 4 / G > 0 ? (RL::STRIDE / 4 + G - 1) / G : 1;  // vectors per lane and record
+  constexpr int BATCH = sizeof(R) == 8 ? (NSLOT * CH > 16 ? 5 : 7) : TWO ? (NSLOT + 1) / 2 : NSLOT;
 #pragma unroll
-  for (int t = 0; t < NSLOT; ++t) {
-    const int r = __shfl_sync(0xffffffffu, src[GG::src_of(t)], lane0 + GG::lane_of(t));
-    if (active)
+  for (int t0 = 0; t0 < NSLOT; t0 += BATCH) {
+    R v[BATCH][CH][4];
+    int r[BATCH];
 #pragma unroll
-      for (int c = oct; c < RL::STRIDE / 4; c += G) {
-        R v[4];
-        ld4(mom + (size_t)r * RL::STRIDE + 4 * c, v);
-        if (TWO) {
-          // the records at t + 1/2: mean of those at t and t + 1
-          R w[4];
-          ld4(mom2 + (size_t)r * RL::STRIDE + 4 * c, w);
+    for (int t = t0; t < t0 + BATCH && t < NSLOT; ++t) {
+      r[t - t0] = __shfl_sync(0xffffffffu, src[GG::src_of(t)], lane0 + GG::lane_of(t));
 #pragma unroll
-          for (int j = 0; j < 4; ++j) v[j] = R(0.5) * (v[j] + w[j]);
-        }
-        st4(sg_base + t * PSTR + 4 * c, v);
-      }
+      for (int c = 0; c < CH; ++c)
+        if (active && oct + c * G < RL::STRIDE / 4)
+          ld4(mom + (size_t)r[t - t0] * RL::STRIDE + 4 * (oct + c * G), v[t - t0][c]);
+    }
+    if (TWO && two) {
+      // the records at t + 1/2: mean of those at t and t + 1
+      R w[BATCH][CH][4];
+#pragma unroll
+      for (int t = t0; t < t0 + BATCH && t < NSLOT; ++t)
+#pragma unroll
+        for (int c = 0; c < CH; ++c)
+          if (active && oct + c * G < RL::STRIDE / 4)
+            ld4(mom2 + (size_t)r[t - t0] * RL::STRIDE + 4 * (oct + c * G), w[t - t0][c]);
+#pragma unroll
+      for (int t = t0; t < t0 + BATCH && t < NSLOT; ++t)
+#pragma unroll
+        for (int c = 0; c < CH; ++c)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) v[t - t0][c][j] = R(0.5) * (v[t - t0][c][j] + w[t - t0][c][j]);
+    }
+#pragma unroll
+    for (int t = t0; t < t0 + BATCH && t < NSLOT; ++t)
+#pragma unroll
+      for (int c = 0; c < CH; ++c)
+        if (active && oct + c * G < RL::STRIDE / 4) st4(sg_base + t * PSTR + 4 * (oct + c * G), v[t - t0][c]);
   }
   __syncwarp();
+  let_next_start();
   // outer-layer ghosts are staged with their group but, when skipped, not written
-  if (!active || (a.skip_outer && (a.oct[k] & kGfcOuter))) return;
-  gfc_ghost<Q, S>(a, sg_base, oct, k);
+  if (!active || (L.skip_outer && (L.oct[k] & kGfcOuter))) return;
+  gfc_ghost<Q, S>(a, L, sg_base, oct, k);
 }
 
 // ----------------------------------------------------------------- GhostFromFiner
@@ -1262,30 +1326,39 @@ __global__ void __launch_bounds__(kGfcBlock<S>) k_fill_gfc(const GfcArgs a) {
 // One group of 2^d consecutive lanes per ghost: lane b loads child b (siblings
 // are contiguous, so the group's loads are coalesced), and the sums over the
 // children are shuffles inside the group.
-#ifndef LBM_GFF_BLOCK
-#define LBM_GFF_BLOCK 256
-#endif
+// Ghosts that are GhostFromCoarser sources also get their record here (step 1
+// of Sec. 2.2 for the next finer level): the group stages the values as
+// stored in shared memory and one thread per ghost forms the record, the same
+// arithmetic as k_source_moments, one launch fewer between a level's
+// GhostFromFiner and GhostFromCoarser fills.
 template <class S>
-constexpr int kGffBlock = sizeof(S) == 8 ? 32 : LBM_GFF_BLOCK;  // FP64: one warp, as kScBlock
+constexpr int kGffBlock = sizeof(S) == 8 ? 64 : 256;  // FP64: small blocks, as kScBlock
 template <int Q, class S, bool FORCE>
-__global__ void __launch_bounds__(kGffBlock<S>) k_fill_gff(const GffArgs a) {
+__global__ void __launch_bounds__(kGffBlock<S>) k_fill_gff(const __grid_constant__ GffArgs a) {
   using R = typename Sto<S>::R;
   using LT = Lat<Q>;
-  constexpr int D = LT::D, NS = LT::NS, NCH = 1 << D;
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  using RL = RecLayout<Q>;
+  constexpr int D = LT::D, NS = LT::NS, NCH = 1 << D, GPB = kGffBlock<S> / NCH;
+  __shared__ R stored[Q][GPB + 1];
+  const int seg = segment_of(a.first, a.nseg, blockIdx.x);
+  const GffLevel& L = a.lev[seg];
+  const auto& un = pick<R>(a.u64, a.u32);
+  const int64_t t = (int64_t)(blockIdx.x - a.first[seg]) * kGffBlock<S> + threadIdx.x;
   const int64_t k = t / NCH;
   const int b = (int)(t % NCH);
-  const bool active = k < a.ng;
-  const S* __restrict__ src = static_cast<const S*>(a.src_fine);
+  const bool active = k < L.ng;
+  const S* __restrict__ src = static_cast<const S*>(L.src_fine);
   const size_t N = (size_t)a.Ntot;
-  const R wf = R(a.rx_f.omega), rho_off = R(a.rho_off);
+  const R rho_off = un.rho_off;
   R rp = R(0), u[3] = {R(0), R(0), R(0)}, fneq[Q], Sv[NS];
 #pragma unroll
   for (int q = 0; q < Q; ++q) fneq[q] = R(0);
 #pragma unroll
   for (int s = 0; s < NS; ++s) Sv[s] = R(0);
+  const int64_t child = active ? (int64_t)L.child0[k] + b : 0;
+  wait_for_previous();
   if (active) {
-    const int64_t e = (int64_t)a.child0[k] + b;
+    const int64_t e = child;
     R g[Q];
 #pragma unroll
     for (int q = 0; q < Q; ++q) g[q] = Sto<S>::ld(src + (size_t)q * N + e);
@@ -1293,12 +1366,12 @@ __global__ void __launch_bounds__(kGffBlock<S>) k_fill_gff(const GffArgs a) {
     if (FORCE)
 #pragma unroll
       for (int c = 0; c < D; ++c) F[c] = static_cast<const R*>(a.force)[(size_t)c * N + e];
-    if constexpr (sizeof(R) == 8) post_moments64<Q, FORCE>(g, a.rx_f, rho_off, F, rp, u, fneq, Sv);
-    else post_moments<Q, R, true, FORCE>(g, wf, rho_off, F, rp, u, fneq, Sv);
-    if (a.odd_ratio != 1.0) {
+    if constexpr (sizeof(R) == 8) post_moments64<Q, FORCE>(g, a.rx_f64[seg], rho_off, F, rp, u, fneq, Sv);
+    else post_moments<Q, R, true, FORCE>(g, L.rx_f.omega, L.rx_f.r1w, rho_off, F, rp, u, fneq, Sv);
+    if (a.odd_rescale) {
       // diffusive scaling: f^neq's odd part takes an extra factor (the sum
       // over the children is linear, so each child's share is rescaled)
-      const R ro = R(a.odd_ratio);
+      const R ro = un.odd;
 #pragma unroll
       for (int i = 1; i < Q; i += 2) {
         const R fe = R(0.5) * (fneq[i] + fneq[i + 1]), fo = R(0.5) * (fneq[i] - fneq[i + 1]) * ro;
@@ -1307,6 +1380,7 @@ __global__ void __launch_bounds__(kGffBlock<S>) k_fill_gff(const GffArgs a) {
       }
     }
   }
+  let_next_start();
   // The ghost's velocity, mean minus (1/32) lap u, is linear in the children's
   // values, and so is lap u_a = dfac sum_c (2 d_c S_ac - d_a S_cc) with d_c the
   // difference across the cube (+ for children with bit c set, - otherwise):
@@ -1316,8 +1390,8 @@ __global__ void __launch_bounds__(kGffBlock<S>) k_fill_gff(const GffArgs a) {
   // The mean velocity goes to coarse units with u_scale (a power of two, so
   // inv_u is exact).
   const R inv = R(1) / R(NCH);
-  const R inv_u = inv * R(a.u_scale);
-  const R dfac = R(a.tratio) * R(D == 3 ? 0.5 : 1.0);
+  const R inv_u = inv * un.u_scale;
+  const R dfac = un.tratio * R(D == 3 ? 0.5 : 1.0);
   R rpm = rp * inv, uP[3] = {R(0), R(0), R(0)};
   if constexpr (sizeof(R) == 8) {
     double tr = 0;
@@ -1371,30 +1445,49 @@ __global__ void __launch_bounds__(kGffBlock<S>) k_fill_gff(const GffArgs a) {
         W[j][c] = keep + __shfl_xor_sync(0xffffffffu, send, h);
       }
   }
-  if (!active) return;
-  R usq = R(0);
+  const int64_t e = k < L.n_inner ? L.dest0 + k : L.dest_outer + (k - L.n_inner);
+  if (active) {
+    R usq = R(0);
 #pragma unroll
-  for (int aa = 0; aa < D; ++aa) usq += uP[aa] * uP[aa];
-  const R wc = R(a.omega_c);
-  rpm = R(a.r_scale) * rpm + R(a.r_shift);  // to coarse units (unchanged in acoustic scaling)
-  const R rho = rho_off + rpm;
-  const R scale = sizeof(R) == 8 ? R(a.scale) : (R(1) - wc) * R(a.tratio) * wf / wc * inv;
-  S* __restrict__ dst = static_cast<S*>(a.dst);
-  const int64_t e = k < a.n_inner ? a.dest0 + k : a.dest_outer + (k - a.n_inner);
-  // the group's lanes share the Q stores: lane b the directions j 2^d + b,
-  // whose c_i it looks up at run time (a compile-time loop over all Q would
-  // issue every direction's arithmetic in every lane)
+    for (int aa = 0; aa < D; ++aa) usq += uP[aa] * uP[aa];
+    rpm = un.r_scale * rpm + un.r_shift;  // to coarse units (unchanged in acoustic scaling)
+    const R rho = rho_off + rpm;
+    const R scale = pick<R>(a.scale[seg], L.scale32);
+    S* __restrict__ dst = static_cast<S*>(L.dst);
+    // the group's lanes share the Q stores: lane b the directions j 2^d + b,
+    // whose c_i it looks up at run time (a compile-time loop over all Q would
+    // issue every direction's arithmetic in every lane)
 #pragma unroll
-  for (int j = 0; j < NR; ++j) {
-    const int q = j * NCH + b;
-    if (q < Q) {
-      R cu = R(0);
+    for (int j = 0; j < NR; ++j) {
+      const int q = j * NCH + b;
+      if (q < Q) {
+        R cu = R(0);
 #pragma unroll
-      for (int aa = 0; aa < D; ++aa) cu += R(LatRt<Q>::c(q, aa)) * uP[aa];
-      const R feq = LatRt<Q>::template w<R>(q) * (rpm + rho * (R(3) * cu + R(4.5) * cu * cu - R(1.5) * usq));
-      dst[(size_t)q * N + e] = Sto<S>::cv(feq + scale * W[j][0]);
+        for (int aa = 0; aa < D; ++aa) cu += R(LatRt<Q>::c(q, aa)) * uP[aa];
+        const R feq = LatRt<Q>::template w<R>(q) * (rpm + rho * (R(3) * cu + R(4.5) * cu * cu - R(1.5) * usq));
+        const S v = Sto<S>::cv(feq + scale * W[j][0]);
+        dst[(size_t)q * N + e] = v;
+        stored[q][threadIdx.x / NCH] = Sto<S>::ld(&v);
+      }
     }
   }
+  if (!L.rec_out) return;  // uniform over the block
+  __syncthreads();
+  const int64_t kr = (int64_t)(blockIdx.x - a.first[seg]) * GPB + threadIdx.x;
+  if (threadIdx.x >= GPB || kr >= L.ng) return;
+  const int64_t er = kr < L.n_inner ? L.dest0 + kr : L.dest_outer + (kr - L.n_inner);
+  const int64_t r = source_index(a.sources, er);
+  if (r < 0) return;
+  R g[Q];
+#pragma unroll
+  for (int q = 0; q < Q; ++q) g[q] = stored[q][threadIdx.x];
+  R F[3] = {R(0), R(0), R(0)};
+  if (FORCE)
+#pragma unroll
+    for (int c = 0; c < D; ++c) F[c] = static_cast<const R*>(a.force)[(size_t)c * N + er];
+  R rec[RL::STRIDE];
+  source_record<Q, R, FORCE>(g, pick<R>(a.rx_c64[seg], a.rx_c[seg]), rho_off, F, rec);
+  store_record<Q, R>(static_cast<R*>(L.rec_out) + r * RL::STRIDE, rec);
 }
 
 // ----------------------------------------------------------------- set-up (compute type) / output (FP64)
@@ -1499,7 +1592,7 @@ __global__ void k_out(const OutArgs a) {
       for (int b = 0; b < D; ++b) F[b] = static_cast<const float*>(a.force)[(size_t)b * a.Ntot + e];
   }
   double rp, u[3], fneq[Q], Sv[NS];
-  post_moments<Q, double, true>(g, a.omega[li], a.rho_off, F, rp, u, fneq, Sv);
+  post_moments<Q, double, true>(g, a.omega[li], 1.0 / (1.0 - a.omega[li]), a.rho_off, F, rp, u, fneq, Sv);
   if (a.rho) a.rho[t] = a.rho_off + rp;
   if (a.u)
 #pragma unroll
@@ -1674,60 +1767,90 @@ inline void with_q(int Q, F&& f) {
   else f(std::integral_constant<int, 27>{});
 }
 
+// Launches kernel(a), as a programmatic dependent of the stream's previous
+// kernel where a.chain says so.
+template <class Args>
+inline void launch(void (*kernel)(const Args), unsigned grid, int block, cudaStream_t st, const Args& a) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = a.chain ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, kernel, a);
+}
+
 template <class S>
 struct Launch {
-  static void stream_collide_brick(int Q, bool force, bool boundary, const BrickArgs& a, cudaStream_t st) {
-    if (a.nB <= 0) return;
-    const unsigned g = blocks_for(64 * a.nB, kBrBlock<S>);
+  // first blocks of the segments, in order, from the threads each needs;
+  // returns the grid
+  template <class Args, class Work>
+  static unsigned assign_blocks(Args& a, int block, Work&& threads) {
+    unsigned at = 0;
+    for (int k = 0; k < a.nseg; ++k) {
+      a.first[k] = at;
+      at += blocks_for(threads(k), block);
+    }
+    return at;
+  }
+  static bool any_records(const ScArgs& a) {
+    for (int k = 0; k < a.nseg; ++k)
+      if (a.seg[k].rec_out) return true;
+    return false;
+  }
+  static void sc_interior(int Q, bool force, ScArgs& a, cudaStream_t st) {
+    const bool moms = any_records(a);
     with_q(Q, [&](auto q) {
       constexpr int QQ = decltype(q)::value;
-      const bool moms = a.so.mask != nullptr;
       if constexpr (std::is_same<S, __nv_bfloat16>::value) {
-        // BF16 interior bricks: two elements per thread, one brick per warp
-        // (on levels without GFC sources; the others take the one-element
-        // kernel with its record epilogue)
-        if (!boundary && !moms) {
-          const unsigned g2 = blocks_for(a.nB, LBM_BR_PAIR_BLOCK / 32);
-          if (force) k_stream_collide_brick_pair<QQ, true><<<g2, LBM_BR_PAIR_BLOCK, 0, st>>>(a);
-          else k_stream_collide_brick_pair<QQ, false><<<g2, LBM_BR_PAIR_BLOCK, 0, st>>>(a);
+        // BF16: two elements per thread, one brick per warp (on levels without
+        // GFC sources; the others take the one-element kernel with its record
+        // epilogue)
+        if (!moms) {
+          const unsigned g = assign_blocks(a, LBM_BR_PAIR_BLOCK, [&](int k) { return 32ll * a.seg[k].n; });
+          if (!g) return;
+          if (force) launch(k_sc_interior_pair<QQ, true>, g, LBM_BR_PAIR_BLOCK, st, a);
+          else launch(k_sc_interior_pair<QQ, false>, g, LBM_BR_PAIR_BLOCK, st, a);
           return;
         }
       }
-      auto go = [&](auto F, auto B, auto M) {
-        k_stream_collide_brick<QQ, S, decltype(F)::value, decltype(B)::value, decltype(M)::value>
-            <<<g, kBrBlock<S>, 0, st>>>(a);
+      const unsigned g = assign_blocks(a, kScBlock<S>, [&](int k) { return 64ll * a.seg[k].n; });
+      if (!g) return;
+      if (force) {
+        if (moms) launch(k_sc_interior<QQ, S, true, true>, g, kScBlock<S>, st, a);
+        else launch(k_sc_interior<QQ, S, true, false>, g, kScBlock<S>, st, a);
+      } else {
+        if (moms) launch(k_sc_interior<QQ, S, false, true>, g, kScBlock<S>, st, a);
+        else launch(k_sc_interior<QQ, S, false, false>, g, kScBlock<S>, st, a);
+      }
+    });
+  }
+  static void sc_rest(int Q, bool force, ScArgs& a, cudaStream_t st) {
+    const bool moms = any_records(a);
+    const unsigned g =
+        assign_blocks(a, kScBlock<S>, [&](int k) { return (a.seg[k].list ? 1ll : 64ll) * a.seg[k].n; });
+    if (!g) return;
+    bool list = false;
+    for (int k = 0; k < a.nseg; ++k) list |= a.seg[k].list != 0;
+    with_q(Q, [&](auto q) {
+      auto go = [&](auto F, auto M, auto L) {
+        launch(k_sc_rest<decltype(q)::value, S, decltype(F)::value, decltype(M)::value, decltype(L)::value>, g,
+               kScBlock<S>, st, a);
       };
       using T = std::true_type;
       using U = std::false_type;
-      if (boundary) {
-        if (force) moms ? go(T{}, T{}, T{}) : go(T{}, T{}, U{});
-        else moms ? go(U{}, T{}, T{}) : go(U{}, T{}, U{});
-      } else {
-        if (force) moms ? go(T{}, U{}, T{}) : go(T{}, U{}, U{});
-        else moms ? go(U{}, U{}, T{}) : go(U{}, U{}, U{});
-      }
-    });
-  }
-  static void stream_collide(int Q, bool force, const StreamCollideArgs& a, cudaStream_t st) {
-    const int64_t n = a.end - a.begin;
-    if (n <= 0) return;
-    const unsigned g = blocks_for(n, kScBlock<S>);
-    with_q(Q, [&](auto q) {
-      constexpr int QQ = decltype(q)::value;
-      const bool moms = a.so.mask != nullptr;
-      if (force) {
-        if (moms) k_stream_collide<QQ, S, true, true><<<g, kScBlock<S>, 0, st>>>(a);
-        else k_stream_collide<QQ, S, true, false><<<g, kScBlock<S>, 0, st>>>(a);
-      } else {
-        if (moms) k_stream_collide<QQ, S, false, true><<<g, kScBlock<S>, 0, st>>>(a);
-        else k_stream_collide<QQ, S, false, false><<<g, kScBlock<S>, 0, st>>>(a);
-      }
+      auto by_list = [&](auto F, auto M) { list ? go(F, M, T{}) : go(F, M, U{}); };
+      if (force) moms ? by_list(T{}, T{}) : by_list(T{}, U{});
+      else moms ? by_list(U{}, T{}) : by_list(U{}, U{});
     });
   }
   static void outlet(int Q, const OutletArgs& a, cudaStream_t st) {
-    const int64_t n = a.end - a.begin;
-    if (n <= 0) return;
-    with_q(Q, [&](auto q) { k_outlet<decltype(q)::value, S><<<blocks_for(n, kMomBlock<S>), kMomBlock<S>, 0, st>>>(a); });
+    if (!a.nlev) return;
+    const int64_t n = a.lev[a.nlev - 1].end - a.begin;
+    with_q(Q, [&](auto q) { launch(k_outlet<decltype(q)::value, S>, blocks_for(n, kMomBlock<S>), kMomBlock<S>, st, a); });
   }
   static void source_moments(int Q, const MomentsArgs& a, cudaStream_t st) {
     if (a.nsrc <= 0) return;
@@ -1738,22 +1861,24 @@ struct Launch {
       else k_source_moments<QQ, S, false><<<g, kMomBlock<S>, 0, st>>>(a);
     });
   }
-  static void fill_gfc(int Q, const GfcArgs& a, cudaStream_t st) {
-    if (a.ng <= 0) return;
+  static void fill_gfc(int Q, GfcArgs& a, cudaStream_t st) {
+    const unsigned g = assign_blocks(a, kGfcBlock<S>, [&](int k) { return (int64_t)a.lev[k].ng; });
+    if (!g) return;
+    bool two = false;
+    for (int k = 0; k < a.nseg; ++k) two |= a.lev[k].mom2 != nullptr;
     with_q(Q, [&](auto q) {
-      constexpr int QQ = decltype(q)::value;
-      const unsigned g = blocks_for(a.ng, kGfcBlock<S>);
-      if (a.mom2) k_fill_gfc<QQ, S, true><<<g, kGfcBlock<S>, 0, st>>>(a);
-      else k_fill_gfc<QQ, S, false><<<g, kGfcBlock<S>, 0, st>>>(a);
+      if (two) launch(k_fill_gfc<decltype(q)::value, S, true>, g, kGfcBlock<S>, st, a);
+      else launch(k_fill_gfc<decltype(q)::value, S, false>, g, kGfcBlock<S>, st, a);
     });
   }
-  static void fill_gff(int Q, const GffArgs& a, cudaStream_t st) {
-    if (a.ng <= 0) return;
+  static void fill_gff(int Q, GffArgs& a, cudaStream_t st) {
     with_q(Q, [&](auto q) {
       constexpr int QQ = decltype(q)::value;
-      const unsigned g = blocks_for(a.ng * (1 << Lat<QQ>::D), kGffBlock<S>);
-      if (a.force) k_fill_gff<QQ, S, true><<<g, kGffBlock<S>, 0, st>>>(a);
-      else k_fill_gff<QQ, S, false><<<g, kGffBlock<S>, 0, st>>>(a);
+      const unsigned g =
+          assign_blocks(a, kGffBlock<S>, [&](int k) { return (int64_t)a.lev[k].ng << Lat<QQ>::D; });
+      if (!g) return;
+      if (a.force) launch(k_fill_gff<QQ, S, true>, g, kGffBlock<S>, st, a);
+      else launch(k_fill_gff<QQ, S, false>, g, kGffBlock<S>, st, a);
     });
   }
   static void fill_rest(int Q, const FillArgs& a, cudaStream_t st) {
@@ -1788,17 +1913,13 @@ struct Launch {
 
 template <class S>
 const Ops* make_ops() {
-  static const Ops ops = {&Launch<S>::stream_collide, &Launch<S>::stream_collide_brick,
+  static const Ops ops = {&Launch<S>::sc_interior,    &Launch<S>::sc_rest,
                           &Launch<S>::outlet,         &Launch<S>::source_moments,
                           &Launch<S>::fill_gfc,       &Launch<S>::fill_gff,   &Launch<S>::fill_rest,
                           &Launch<S>::init,           &Launch<S>::init_place, &Launch<S>::out,
                           &Launch<S>::set_state,
                           &Launch<S>::gather_ghosts,
-                          &Launch<S>::reduce,         sizeof(S),              sizeof(typename Sto<S>::R),
-                          // every storage type streams its boundary bricks through the
-                          // brick tables (BF16: 2.85 against 5.50 ms per sphere step
-                          // through the neighbour list, measured)
-                          true};
+                          &Launch<S>::reduce,         sizeof(S),              sizeof(typename Sto<S>::R)};
   return &ops;
 }
 

@@ -13,6 +13,17 @@
 namespace lbm {
 // Ops of the recursive level step, in the order lbm_ctx::advance issues them.
 enum StepOp { OP_GFF = 0, OP_MOM_A = 1, OP_GFC_A = 2, OP_SC = 3, OP_MOM_B = 4, OP_GFC_B = 5 };
+// Instants that advance at most this many fluid elements launch their kernels
+// as programmatic dependents of one another (let_next_start in kernels.cuh).
+// Below it the step is a chain of latencies and hiding a launch pays; beyond
+// it the waiting blocks take slots that the interior bricks' kernel, beside
+// the chain, could use.  Measured per coarse step, chained / not: four-level
+// D2Q9 cylinder (6e4 elements) 56 / 67 us, two-level D3Q27 (9e5) 131 / 139 us,
+// four-level BF16 sphere (3.6e6) 866 / 857 us.  FP64: a kernel takes as long
+// as the SM with the most of its one-warp blocks, and dependents start where
+// slots happen to be free, not evenly: 1,800 elements 43.5 / 46.5 us, but
+// 4.6e4 elements 60 / 40 us; the line is where every SM has about one warp.
+constexpr int64_t kChainElements = 1 << 20, kChainElements64 = 1 << 12;
 // Kernel kinds of the per-launch timing (lbm_timing_read row kTimedKinds * L + kind)
 enum TimedKind { TK_INTERIOR = 0, TK_LIST = 1, TK_BOUNDARY = 2, TK_GFF = 3, TK_MOM = 4, TK_GFC = 5, TK_OUTLET = 6,
                  TK_SC_SPAN = 7 };
@@ -134,17 +145,14 @@ struct lbm_ctx {
   };
   std::vector<StepGraph> graphs;
   cudaStream_t cap_stream = nullptr;
-  // branch streams and fork/join events of the captured graphs, per level:
-  // the level's stream-collide runs on branch `sc` (forked after its
-  // GhostFromFiner, joined before the ops that read its result), and its three
-  // kernels (disjoint elements, same source buffer) on `sc` and the two `side`
-  // streams
-  struct LevelStreams {
-    cudaStream_t sc = nullptr, side[2] = {nullptr, nullptr};
-    cudaEvent_t fork_sc = nullptr, done_sc = nullptr, fork = nullptr, join[2] = {nullptr, nullptr};
-  };
-  std::vector<LevelStreams> lvs;
-  bool make_level_streams();
+  // branch streams and fork/join events of the captured graphs: [0] the
+  // interior bricks, [1] the boundary values
+  struct Branches {
+    cudaStream_t s[2] = {nullptr, nullptr};
+    cudaEvent_t fork[2] = {nullptr, nullptr}, join[2] = {nullptr, nullptr};
+    bool ok = false;
+  } br;
+  bool make_branches();
   // copy stream of lbm_init's double-buffered host uploads: copy_ev[0..1]
   // mark each staging half free again, [2] the bound stream's earlier work,
   // [3] a half-chunk's copies done (made on first use; false if unavailable)
@@ -167,24 +175,6 @@ struct lbm_ctx {
     }
     return copy_st != nullptr;
   }
-#ifndef LBM_CONCURRENT_SC
-#define LBM_CONCURRENT_SC 1
-#endif
-  bool concurrent_sc = LBM_CONCURRENT_SC != 0;
-  // the finer level's GhostFromCoarser fill at t + 1/2 on the coarse level's
-  // stream-collide branch, beside the finer level's first substep (off:
-  // measured 35.5 against 32.8 ms per sphere step, the finest stream-collide
-  // slowed by its neighbour)
-#ifndef LBM_GFC_B_BRANCH
-#define LBM_GFC_B_BRANCH 0
-#endif
-  bool gfc_b_branch = LBM_GFC_B_BRANCH != 0;
-  // a level's stream-collide as a graph branch of its own (on: 33.06 against
-  // 33.14 ms per sphere step with the level's three kernels forked either way)
-#ifndef LBM_LEVEL_BRANCH
-#define LBM_LEVEL_BRANCH 1
-#endif
-  bool level_branch = LBM_LEVEL_BRANCH != 0;
   bool graphs_on = true;
   int last_graph = -1;        // graph of the most recent replay
   bool graph_unread = false;  // its events hold a replay not yet read
@@ -208,10 +198,9 @@ struct lbm_ctx {
     if (copy_st) cudaStreamDestroy(copy_st);
     for (cudaEvent_t e : copy_ev)
       if (e) cudaEventDestroy(e);
-    for (auto& L : lvs) {
-      for (cudaStream_t s : {L.sc, L.side[0], L.side[1]})
-        if (s) cudaStreamDestroy(s);
-      for (cudaEvent_t e : {L.fork_sc, L.done_sc, L.fork, L.join[0], L.join[1]})
+    for (int b = 0; b < 2; ++b) {
+      if (br.s[b]) cudaStreamDestroy(br.s[b]);
+      for (cudaEvent_t e : {br.fork[b], br.join[b]})
         if (e) cudaEventDestroy(e);
     }
   }
@@ -241,21 +230,37 @@ struct lbm_ctx {
   lbm_status launched(const char* where) { return cuda_check(cudaGetLastError(), where); }
 
   void layout();
-  // driver pieces
+  // driver pieces: launch arguments of a level's part of an op, added to
+  // those of the levels that share the launch
+  lbm::GffArgs gff_args() const;
+  void add_gff(lbm::GffArgs& a, int li) const;
+  lbm::GfcArgs gfc_args() const;
+  // two_times: the fill at t + 1/2; all_layers false: in LINEAR mode the outer
+  // ghost layer, which no stream-collide reads, is left unwritten
+  void add_gfc(lbm::GfcArgs& a, int li_fine, bool two_times, bool all_layers) const;
+  lbm::OutletArgs outlet_args(const void* side) const;
+  void add_outlet(lbm::OutletArgs& o, int li, const void* src) const;
+  lbm::ScArgs sc_args() const;
+  // elements of one kind (TK_INTERIOR, TK_BOUNDARY, TK_LIST) of level li as a
+  // segment, the level in slot `slot`; returns 1 if there are any, else 0
+  int add_sc(lbm::ScArgs& a, int slot, int li, int kind) const;
+  lbm::SourceTable source_table() const;
+  template <class Args>
+  void ghost_units(Args& a, bool to_coarse) const;
+  // ops of one level, on the bound stream
   void fill_gff(int li);
-  // records of the level's sources into mom_off: subset SRC_ALL every
-  // source, SRC_GFF the GhostFromFiner ones, SRC_GFF_OUTER those of the outer
-  // GhostFromFiner layer
-  void source_moments(int li, size_t mom_off, size_t prev_off = 0, cudaStream_t s = nullptr, int subset = 0);
-  enum { SRC_ALL = 0, SRC_GFF = 1, SRC_GFF_OUTER = 2 };
-  // all_layers false: in LINEAR mode the outer ghost layer, which no
-  // stream-collide reads, is left unwritten
-  // next_buffer: write the ghosts into the fine level's other buffer (the
-  // one its next stream-collide writes, issued before that stream-collide)
-  void fill_gfc(int li_fine, bool two_times, bool all_layers = false, cudaStream_t s = nullptr,
-                bool next_buffer = false);
-  // launches on stream s (default: the bound stream)
-  void stream_collide(int li, cudaStream_t s = nullptr);
+  // records of the level's sources into mom_off: subset SRC_ALL every source,
+  // SRC_GFF_OUTER the ghosts of the outer GhostFromFiner layer
+  void source_moments(int li, size_t mom_off, cudaStream_t s = nullptr, int subset = 0);
+  enum { SRC_ALL = 0, SRC_GFF_OUTER = 1 };
+  void fill_gfc(int li_fine, bool two_times, bool all_layers);
+  void stream_collide(int li);
+  // one coarse step in a graph capture, the levels batched by instant
+  void step_batched();
+  void tick_batched(int l0, int n);
+  int n_filled = 1;                  // levels up to the finest one with elements
+  bool outlet_reads_ghosts = false;  // a boundary value reads a ghost's pdfs
+  // one coarse step, level by level
   void advance(int li);
   // one coarse step from the top: ensure_records(), then advance(0)
   void coarse_step() {

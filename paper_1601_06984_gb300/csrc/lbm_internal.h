@@ -6,11 +6,18 @@
 
 #include <climits>
 #include <cmath>
+#include <cstddef>
 #include <cstdint>
 #include <string>
 #include <vector>
 
 #include "lbm.h"
+
+#ifdef __CUDACC__
+#define LBM_HD __host__ __device__ __forceinline__
+#else
+#define LBM_HD inline
+#endif
 
 namespace lbm {
 
@@ -76,38 +83,57 @@ inline double odd_fneq_ratio(int mode, bool to_coarse) {
 // the same flow's lattice velocity on level index li over that on the coarsest level
 inline double level_velocity_ratio(int li, int mode) { return mode == LBM_TIME_DIFFUSIVE ? std::ldexp(1.0, -li) : 1.0; }
 
-// Relaxation constants of a level for the FP64 kernels, whose pipe is GB300's
-// narrowest unit (1.7 multiply-adds per clock and SM): every factor that is
-// the same for all elements is formed here once, and the kernels read it as a
-// constant operand.  Arrays are indexed by |c_i|^2.
-struct Relax {
-  double omega;
-  double keep;                     // 1 - omega
-  double eq[4], quad[4], lin[4];   // omega w {1, 9/2, 3}
-  double force[4];                 // 3 w (1 - omega / 2)
-  double r1w;                      // 1 / (1 - omega)
-  double neq[4], nquad[4], nlin[4], nforce[4];  // w {1, 9/2, 3}, 3 w (1 - omega / 2), each times r1w
-  double strain;                   // -3 omega / 2
+// Relaxation constants of a level.  The FP32 kernels read omega and
+// r1w = 1 / (1 - omega) as floats (a conversion in the kernel would be an
+// instruction on the FP64 pipe in every thread); for the FP64 kernels every
+// factor that is the same for all elements is formed here once.  Indexed by
+// the weight class |c_i|^2; laid out in 64-byte lines by use (see LaunchArgs).
+struct Relax32 {
+  float omega, r1w;
 };
+struct alignas(64) Relax {
+  // collision, classes 0..2
+  double keep;                              // 1 - omega
+  double eq_[3], quad_[2], lin_[2];         // omega w {1, 9/2, 3}
+  // class 3 (D3Q27 corners), Guo forcing 3 w (1 - omega / 2), -3 omega / 2
+  double eq3, quad3, lin3, force[4], strain;
+  // f^neq from the stored state, classes 0..2: the same factors over omega times r1w
+  double r1w;
+  double neq_[3], nquad_[2], nlin_[2];
+  double neq3, nquad3, nlin3, nforce[4], omega;
+  LBM_HD double eq(int c) const { return c < 3 ? eq_[c] : eq3; }
+  LBM_HD double quad(int c) const { return c < 3 ? quad_[c - 1] : quad3; }  // c >= 1
+  LBM_HD double lin(int c) const { return c < 3 ? lin_[c - 1] : lin3; }
+  LBM_HD double neq(int c) const { return c < 3 ? neq_[c] : neq3; }
+  LBM_HD double nquad(int c) const { return c < 3 ? nquad_[c - 1] : nquad3; }
+  LBM_HD double nlin(int c) const { return c < 3 ? nlin_[c - 1] : nlin3; }
+};
+static_assert(sizeof(Relax) == 256, "four lines");
+inline Relax32 make_relax32(double omega) {
+  const float w = (float)omega;
+  return {w, 1.0f / (1.0f - w)};
+}
 inline Relax make_relax(int Q, double omega) {
   int c[kQmax][3];
-  double w[kQmax];
+  double w[kQmax], wc[4] = {0, 0, 0, 0};
   host_lattice(Q, c, w);
+  for (int i = 0; i < Q; ++i) wc[c[i][0] * c[i][0] + c[i][1] * c[i][1] + c[i][2] * c[i][2]] = w[i];
   Relax r{};
   r.omega = omega;
   r.keep = 1.0 - omega;
   r.r1w = 1.0 / (1.0 - omega);
   r.strain = -1.5 * omega;
-  for (int i = 0; i < Q; ++i) {
-    const int n = c[i][0] * c[i][0] + c[i][1] * c[i][1] + c[i][2] * c[i][2];
-    r.eq[n] = omega * w[i];
-    r.quad[n] = 4.5 * r.eq[n];
-    r.lin[n] = 3.0 * r.eq[n];
-    r.force[n] = 3.0 * w[i] * (1.0 - 0.5 * omega);
-    r.neq[n] = w[i] * r.r1w;
-    r.nquad[n] = 4.5 * r.neq[n];
-    r.nlin[n] = 3.0 * r.neq[n];
+  for (int n = 0; n < 4; ++n) {
+    r.force[n] = 3.0 * wc[n] * (1.0 - 0.5 * omega);
     r.nforce[n] = r.force[n] * r.r1w;
+    const double e = omega * wc[n], q = wc[n] * r.r1w;
+    (n < 3 ? r.eq_[n] : r.eq3) = e;
+    (n < 3 ? r.neq_[n] : r.neq3) = q;
+    if (n == 0) continue;
+    (n < 3 ? r.quad_[n - 1] : r.quad3) = 4.5 * e;
+    (n < 3 ? r.lin_[n - 1] : r.lin3) = 3.0 * e;
+    (n < 3 ? r.nquad_[n - 1] : r.nquad3) = 4.5 * q;
+    (n < 3 ? r.nlin_[n - 1] : r.nlin3) = 3.0 * q;
   }
   return r;
 }
@@ -193,61 +219,80 @@ lbm_status sfc_partition(const int64_t* tree_ids, int64_t n, int d, int nparts, 
 // ----------------------------------------------------------------- kernels
 // Launch arguments are plain data; pointers are device pointers into the
 // workspace.  "src"/"dst" are pdf arrays [Q][Ntot] of the storage type.
-// GFC source records written by a stream-collide (interpolation step 1 of
-// Sec. 2.2 fused into the kernel that produces the source state): for every
-// processed element marked in mask, the record of its new state goes to
-// rec_out.  mask null: no records.
-struct SourceOut {
+// LaunchArgs: what a launch reads from its parameters is cold on every SM
+// (about 0.3 us per 64-byte line, one after the other), which is as much as a
+// small level's work.  So the structs below hold together, in as few aligned
+// lines as possible, what a block reads: a header with the first block of
+// every segment, the shared pointers, and one line per segment.  (Spread over
+// nine lines, more with the FP64 constants, the kernels of small levels took
+// 1 to 4 us longer.)
+//
+// A launch takes elements of several levels: every level that advances at one
+// instant of the step (at most kMaxBatch), in segments of whole blocks.
+constexpr int kMaxBatch = 6;
+constexpr int kMaxSeg = 2 * kMaxBatch;
+
+// GFC source records (interpolation step 1 of Sec. 2.2) are written by the
+// kernel that produces the source state: for every element marked in mask the
+// record of its new state goes to its level's rec_out (null: none).
+struct SourceTable {
   const uint32_t* mask;  // [Ntot / 32] source bits per 32 slots
   const int32_t* first;  // [Ntot / 32] record index of each block's first source
-  void* rec_out;         // [nsrc][mom_stride(Q)] records of the new state
-};
-struct StreamCollideArgs {
-  const void* src;
-  void* dst;
-  const uint32_t* nbr;
-  const void* force;  // [d][Ntot] compute type, or null
-  const void* side;   // boundary values, compute type, or null
-  const double* inlet_s;  // inlet profile factor per inlet link
-  int64_t Ntot, begin, end;  // linear range; element = lin + (lin >= hole_at ? hole_len : 0)
-  int64_t hole_at, hole_len;  // interior bricks skipped by this kernel (0 length: none)
-  Relax rx;
-  double rho_off;
-  double inlet[kQmax];  // 6 w_i rho0 (c_i . u_in)
-  SourceOut so;
 };
 
-// Stream-collide of the interior bricks of one level: nB bricks of 64
-// elements from global index begin; neighbour bricks and link table as in
-// HostMesh::brick_nb / brick_tab.
-struct BrickArgs {
+// Stream-collide segment: a run of bricks of 64 elements (interior or
+// boundary; nb their rows as in HostMesh::brick_nb) or, in the launch of the
+// boundary bricks, a linear range of the elements that go through the
+// neighbour list (element = lin + (lin >= hole_at ? hole_len : 0), stepping
+// over the bricks).
+struct alignas(64) ScSeg {
   const void* src;
   void* dst;
+  const int32_t* nb;
+  void* rec_out;            // [nsrc][mom_stride(Q)] records of the new state, or null
+  int32_t n;                // bricks, or elements of the list range
+  int32_t begin;            // first element of the bricks, or first linear position
+  int32_t hole_at, hole_len;
+  Relax32 rx;
+  float uin;                // the inlet velocity's factor to this level's lattice units
+  int16_t level, list;      // index of the level's Relax; neighbour-list range instead of bricks
+};
+struct alignas(64) ScArgs {
+  uint32_t first[kMaxSeg];  // first block of each segment (set by the launcher)
+  int nseg;
+  float rho_off32;
+  double rho_off;
   const void* force;    // [d][Ntot] compute type, or null
-  const int32_t* nb;    // [nB][27] rows (offsets from the brick's first element, or kBrickMissing)
-  const uint16_t* tab;  // [Q-1][64]
-  int64_t Ntot, begin, nB;
-  Relax rx;
-  double rho_off;
-  // boundary bricks: links through a missing neighbour brick use the element's
-  // neighbour-list code (pull, bounce-back, inlet, boundary value)
+  const uint16_t* tab;  // [Q-1][64] link table
   const uint32_t* nbr;
-  const void* side;
-  const double* inlet_s;
-  double inlet[kQmax];
-  SourceOut so;
+  const void* side;     // boundary values, compute type
+  const double* inlet_s;  // inlet profile factor per inlet link
+  SourceTable sources;
+  int64_t Ntot;
+  ScSeg seg[kMaxSeg];
+  Relax rx[kMaxBatch];  // FP64 kernels
+  double inlet[kQmax];  // 6 w_i rho0 (c_i . u_in), coarsest level's units
+  int chain;            // host: launch as a programmatic dependent
 };
+static_assert(sizeof(ScSeg) == 64 && offsetof(ScArgs, seg) == 128, "lines");
 
-struct OutletArgs {
+struct OutletLevel {
   const void* src;
+  int64_t end;  // end of the level's links
+  double omega;
+};
+struct OutletArgs {  // links begin .. end of the last level, levels in order
+  OutletLevel lev[kMaxBatch];
+  int nlev;
+  int zero_gradient;  // extrapolate with f(x - n) instead of 2 f(x - n) - f(x - 2n)
   void* side;
   const int32_t *elem, *a, *b;
   const int8_t *dir, *kind;
   const void* force;
-  int64_t Ntot, begin, end;
-  double omega, rho_off, rho0;
-  int zero_gradient;  // extrapolate with f(x - n) instead of 2 f(x - n) - f(x - 2n)
+  int64_t Ntot, begin;
+  double rho_off, rho0;
   const double* q;    // wall distance of interpolated bounce-back links
+  int chain;          // host: launch as a programmatic dependent
 };
 
 // GFC source moments: one record of mom_stride(Q) values per source (compute
@@ -262,44 +307,70 @@ struct MomentsArgs {
   const void* prev;  // if set: mom = (prev + moments now) / 2 (mean of two time levels)
   const int32_t* rec;  // record index of elem[k] (null: k)
   int64_t Ntot, nsrc;
-  Relax rx;
   double rho_off;
+  float rho_off32;
+  Relax32 rx32;
+  Relax rx;
 };
 
-struct GfcArgs {
+// Unit conversion between two levels (to the ghost's): velocity times
+// u_scale, density deviation rho' := r_scale rho' + r_shift (relative to
+// rho_off), dt_c / dt_f = tratio; odd: the extra factor of f^neq's odd part
+// (odd_fneq_ratio), applied where it is not 1.
+template <class R>
+struct GhostUnits {
+  R rho_off, tratio, u_scale, r_scale, r_shift, odd;
+};
+struct alignas(64) GfcLevel {
   const void* mom;       // [nsrc][mom_stride(Q)] source records
   const void* mom2;      // if set: the records are the means of mom and mom2 (t + 1/2)
-  int64_t nsrc;
   const int32_t* gsrc;   // [4][ng]
   const uint8_t* oct;    // [ng]
-  int64_t ng, dest0;     // global index of the first GFC
   void* dst;
-  int64_t Ntot;
-  double omega_c, omega_f, rho_off;
-  double scale;          // (1 - omega_f) omega_c / (tratio omega_f) (FP64 kernels)
-  int skip_outer;        // leave the outer-layer ghosts (oct & kGfcOuter) unwritten
-  // unit conversion coarse -> fine: dt_c / dt_f, u_f = u_scale u_c and the
-  // density deviation rho'_f = r_scale rho'_c + r_shift (relative to rho_off);
-  // odd_ratio: the extra factor of f^neq's odd part (odd_fneq_ratio)
-  double tratio, u_scale, r_scale, r_shift, odd_ratio;
+  int32_t ng, dest0;     // global index of the first GFC
+  int32_t skip_outer;    // leave the outer-layer ghosts (oct & kGfcOuter) unwritten
+  float scale32;         // (1 - omega_f) omega_c / (tratio omega_f)
+  double scale;
 };
+struct alignas(64) GfcArgs {
+  uint32_t first[kMaxBatch];  // first block of each level (set by the launcher)
+  int nseg;
+  int odd_rescale;
+  int64_t Ntot;
+  GhostUnits<float> u32;
+  GfcLevel lev[kMaxBatch];
+  GhostUnits<double> u64;
+  int chain;  // host: launch as a programmatic dependent
+};
+static_assert(sizeof(GfcLevel) == 64 && offsetof(GfcArgs, lev) == 64, "lines");
 
-struct GffArgs {
+struct alignas(64) GffLevel {
   const void* src_fine;  // pdfs holding the children
-  const void* force;
   const int32_t* child0; // [ng], inner layer first
-  int64_t ng, n_inner;   // ghosts k < n_inner go to dest0 + k, the rest to dest_outer + (k - n_inner)
-  int64_t dest0, dest_outer;
   void* dst;             // pdfs holding the coarse ghosts
-  int64_t Ntot;
-  Relax rx_f;            // of the children's level
-  double omega_c, rho_off;
-  double scale;          // factor of the children's f^neq sum in the stored ghost (FP64 kernels)
-  // unit conversion fine -> coarse: dt_c / dt_f, u_c = u_scale u_f and the
-  // density deviation rho'_c = r_scale rho'_f + r_shift (relative to rho_off);
-  // odd_ratio: the extra factor of f^neq's odd part (odd_fneq_ratio)
-  double tratio, u_scale, r_scale, r_shift, odd_ratio;
+  void* rec_out;         // records of the ghosts that are GFC sources, or null
+  int32_t ng, n_inner;   // ghosts k < n_inner go to dest0 + k, the rest to dest_outer + (k - n_inner)
+  int32_t dest0, dest_outer;
+  Relax32 rx_f;          // of the children's level
+  float scale32;         // (1 - omega_c) tratio omega_f / omega_c / 2^d
+  int32_t pad;
 };
+struct alignas(64) GffArgs {
+  uint32_t first[kMaxBatch];  // first block of each level (set by the launcher)
+  int nseg;
+  int odd_rescale;
+  int64_t Ntot;
+  GhostUnits<float> u32;
+  const void* force;
+  SourceTable sources;
+  GhostUnits<double> u64;
+  GffLevel lev[kMaxBatch];
+  Relax rx_c64[kMaxBatch], rx_f64[kMaxBatch];  // FP64 kernels
+  Relax32 rx_c[kMaxBatch];       // the ghosts' levels (records)
+  double scale[kMaxBatch];
+  int chain;  // host: launch as a programmatic dependent
+};
+static_assert(sizeof(GffLevel) == 64 && offsetof(GffArgs, force) == 64, "lines");
 
 struct FillArgs {  // rest equilibrium everywhere
   void* pdf;
@@ -388,12 +459,14 @@ struct FinalArgs {
 };
 
 struct Ops {
-  void (*stream_collide)(int Q, bool force, const StreamCollideArgs&, cudaStream_t);
-  void (*stream_collide_brick)(int Q, bool force, bool boundary, const BrickArgs&, cudaStream_t);
+  // interior bricks of the segments' levels (record epilogue where a level has sources)
+  void (*sc_interior)(int Q, bool force, ScArgs&, cudaStream_t);
+  // boundary bricks and neighbour-list elements
+  void (*sc_rest)(int Q, bool force, ScArgs&, cudaStream_t);
   void (*outlet)(int Q, const OutletArgs&, cudaStream_t);
   void (*source_moments)(int Q, const MomentsArgs&, cudaStream_t);
-  void (*fill_gfc)(int Q, const GfcArgs&, cudaStream_t);
-  void (*fill_gff)(int Q, const GffArgs&, cudaStream_t);
+  void (*fill_gfc)(int Q, GfcArgs&, cudaStream_t);
+  void (*fill_gff)(int Q, GffArgs&, cudaStream_t);
   void (*fill_rest)(int Q, const FillArgs&, cudaStream_t);
   void (*init)(int Q, const InitArgs&, cudaStream_t);
   void (*init_place)(int Q, const PlaceArgs&, cudaStream_t);
@@ -403,7 +476,6 @@ struct Ops {
   void (*reduce)(int Q, const ReduceArgs&, cudaStream_t);
   size_t storage_bytes;  // bytes per stored pdf
   size_t compute_bytes;  // bytes of the compute type
-  bool boundary_bricks;  // stream boundary bricks with the brick kernel (else with the neighbour list)
 };
 
 // ----------------------------------------------------------------- adjoint kernels
