@@ -325,10 +325,10 @@ void lbm_ctx::stream_collide(int li) {
 // small levels share a launch (cylinder 109 -> 67 us a coarse step, 56 us
 // with the launches chained; sphere of 1.1e7 elements 5.08 -> 4.94 ms).
 // Every op has the inputs it has in advance(): same results bit for bit.
-// Starting the interior bricks, which read no ghost, beside the ghost fills
-// slowed both (two-level 64^3, FP32: 50 against 48 us; FP64 D2Q9: 84 against
-// 40 us), and taking them into the other stream-collide launch cost more than
-// the fork it saves (49 against 48 us).
+// Starting the interior bricks, which read no ghost, beside the GhostFromFiner
+// fill slowed both (two-level 64^3, FP32: 50 against 48 us; FP64 D2Q9: 84
+// against 40 us), and taking them into the other stream-collide launch cost
+// more than the fork it saves (49 against 48 us).
 void lbm_ctx::step_batched() {
   const int n = n_filled, r = time_ratio(p.time_mode);
   int64_t T = 1;
@@ -367,20 +367,21 @@ void lbm_ctx::tick_batched(int l0, int n) {
   }
   const bool chain = elements <= (p.precision == LBM_FP64 ? kChainElements64 : kChainElements);
   rest.chain = chain;
-  auto run_interior = [&] {
-    fork(0);
-    // BF16 streams the finest level two elements per thread, which has no
-    // record epilogue, so that level goes apart from the coarser ones
-    ScArgs a = in;
-    if (p.precision == LBM_BF16DEV && in.nseg > 1 && !in.seg[in.nseg - 1].rec_out) {
-      a.nseg = 1;
-      a.seg[0] = in.seg[in.nseg - 1];
-      ScArgs b = in;
-      --b.nseg;
-      ops->sc_interior(Q, p.use_force != 0, b, br.s[0]);
-    }
-    timed_launch(timed_level, TK_INTERIOR, [&] { ops->sc_interior(Q, p.use_force != 0, a, br.s[0]); }, br.s[0]);
-  };
+  const bool force = p.use_force != 0;
+  // Interior bricks read no ghost.  At small instants they all run beside the
+  // GhostFromCoarser fill; beyond kBesideElements the finest level's, which
+  // fill the GPU by themselves, only after it, apart from the coarser ones'
+  // (and so with BF16 storage, whose two-element kernel has no record
+  // epilogue).
+  const bool beside = elements <= kBesideElements;
+  ScArgs fin = in;
+  int coarse_segs = 0;
+  if (in.nseg > 1 && !in.seg[in.nseg - 1].rec_out && (!beside || p.precision == LBM_BF16DEV)) {
+    coarse_segs = in.nseg - 1;
+    fin.nseg = 1;
+    fin.seg[0] = in.seg[in.nseg - 1];
+    in.nseg = coarse_segs;
+  }
   auto run_outlet = [&](cudaStream_t s) { ops->outlet(Q, out, s); };
   const bool out_branch = out.nlev && !outlet_reads_ghosts;
   if (out_branch) {
@@ -395,6 +396,21 @@ void lbm_ctx::tick_batched(int l0, int n) {
     if (gff.nseg > k) launches += 1 + (gff.lev[k].rec_out != nullptr);
   }
   if (gff.nseg) ops->fill_gff(Q, gff, st);
+  // Interior bricks beside the GhostFromCoarser fill: queued before it (the
+  // other way round, blocks of the bricks start on SMs set up for the fill's
+  // shared memory, with little L1: sphere 6.26 against 4.94 ms a step), but
+  // after it in FP64, where one-warp blocks of the bricks would fill the slots
+  // the fill needs (D2Q9 channel 52 against 40 us)
+  const bool early = fin.nseg && (beside || coarse_segs);
+  auto run_early = [&] {
+    if (coarse_segs) ops->sc_interior(Q, force, in, br.s[0]);
+    if (beside) timed_launch(timed_level, TK_INTERIOR, [&] { ops->sc_interior(Q, force, fin, br.s[0]); }, br.s[0]);
+  };
+  const bool fill_first = p.precision == LBM_FP64;
+  if (early) {
+    fork(0);
+    if (!fill_first) run_early();
+  }
   GfcArgs gfc = gfc_args();
   gfc.chain = chain;
   if (p.time_mode == LBM_TIME_LINEAR && l0 > 0) {
@@ -404,13 +420,16 @@ void lbm_ctx::tick_batched(int l0, int n) {
   for (int l = l0 + 1; l < n; ++l) add_gfc(gfc, l, false, false);
   launches += gfc.nseg;
   if (gfc.nseg) ops->fill_gfc(Q, gfc, st);
+  if (early && fill_first) run_early();
   if (out.nlev && !out_branch) run_outlet(st);
   if (out_branch) join(1);
   timed_launch(timed_level, TK_SC_SPAN, [&] {
-    if (in.nseg) run_interior();
-    if (rest.nseg)
-      timed_launch(timed_level, TK_BOUNDARY, [&] { ops->sc_rest(Q, p.use_force != 0, rest, st); });
-    if (in.nseg) join(0);
+    if (fin.nseg && !beside) {
+      fork(0);
+      timed_launch(timed_level, TK_INTERIOR, [&] { ops->sc_interior(Q, force, fin, br.s[0]); }, br.s[0]);
+    }
+    if (rest.nseg) timed_launch(timed_level, TK_BOUNDARY, [&] { ops->sc_rest(Q, force, rest, st); });
+    if (fin.nseg) join(0);
   });
   for (int l = l0; l < n; ++l) parity[l] ^= 1;
 }

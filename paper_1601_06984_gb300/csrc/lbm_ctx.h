@@ -24,6 +24,11 @@ enum StepOp { OP_GFF = 0, OP_MOM_A = 1, OP_GFC_A = 2, OP_SC = 3, OP_MOM_B = 4, O
 // slots happen to be free, not evenly: 1,800 elements 43.5 / 46.5 us, but
 // 4.6e4 elements 60 / 40 us; the line is where every SM has about one warp.
 constexpr int64_t kChainElements = 1 << 20, kChainElements64 = 1 << 12;
+// Instants of at most this many elements run all interior bricks beside the
+// GhostFromCoarser fill (us per coarse step, beside / after: cylinder 54.5 /
+// 57.3, two-level 64^3 44.9 / 45.7, D3Q27 9e5 elements 131 / 132; beyond it the
+// sphere of 1.1e7 elements took 7.4 against 4.94 ms).
+constexpr int64_t kBesideElements = 1 << 20;
 // Kernel kinds of the per-launch timing (lbm_timing_read row kTimedKinds * L + kind)
 enum TimedKind { TK_INTERIOR = 0, TK_LIST = 1, TK_BOUNDARY = 2, TK_GFF = 3, TK_MOM = 4, TK_GFC = 5, TK_OUTLET = 6,
                  TK_SC_SPAN = 7 };
