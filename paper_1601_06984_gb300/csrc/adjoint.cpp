@@ -16,12 +16,6 @@
 #include <vector>
 
 #include "lbm_ctx.h"
-
-// run the brick and neighbour-list reverse stream-collide of a level
-// concurrently (disjoint elements and scatter targets, rows of their own)
-#ifndef LBM_ADJ_CONCURRENT
-#define LBM_ADJ_CONCURRENT 1
-#endif
 #include "lbm_internal.h"
 
 using namespace lbm;
@@ -41,7 +35,7 @@ struct TapeOp {
 
 struct AdjLayout {
   size_t lamA = 0, lamB = 0, lamF = 0, side_fwd = 0, lam_side = 0, partial = 0, acc = 0, contrib = 0;
-  std::vector<size_t> lam_recA, lam_recB, recA, recB, csr_off, csr_item;
+  std::vector<size_t> lam_rec, recA, recB, csr_off, csr_item;
   size_t ck = 0, steps = 0, snaps = 0, ends = 0, fin = 0;
   int n_ck = 0, n_steps = 0, n_snaps = 0;
   // tape_all: a segment's recompute records every step's tape (two forward
@@ -198,6 +192,12 @@ int count_snapshots(lbm_ctx* c) {
   return per_level.empty() ? 0 : *std::max_element(per_level.begin(), per_level.end());
 }
 
+const AdjOps* adj_ops_for(int precision) {
+  if (precision == LBM_FP64) return adj_ops_fp64();
+  if (precision == LBM_FP32DEV) return adj_ops_fp32dev();
+  return adj_ops_bf16dev();
+}
+
 AdjLayout adj_layout(lbm_ctx* c, int64_t n, int K) {
   AdjLayout L;
   size_t o = 0;
@@ -213,21 +213,24 @@ AdjLayout adj_layout(lbm_ctx* c, int64_t n, int K) {
   L.lamF = take((size_t)c->d * N * 8);
   L.side_fwd = take(c->M.out_elem.size() * lb);
   L.lam_side = take(c->M.out_elem.size() * lb);
-  L.partial_rows = kAdjBlocks;
-  for (int li = 0; li < c->nlev; ++li)
-    L.partial_rows = std::max<int>(L.partial_rows, (int)((c->M.lv[li].nB + LBM_BRICKS_PER_BLOCK - 1) / LBM_BRICKS_PER_BLOCK));
-  // the neighbour-list reverse runs concurrently with the brick reverse, so
-  // its blocks add to rows of their own
-  L.side_row0 = LBM_ADJ_CONCURRENT ? L.partial_rows : 0;
-  if (LBM_ADJ_CONCURRENT) L.partial_rows += kAdjBlocks;
+  const int64_t block = adj_ops_for(c->p.precision)->sc_block;
+  int64_t interior = kAdjBlocks, rest = 0;
+  for (int li = 0; li < c->nlev; ++li) {
+    const HostLevel& H = c->M.lv[li];
+    interior = std::max(interior, (64 * H.nB + block - 1) / block);
+    rest = std::max(rest, (64 * H.nBb + block - 1) / block + (H.N - 64 * (H.nB + H.nBb)) / block + 2);
+  }
+  // the rest of the reverse stream-collide runs beside the interior bricks',
+  // so its blocks add to rows of their own
+  L.side_row0 = (int)interior;
+  L.partial_rows = (int)(interior + rest);
   L.partial = take((size_t)L.partial_rows * kAccCols * 8);
   L.acc = take(32 * 8);
   int64_t max_contrib = 0;
   for (int li = 0; li < c->nlev; ++li) {
     const HostLevel& H = c->M.lv[li];
     const int64_t nsrc = (int64_t)H.src_elem.size();
-    L.lam_recA.push_back(take((size_t)nsrc * mom_stride(c->Q) * lb));
-    L.lam_recB.push_back(take((size_t)nsrc * mom_stride(c->Q) * lb));
+    L.lam_rec.push_back(take((size_t)nsrc * mom_stride(c->Q) * lb));
     L.recA.push_back(take((size_t)nsrc * mom_stride(c->Q) * lb));
     L.recB.push_back(take((size_t)nsrc * mom_stride(c->Q) * lb));
     L.csr_off.push_back(take((size_t)(nsrc + 1) * 4));
@@ -235,7 +238,7 @@ AdjLayout adj_layout(lbm_ctx* c, int64_t n, int K) {
     L.csr_item.push_back(take((size_t)4 * nfine * 4));
     max_contrib = std::max(max_contrib, nfine);
   }
-  L.contrib = take((size_t)max_contrib * 4 * mom_stride(c->Q) * lb);
+  L.contrib = take((size_t)max_contrib * ((c->Q + 3) / 4 * 4 + 4) * lb);
   L.state_bytes = align_up((size_t)c->Q * N * c->ops->storage_bytes);
   L.n_ck = (int)((n + K - 1) / K);
   L.n_steps = K;
@@ -259,12 +262,6 @@ AdjLayout adj_layout(lbm_ctx* c, int64_t n, int K) {
   o += L.state_bytes;
   L.total = o;
   return L;
-}
-
-const AdjOps* adj_ops_for(int precision) {
-  if (precision == LBM_FP64) return adj_ops_fp64();
-  if (precision == LBM_FP32DEV) return adj_ops_fp32dev();
-  return adj_ops_bf16dev();
 }
 
 // side stream and fork/join events of the concurrent reverse kernels (ok
@@ -509,34 +506,33 @@ lbm_status lbm_adjoint(lbm_ctx* c, int64_t n, int32_t K, int32_t objective, void
         a.omega = H.omega;
         std::memcpy(a.inlet, c->inlet, sizeof(a.inlet));
         a.inlet_s = c->at<double>(c->oInletS);
-        // interior bricks (the first 64 nB fluid elements) through the brick
-        // tables, everything else through the neighbour list
-        const int64_t nbrick = 64 * H.nB;
-        AdjSCArgs ab = a;
-        ab.begin = H.base + H.oF;
-        ab.nB = H.nB;
-        ab.brick_nb = c->at<int32_t>(c->oBrickNb) + (size_t)H.brick_first * 27;
-        ab.brick_tab = c->at<uint16_t>(c->oBrickTab);
-        // the neighbour-list reverse on the side stream, beside the brick reverse
-        const bool fork = LBM_ADJ_CONCURRENT && side.ok;
+        // bricks through the brick tables, the rest through the neighbour
+        // list, beside the interior bricks on the side stream
+        const int64_t nbrick = 64 * (H.nB + H.nBb);
+        a.begin = H.base + H.oF;
+        a.n_interior = H.nB;
+        a.n_boundary = H.nBb;
+        a.brick_nb = c->at<int32_t>(c->oBrickNb) + (size_t)H.brick_first * 27;
+        a.brick_tab = c->at<uint16_t>(c->oBrickTab);
+        if (c->p.time_mode == LBM_TIME_TWO_LAYER) {
+          a.list_begin = H.base + H.oC;
+          a.list_end = H.base + H.oG1 - nbrick;
+          a.hole_at = H.base + H.oF;
+          a.hole_len = nbrick;
+        } else {
+          a.list_begin = H.base + H.oF + nbrick;
+          a.list_end = H.base + H.oG2;
+          a.hole_at = a.list_end;
+          a.hole_len = 0;
+        }
+        a.row0 = L.side_row0;
+        const bool fork = side.ok && H.nB > 0;
         if (fork) {
           cudaEventRecord(side.fork, st);
           cudaStreamWaitEvent(side.s, side.fork, 0);
         }
-        aops->sc_brick(c->Q, ab, st);
-        if (c->p.time_mode == LBM_TIME_TWO_LAYER) {
-          a.begin = H.base + H.oC;
-          a.end = H.base + H.oG1 - nbrick;
-          a.hole_at = H.base + H.oF;
-          a.hole_len = nbrick;
-        } else {
-          a.begin = H.base + H.oF + nbrick;
-          a.end = H.base + H.oG2;
-          a.hole_at = a.end;
-          a.hole_len = 0;
-        }
-        a.c.partial = partial + (size_t)L.side_row0 * kAccCols;
-        aops->sc(c->Q, a, fork ? side.s : st);
+        aops->sc_interior(c->Q, a, st);
+        aops->sc_rest(c->Q, a, fork ? side.s : st);
         if (fork) {
           cudaEventRecord(side.join, side.s);
           cudaStreamWaitEvent(st, side.join, 0);
@@ -562,11 +558,16 @@ lbm_status lbm_adjoint(lbm_ctx* c, int64_t n, int32_t K, int32_t objective, void
         }
       } else if (t.op == OP_MOM_A || t.op == OP_MOM_B) {
         if (c->ld[li].nsrc == 0) continue;
+        // the fill of the finer level's ghosts has just been reversed into contrib
+        const bool half = t.op == OP_MOM_B;
         AdjMomArgs a{};
         a.c = common(snap(t.snap), nullptr, lam_for(t.parity[li]), li);
         a.elem = c->at<int32_t>(c->ld[li].src_elem);
-        a.lam_rec = W + (t.op == OP_MOM_A ? L.lam_recA[li] : L.lam_recB[li]);
-        a.lam_rec_prev = t.op == OP_MOM_B ? W + L.lam_recA[li] : nullptr;
+        a.contrib = W + L.contrib;
+        a.off = reinterpret_cast<const int32_t*>(W + L.csr_off[li]);
+        a.item = reinterpret_cast<const int32_t*>(W + L.csr_item[li]);
+        a.rec_half = c->p.time_mode == LBM_TIME_LINEAR ? W + L.lam_rec[li] : nullptr;
+        a.half = half;
         a.nsrc = c->ld[li].nsrc;
         a.omega = H.omega;
         aops->moments(c->Q, a, st);
@@ -585,11 +586,6 @@ lbm_status lbm_adjoint(lbm_ctx* c, int64_t n, int32_t K, int32_t objective, void
         a.omega_c = c->M.lv[lc].omega;
         a.omega_f = H.omega;
         aops->gfc(c->Q, a, st);
-        AdjGatherArgs g{W + L.contrib, reinterpret_cast<const int32_t*>(W + L.csr_off[lc]),
-                        reinterpret_cast<const int32_t*>(W + L.csr_item[lc]),
-                        W + (t.op == OP_GFC_A ? L.lam_recA[lc] : L.lam_recB[lc]), c->ld[lc].nsrc,
-                        mom_stride(c->Q)};
-        launch_adj_gather(fp64, g, st);
       } else if (t.op == OP_GFF) {
         if (H.nG1 + H.nG2 == 0) continue;
         AdjGffArgs a{};

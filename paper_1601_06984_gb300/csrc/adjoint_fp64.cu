@@ -88,18 +88,6 @@ void launch_copy_rows(const void* src, void* dst, size_t pitch, size_t off, size
   }
 }
 
-void launch_adj_gather(bool fp64, const AdjGatherArgs& a, cudaStream_t st) {
-  if (a.nsrc <= 0) return;
-  const unsigned g = dev::blocks_for(a.nsrc, 128);
-  if (a.stride == 32) {
-    if (fp64) dev::k_adj_gather<double, 32><<<g, 128, 0, st>>>(a);
-    else dev::k_adj_gather<float, 32><<<g, 128, 0, st>>>(a);
-  } else {
-    if (fp64) dev::k_adj_gather<double, 40><<<g, 128, 0, st>>>(a);
-    else dev::k_adj_gather<float, 40><<<g, 128, 0, st>>>(a);
-  }
-}
-
 void launch_gather_force_user(const double* lam_force, const int32_t* uslot, double* stage, int64_t first,
                               int64_t cnt, int64_t Ntot, int d, cudaStream_t st) {
   if (cnt <= 0) return;

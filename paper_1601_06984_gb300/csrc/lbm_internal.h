@@ -483,8 +483,7 @@ struct Ops {
 // [d][Ntot] FP64; partial holds one running row of parameter derivatives per
 // block (cols 0..15 d/d omega of each level, 16..18 d/d u_in): block b of
 // every launch adds its sums to row b, so the totals are deterministic.
-constexpr int kAdjBlocks = 1024;  // fixed grid of the adjoint kernels (deterministic partials)
-#define LBM_BRICKS_PER_BLOCK 4       // bricks of 64 elements per 256-thread block of the brick kernels
+constexpr int kAdjBlocks = 1024;  // largest grid of the reverse ghost and boundary kernels
 constexpr int kAccCols = 32;
 
 struct AdjCommon {
@@ -493,7 +492,7 @@ struct AdjCommon {
   void* lam_a;        // adjoint buffer the op's outputs live in (consumed, zeroed)
   void* lam_b;        // adjoint buffer of the op's inputs (accumulated)
   double* lam_force;  // [d][Ntot] FP64 accumulated (null: not wanted)
-  double* partial;    // [kAdjBlocks][kAccCols] running sums
+  double* partial;    // [rows][kAccCols] running sums
   int64_t Ntot;
   double rho_off, rho0;
   int la, lb;         // levels whose omega the launch's first / second sums belong to (lb < 0: none)
@@ -501,19 +500,22 @@ struct AdjCommon {
 
 struct AdjSCArgs {
   AdjCommon c;
-  const uint32_t* nbr;
-  const void* side_fwd;  // outlet values the forward used (compute type)
-  void* lam_side;        // adjoint of the outlet values (written)
-  int64_t begin, end;    // neighbour-list kernel: linear range; element = lin + (lin >= hole_at ? hole_len : 0)
-  int64_t hole_at, hole_len;
-  double omega;
-  double inlet[kQmax];   // 6 w_i rho0 (c_i . u_in) of the forward
-  const double* inlet_s;  // inlet profile factor per inlet link
-  // interior-brick kernel: nB bricks of 64 elements from begin, their rows
-  // [nB][27] and the link table [Q-1][64] (as BrickArgs)
+  // bricks: n_interior from element begin, then n_boundary, their rows in the
+  // same order [.][27], link table [Q-1][64]
+  int64_t begin, n_interior, n_boundary;
   const int32_t* brick_nb;
   const uint16_t* brick_tab;
-  int64_t nB;
+  // the rest through the neighbour list: linear range; element = lin + (lin >=
+  // hole_at ? hole_len : 0)
+  const uint32_t* nbr;
+  int64_t list_begin, list_end, hole_at, hole_len;
+  int bnd_blocks;        // blocks of the boundary bricks (set by the launcher)
+  int row0;              // first running row of k_adj_sc_rest, which may run beside the interior
+  double omega;
+  const void* side_fwd;  // outlet values the forward used (compute type)
+  void* lam_side;        // adjoint of the outlet values (written)
+  double inlet[kQmax];   // 6 w_i rho0 (c_i . u_in) of the forward
+  const double* inlet_s;  // inlet profile factor per inlet link
 };
 
 struct AdjOutletArgs {
@@ -530,11 +532,14 @@ struct AdjOutletArgs {
   const double* q;
 };
 
-struct AdjMomArgs {  // reverse of the source moments
+struct AdjMomArgs {  // reverse of the source records
   AdjCommon c;       // lam_b: adjoint of the coarse state
   const int32_t* elem;
-  void* lam_rec;       // [nsrc][mom_stride(Q)] adjoint of the records (consumed, zeroed)
-  void* lam_rec_prev;  // averaging mode: receives half of lam_rec (else null)
+  const void* contrib;  // what k_adj_gfc left per ghost
+  const int32_t* off;   // [nsrc+1] transposed source list
+  const int32_t* item;  // ghost*4 + source slot
+  void* rec_half;       // LINEAR mode: [nsrc][mom_stride(Q)] half of the records' adjoint at t + 1/2
+  int half;             // reverse of the fill at t + 1/2: writes rec_half (else it is added)
   int64_t nsrc;
   double omega;
 };
@@ -544,18 +549,9 @@ struct AdjGfcArgs {  // reverse of the GhostFromCoarser fill, per ghost
   const void* rec;   // forward source records [nsrc][mom_stride(Q)]
   const int32_t* gsrc;
   const uint8_t* oct;
-  void* contrib;     // [ng][4][mom_stride(Q)] per-ghost adjoint of each source record
+  void* contrib;     // per ghost the adjoints of its f^neq, density and velocity
   int64_t ng, dest0;
   double omega_c, omega_f;
-};
-
-struct AdjGatherArgs {  // deterministic sum of the per-ghost contributions per source
-  const void* contrib;
-  const int32_t* off;   // [nsrc+1]
-  const int32_t* item;  // ghost*4 + source slot
-  void* lam_rec;        // [nsrc][stride] accumulated
-  int64_t nsrc;
-  int stride;           // mom_stride(Q): 32 or 40
 };
 
 struct AdjGffArgs {
@@ -587,18 +583,18 @@ struct AccumArgs {
 
 struct AdjOps {
   void (*seed)(int Q, const AdjSeedArgs&, cudaStream_t);
-  void (*sc)(int Q, const AdjSCArgs&, cudaStream_t);
-  void (*sc_brick)(int Q, const AdjSCArgs&, cudaStream_t);  // grid ceil(nB / 4) blocks
+  void (*sc_interior)(int Q, const AdjSCArgs&, cudaStream_t);
+  void (*sc_rest)(int Q, AdjSCArgs&, cudaStream_t);  // boundary bricks and neighbour-list elements
   void (*outlet)(int Q, const AdjOutletArgs&, cudaStream_t);
   void (*moments)(int Q, const AdjMomArgs&, cudaStream_t);
   void (*gfc)(int Q, const AdjGfcArgs&, cudaStream_t);
   void (*gff)(int Q, const AdjGffArgs&, cudaStream_t);
   size_t lam_bytes;  // bytes per adjoint value (compute type)
+  int sc_block;      // threads per block of the reverse stream-collide (one running row per block)
 };
 const AdjOps* adj_ops_fp64();
 const AdjOps* adj_ops_fp32dev();
 const AdjOps* adj_ops_bf16dev();
-void launch_adj_gather(bool fp64, const AdjGatherArgs&, cudaStream_t);
 void launch_accum(const AccumArgs&, cudaStream_t);
 // Copies bytes [off, off + len) of each of `rows` rows of pitch `pitch` from
 // src to dst (same layout); elem is the element size the offsets are multiples of.
