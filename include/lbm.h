@@ -128,11 +128,12 @@ enum { LBM_INLET_UNIFORM = 0, LBM_INLET_PARABOLIC = 1 };
  *                or not finite: LBM_ERR_ARG).
  *  adjoint_tape  how lbm_adjoint records the forward steps it reverses (the
  *                gradients are the same either way): 1 records all steps of a
- *                checkpoint segment in one recompute (two forward passes per
- *                step); 2 recomputes the segment, then each step once more
- *                while recording it (three passes, less memory); 0 picks 1
- *                when its workspace holds at most twice the states of 2 or at
- *                most 8 GiB of states, else 2.  Other values: LBM_ERR_ARG. */
+ *                checkpoint segment in one recompute, the last segment's in
+ *                the forward itself (at most two forward passes per step); 2
+ *                recomputes the segment, then each step once more while
+ *                recording it (three passes, less memory); 0 picks 1 when its
+ *                tape is at most twice the states of 2 or at most 8 GiB, else
+ *                2.  Other values: LBM_ERR_ARG. */
 typedef struct {
   int32_t stencil;
   int32_t precision;
@@ -348,8 +349,8 @@ lbm_status lbm_set_params(lbm_ctx* ctx, double omega_coarse, const double* u_in)
  * dependence of the lbm_init non-equilibrium part); any output may be NULL
  * (with dJ_dF NULL the per-element force adjoint is not accumulated at all).
  * Checkpoints: the state every K
- * coarse steps; each segment is recomputed once, and every step once more while
- * its op inputs are recorded.  adj_ws is a device workspace of
+ * coarse steps; the steps of a segment are recorded onto a tape of states
+ * (params.adjoint_tape) and reversed.  adj_ws is a device workspace of
  * lbm_adjoint_bytes(n_coarse, K) bytes owned by the caller.  Afterwards the
  * simulation is at the final state, as after lbm_step(n_coarse).  The
  * gradient with respect to F is that of the forced scheme (also when
@@ -357,9 +358,9 @@ lbm_status lbm_set_params(lbm_ctx* ctx, double omega_coarse, const double* u_in)
  * adjoint: both calls return LBM_ERR_STATE there. */
 lbm_status lbm_adjoint_bytes(lbm_ctx* ctx, int64_t n_coarse, int32_t K, uint64_t* bytes);
 /* The workspace holds, besides the adjoint buffers, ceil(n_coarse / K)
- * checkpoints and the final state, and (params.adjoint_tape) either K step
- * states plus one step's snapshots, or K steps' snapshots plus two states per
- * step but the last (each a full [Q][Ntot] state of the storage type). */
+ * checkpoints and the final state, and (params.adjoint_tape) the tape of K
+ * steps, or K step states and the tape of one step.  A step's tape holds one
+ * full [Q][Ntot] state of the storage type per substep of the finest level. */
 lbm_status lbm_adjoint(lbm_ctx* ctx, int64_t n_coarse, int32_t K, int32_t objective, void* adj_ws,
                        uint64_t bytes, double* J, double* dJ_dF, double* dJ_domega, double* dJ_duin,
                        double* dJ_df0);

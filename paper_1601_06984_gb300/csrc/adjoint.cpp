@@ -2,16 +2,17 @@
 //
 // lbm_adjoint runs the forward steps from the current state, keeping a copy of
 // the state every K coarse steps.  Going backwards segment by segment, it
-// recomputes the segment once to keep every step's starting state, then for
-// each step (last to first) recomputes that step once more while recording its
-// op sequence (the "tape") together with copies of every level state an op
-// read, and applies the reverse kernels to the tape in reverse order.
+// records the segment's steps: the stream-collides write every new state into
+// a tape of states instead of the two buffers, so that the reverse reads them
+// in place, nothing copied.  Either the whole segment is recorded at once (the
+// last one already while the forward passes through it), or each step, last to
+// first, from its starting state.  The reverse kernels then run the steps' ops
+// in the reverse of the recursive order.
 #include <cuda_runtime_api.h>
 
 #include <algorithm>
 #include <cmath>
 #include <cstring>
-#include <map>
 #include <string>
 #include <vector>
 
@@ -27,22 +28,23 @@ inline size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 struct TapeOp {
   int op = 0, level = 0;
-  int snap = -1;       // snapshot of the state the op reads (level, or level+1 for GFF)
-  int snap_a = -1;     // GFC: snapshot for the records at t (momA)
-  int snap_b = -1;     // GFC B: snapshot for the records at t+1
+  int k = 0;   // state the op reads, of its level (GFF: of the finer level; GFC: records at t of the coarser
+               // level): 0 the step's start, k the one its k-th stream-collide in the step wrote
+  int kb = 0;  // GFC B: state of the records at t + 1
+  int mid = 0; // MOM B, GFC B: how many of the level's mid-step saves precede the op's
   std::vector<int> parity;  // parities of all levels before the op
 };
 
 struct AdjLayout {
   size_t lamA = 0, lamB = 0, lamF = 0, side_fwd = 0, lam_side = 0, partial = 0, acc = 0, contrib = 0;
   std::vector<size_t> lam_rec, recA, recB, csr_off, csr_item;
-  size_t ck = 0, steps = 0, snaps = 0, ends = 0, fin = 0;
-  int n_ck = 0, n_steps = 0, n_snaps = 0;
-  // tape_all: a segment's recompute records every step's tape (two forward
-  // passes per step instead of three); needs K tapes' copies plus, per step but
-  // the last, copies of the states the reverse reads in place (both buffers)
-  bool tape_all = false;
-  size_t state_bytes = 0, total = 0;
+  std::vector<size_t> src_saved;  // per level: index of each record among the saved sources, or -1
+  std::vector<size_t> save_off, save_bytes;  // per level: its saves in a step's part of the tape
+  size_t ck = 0, steps = 0, tape = 0, fin = 0;
+  int n_ck = 0, n_steps = 0;
+  int n_slots = 0;        // states of the most often advanced level in one coarse step
+  bool tape_all = false;  // a whole segment on the tape, else one step
+  size_t state_bytes = 0, step_bytes = 0, total = 0;
   int partial_rows = 0;  // running rows of the parameter sums: the largest grid of a reverse launch
   int side_row0 = 0;     // first row of the neighbour-list reverse, which runs beside the brick reverse
 };
@@ -54,142 +56,57 @@ void copy_level(lbm_ctx* c, const void* from, void* to, int li) {
   launch_copy_rows(from, to, (size_t)c->M.Ntot * s, (size_t)H.base * s, (size_t)H.N * s, c->Q, s, c->st);
 }
 
-// Walks (dry) or follows (recording) one coarse step and decides, per level
-// state an op reads, where the reverse sweep finds it.  A state is identified
-// by (level, version); the version of a level is bumped by every op that
-// writes it.  A state that no later op of the step overwrites (its buffer
-// keeps it until the next restore) is read in place; the others are copied to
-// the snapshot store when they are first read.  A copy fills only its level's
-// segment of a full-size slot, so copies of different levels share slots: the
-// k-th copy of every level goes to slot k.
-struct Recorder {
-  lbm_ctx* c;
-  bool counting = true;
-  std::vector<int> version;                    // per level, bumped by every write
-  std::map<std::pair<int, int>, int> snap_of;  // (level, version) -> snapshot index
-  std::vector<std::pair<int, int>> snap_key;
-  std::vector<int> snap_buf;                   // buffer (parity) the state lives in
-  std::vector<char> clobbered;                 // a later op of the step wrote that buffer
-  std::vector<char> need_copy;                 // from the dry walk: copy instead of reading in place
-  std::vector<const void*> where;              // recording: where the reverse reads each state
+// The ops of one coarse step in the order of the recursion (a dry walk from
+// the current parities, launching nothing): the reverse sweep's program.
+std::vector<TapeOp> plan_step(lbm_ctx* c) {
   std::vector<TapeOp> tape;
-  int last_mom_a_snap[16], last_mom_b_snap[16];
-  char* snap_base = nullptr;
-  size_t state_bytes = 0;
-  int max_snaps = 0;
-  int n_copies[16] = {};                       // copies taken so far, per level
-  bool overflow = false;
-
-  explicit Recorder(lbm_ctx* ctx) : c(ctx), version(ctx->nlev, 0) {
-    std::fill(last_mom_a_snap, last_mom_a_snap + 16, -1);
-    std::fill(last_mom_b_snap, last_mom_b_snap + 16, -1);
-  }
-
-
-  void wrote(int li, int buf) {
-    for (size_t id = 0; id < snap_key.size(); ++id)
-      if (snap_key[id].first == li && snap_buf[id] == buf) clobbered[id] = 1;
-    version[li]++;
-  }
-
-  int snapshot(int li) {
-    auto key = std::make_pair(li, version[li]);
-    auto it = snap_of.find(key);
-    if (it != snap_of.end()) return it->second;
-    const int id = (int)snap_key.size();
-    snap_of[key] = id;
-    snap_key.push_back(key);
-    snap_buf.push_back(c->parity[li]);
-    clobbered.push_back(0);
-    if (!counting) {
-      const bool copy = id < (int)need_copy.size() ? need_copy[id] != 0 : true;
-      if (!copy) {
-        where.push_back(c->cur(li));
-      } else if (n_copies[li] >= max_snaps) {
-        overflow = true;
-        where.push_back(nullptr);
-        return id;
-      } else {
-        char* dst = snap_base + (size_t)n_copies[li]++ * state_bytes;
-        copy_level(c, c->cur(li), dst, li);
-        where.push_back(dst);
-      }
-    }
-    return id;
-  }
-
-  void on(int op, int li) {
+  std::vector<int> sc(c->nlev, 0), at_a(c->nlev, 0), mids(c->nlev, 0);
+  const std::vector<int> saved = c->parity;
+  c->hook = [&](int op, int li) {
     TapeOp t;
     t.op = op;
     t.level = li;
     t.parity = c->parity;
     switch (op) {
-      case OP_GFF:
-        t.snap = snapshot(li + 1);
-        tape.push_back(t);
-        wrote(li, c->parity[li]);
-        break;
-      case OP_MOM_A:
-        t.snap = snapshot(li);
-        last_mom_a_snap[li] = t.snap;
-        tape.push_back(t);
-        break;
-      case OP_GFC_A:
-        t.snap_a = last_mom_a_snap[li - 1];
-        tape.push_back(t);
-        wrote(li, c->parity[li]);
-        break;
-      case OP_SC:
-        t.snap = snapshot(li);
-        tape.push_back(t);
-        wrote(li, c->parity[li] ^ 1);
-        break;
+      case OP_GFF: t.k = sc[li + 1]; break;
+      case OP_MOM_A: t.k = at_a[li] = sc[li]; break;
+      case OP_GFC_A: t.k = at_a[li - 1]; break;
+      case OP_SC: t.k = sc[li]++; break;
       case OP_MOM_B:
-        t.snap = snapshot(li);
-        t.snap_a = last_mom_a_snap[li];
-        last_mom_b_snap[li] = t.snap;
-        tape.push_back(t);
+        t.k = sc[li];
+        t.mid = mids[li]++;
         break;
       case OP_GFC_B:
-        t.snap_a = last_mom_a_snap[li - 1];
-        t.snap_b = last_mom_b_snap[li - 1];
-        tape.push_back(t);
-        wrote(li, c->parity[li]);
+        t.k = at_a[li - 1];
+        t.kb = sc[li - 1];
+        t.mid = mids[li - 1] - 1;
         break;
     }
-  }
-};
-
-// Dry walk of one coarse step from the current parities (launches nothing):
-// the states its ops read and which of them a later op overwrites.
-void dry_walk(lbm_ctx* c, Recorder& r) {
-  r.counting = true;
-  std::vector<int> saved = c->parity;
-  c->hook = [&](int op, int li) { r.on(op, li); };
+    tape.push_back(t);
+  };
   c->dry = true;
   c->advance(0);
   c->dry = false;
   c->hook = nullptr;
   c->parity = saved;
+  return tape;
 }
 
-// Which of the states the next coarse step's ops read must be copied.
-std::vector<char> plan_snapshots(lbm_ctx* c) {
-  Recorder r(c);
-  dry_walk(c, r);
-  return r.clobbered;
-}
+// One recorded coarse step: per level its states in the step (the start, then
+// one per stream-collide), and the GhostFromFiner sources' pdfs at the end of
+// each of its substeps, which the next GhostFromFiner fill overwrites in place
+// (LINEAR mode: the records at t + 1 include them).
+struct Recorded {
+  std::vector<std::vector<const void*>> states, mids;
+  const void* state(int li, int k) const { return k < (int)states[li].size() ? states[li][k] : nullptr; }
+  const void* mid(int li, int k) const { return k < (int)mids[li].size() ? mids[li][k] : nullptr; }
+};
 
-// Snapshot slots one coarse step's tape needs: the largest number of copies of
-// one level (the same for every step: the pattern depends only on which of a
-// level's two buffers an op touches).
-int count_snapshots(lbm_ctx* c) {
-  Recorder r(c);
-  dry_walk(c, r);
-  std::vector<int> per_level(c->nlev, 0);
-  for (size_t id = 0; id < r.snap_key.size(); ++id)
-    if (r.clobbered[id]) per_level[r.snap_key[id].first]++;
-  return per_level.empty() ? 0 : *std::max_element(per_level.begin(), per_level.end());
+// substeps of level li in a coarse step
+int64_t substeps(const lbm_ctx* c, int li) {
+  int64_t n = 1;
+  for (int l = 0; l < li; ++l) n *= time_ratio(c->p.time_mode);
+  return n;
 }
 
 const AdjOps* adj_ops_for(int precision) {
@@ -239,25 +156,32 @@ AdjLayout adj_layout(lbm_ctx* c, int64_t n, int K) {
     max_contrib = std::max(max_contrib, nfine);
   }
   L.contrib = take((size_t)max_contrib * ((c->Q + 3) / 4 * 4 + 4) * lb);
+  for (int li = 0; li < c->nlev; ++li) L.src_saved.push_back(take(c->M.lv[li].src_elem.size() * 4));
   L.state_bytes = align_up((size_t)c->Q * N * c->ops->storage_bytes);
   L.n_ck = (int)((n + K - 1) / K);
   L.n_steps = K;
-  L.n_snaps = count_snapshots(c);
+  L.n_slots = (int)substeps(c, c->n_filled - 1);
+  // a step's part of the tape: n_slots states (a state fills only its level's
+  // rows of a full-size slot, so the k-th of every level share slot k), then
+  // the levels' saves
+  L.step_bytes = (size_t)L.n_slots * L.state_bytes;
+  for (int li = 0; li < c->nlev; ++li) {
+    L.save_off.push_back(L.step_bytes);
+    L.save_bytes.push_back(align_up((size_t)c->Q * c->M.lv[li].gsrc_elem.size() * c->ops->storage_bytes));
+    if (c->p.time_mode == LBM_TIME_LINEAR && li + 1 < c->nlev) L.step_bytes += L.save_bytes[li] * (size_t)substeps(c, li);
+  }
   // workspace rule: record the whole segment when that needs at most twice the
-  // states of the step-by-step scheme, or at most 8 GiB of states
-  const size_t per_step_old = (size_t)K + (size_t)L.n_snaps;
-  const size_t per_step_new = (size_t)K * (size_t)(L.n_snaps + 2);
+  // states of the step-by-step scheme, or at most 8 GiB
+  const size_t by_step = (size_t)K * L.state_bytes + L.step_bytes, whole = (size_t)K * L.step_bytes;
   if (c->p.adjoint_tape == 1) L.tape_all = true;
   else if (c->p.adjoint_tape == 2) L.tape_all = false;
-  else L.tape_all = per_step_new <= 2 * per_step_old || per_step_new * L.state_bytes <= ((size_t)8 << 30);
+  else L.tape_all = whole <= 2 * by_step || whole <= ((size_t)8 << 30);
   L.ck = o;
   o += (size_t)L.n_ck * L.state_bytes;
   L.steps = o;
   if (!L.tape_all) o += (size_t)L.n_steps * L.state_bytes;
-  L.snaps = o;
-  o += (size_t)L.n_snaps * L.state_bytes * (L.tape_all ? (size_t)K : 1);
-  L.ends = o;
-  if (L.tape_all) o += (size_t)2 * (size_t)(K - 1) * L.state_bytes;
+  L.tape = o;
+  o += L.step_bytes * (L.tape_all ? (size_t)std::min<int64_t>(K, n) : 1);
   L.fin = o;
   o += L.state_bytes;
   L.total = o;
@@ -354,6 +278,10 @@ lbm_status lbm_adjoint(lbm_ctx* c, int64_t n, int32_t K, int32_t objective, void
     s = chk(cudaMemcpyAsync(W + L.csr_off[li], off.data(), off.size() * 4, cudaMemcpyHostToDevice, st), "csr");
     if (s == LBM_OK && !item.empty())
       s = chk(cudaMemcpyAsync(W + L.csr_item[li], item.data(), item.size() * 4, cudaMemcpyHostToDevice, st), "csr");
+    std::vector<int32_t> saved(nsrc, -1);
+    for (size_t k = 0; k < Hc.gsrc_rec.size(); ++k) saved[Hc.gsrc_rec[k]] = (int32_t)k;
+    if (s == LBM_OK && nsrc > 0)
+      s = chk(cudaMemcpyAsync(W + L.src_saved[li], saved.data(), saved.size() * 4, cudaMemcpyHostToDevice, st), "csr");
     if (s == LBM_OK) s = chk(cudaStreamSynchronize(st), "csr sync");
     if (s != LBM_OK) return s;
   }
@@ -361,6 +289,7 @@ lbm_status lbm_adjoint(lbm_ctx* c, int64_t n, int32_t K, int32_t objective, void
     for (int li = 0; li < c->nlev; ++li) copy_level(c, c->cur(li), dst, li);
   };
   auto restore_state = [&](const char* src, const std::vector<int>& par) {
+    c->reset_state_buffers();
     for (int li = 0; li < c->nlev; ++li) {
       c->parity[li] = par[li];
       copy_level(c, src, c->cur(li), li);
@@ -381,13 +310,83 @@ lbm_status lbm_adjoint(lbm_ctx* c, int64_t n, int32_t K, int32_t objective, void
     parity_at[n] = c->parity;
     c->parity = p0;
   }
+  // however this call ends, the context is back on its own two buffers
+  struct Buffers {
+    lbm_ctx* c;
+    ~Buffers() {
+      c->new_state = nullptr;
+      c->at_mid_step = nullptr;
+      c->reset_state_buffers();
+    }
+  } buffers{c};
+  // rows [at, at + cnt) of level li
+  auto copy_rows_of = [&](const void* from, void* to, int li, int64_t at, int64_t cnt) {
+    const size_t sb = c->ops->storage_bytes;
+    launch_copy_rows(from, to, N * sb, (size_t)(c->M.lv[li].base + at) * sb, (size_t)cnt * sb, c->Q, sb, st);
+  };
+  // runs one coarse step, its new states going to the tape's part at `part`
+  auto record_step = [&](Recorded& r, char* part) {
+    r.states.assign(c->nlev, {});
+    r.mids.assign(c->nlev, {});
+    c->ensure_records();
+    for (int li = 0; li < c->nlev; ++li) r.states[li].push_back(c->cur(li));
+    c->new_state = [&](int li) -> void* {
+      char* slot = part + (r.states[li].size() - 1) * L.state_bytes;
+      r.states[li].push_back(slot);
+      // slots that no op of the step writes before they are read: an outer
+      // GhostFromFiner ghost that is a source, at t + 1 (no mesh has one so far)
+      if (c->ld[li].n_gsrc > c->ld[li].n_gsrc_inner) copy_rows_of(c->nxt(li), slot, li, c->M.lv[li].oG2, c->M.lv[li].nG2);
+      return slot;
+    };
+    c->at_mid_step = [&](int li) {
+      const HostLevel& H = c->M.lv[li];
+      char* to = part + L.save_off[li] + r.mids[li].size() * L.save_bytes[li];
+      r.mids[li].push_back(to);
+      launch_gather_elements(c->cur(li), to, c->at<int32_t>(c->ld[li].gsrc_elem), (int64_t)H.gsrc_elem.size(), (int64_t)N,
+                             c->Q, c->ops->storage_bytes, st);
+    };
+    if (c->timing != 1 && c->can_batch()) c->step_batched();
+    else c->advance(0);
+    c->new_state = nullptr;
+    c->at_mid_step = nullptr;
+  };
+  std::vector<Recorded> recs(L.tape_all ? std::min<int64_t>(K, n) : 1);
   for (int64_t t = 0; t < n && s == LBM_OK; t += K) {
-    save_state(W + L.ck + (size_t)(t / K) * L.state_bytes);
-    s = c->run_steps(std::min<int64_t>(K, n - t));
+    if (L.tape_all && t + K >= n) {
+      // the last segment is recorded as the forward passes through it
+      for (int64_t k = t; k < n; ++k) record_step(recs[k - t], W + L.tape + (size_t)(k - t) * L.step_bytes);
+      s = c->launched("adjoint forward");
+    } else {
+      save_state(W + L.ck + (size_t)(t / K) * L.state_bytes);
+      s = c->run_steps(std::min<int64_t>(K, n - t));
+    }
   }
   if (s == LBM_OK && c->parity != parity_at[n]) s = c->fail(LBM_ERR_INTERNAL, "adjoint forward parities differ");
   if (s != LBM_OK) return s;
   save_state(W + L.fin);
+  if (L.tape_all) {
+    // The ghost slots that no stream-collide writes, as lbm_step leaves them:
+    // what the fills put into the same buffer two substeps earlier, and in
+    // LINEAR mode the outer GhostFromCoarser layer, which the steps leave
+    // alone, as the context's buffer holds it.
+    const bool linear = c->p.time_mode == LBM_TIME_LINEAR;
+    for (int li = 0; li < c->nlev; ++li) {
+      const HostLevel& H = c->M.lv[li];
+      std::vector<const void*> seq;  // the states of the recorded steps
+      for (int64_t k = 0; k < n - (int64_t)(L.n_ck - 1) * K; ++k)
+        seq.insert(seq.end(), recs[k].states[li].begin() + (k ? 1 : 0), recs[k].states[li].end());
+      const void* own = parity_at[n][li] ? c->at(c->oB) : c->at(c->oA);
+      const void* before = seq.size() >= 3 ? seq[seq.size() - 3] : own;
+      if (linear) {
+        launch_copy_ghosts(before, own, W + L.fin, c->at<uint8_t>(c->ld[li].gfc_oct), H.base + H.oC, H.nC, (int64_t)N, c->Q,
+                           c->ops->storage_bytes, st);
+        copy_rows_of(before, W + L.fin, li, H.oG2, H.nG2);
+      } else {
+        copy_rows_of(before, W + L.fin, li, H.oG1, H.nG1);
+        copy_rows_of(before, W + L.fin, li, H.oG2, H.nG2);
+      }
+    }
+  }
   s = c->launched("adjoint forward");
   if (s != LBM_OK) return s;
   // ---- objective and seed
@@ -445,26 +444,27 @@ lbm_status lbm_adjoint(lbm_ctx* c, int64_t n, int32_t K, int32_t objective, void
   }
   // ---- reverse sweep
   const int nseg = L.n_ck;
-  // records one coarse step's tape while running it (copies into snap_base)
-  auto record_step = [&](Recorder& r, char* snap_base) -> lbm_status {
-    r.counting = false;
-    r.need_copy = plan_snapshots(c);
-    r.snap_base = snap_base;
-    r.state_bytes = L.state_bytes;
-    r.max_snaps = L.n_snaps;
-    c->ensure_records();  // before the hook: the tape holds the step's own ops only
-    c->hook = [&](int op, int li) { r.on(op, li); };
-    c->advance(0);
-    c->hook = nullptr;
-    if (r.overflow) return c->fail(LBM_ERR_INTERNAL, "adjoint tape needs more snapshots than counted");
-    if (r.clobbered != r.need_copy) return c->fail(LBM_ERR_INTERNAL, "adjoint tape differs from its plan");
-    return LBM_OK;
+  // the op sequence depends only on the starting parity of the coarsest level
+  std::vector<TapeOp> plans[2];
+  auto plan = [&](const std::vector<int>& par) -> const std::vector<TapeOp>& {
+    std::vector<TapeOp>& t = plans[par[0] & 1];
+    if (t.empty()) {
+      const std::vector<int> p0 = c->parity;
+      c->parity = par;
+      t = plan_step(c);
+      c->parity = p0;
+    }
+    return t;
   };
   // runs one recorded step backwards
-  auto reverse_step = [&](Recorder& r) {
-    auto snap = [&](int id) { return r.where[id]; };
-    // forward records of an interface, recomputed from the snapshots
-    auto records = [&](int lc, int sa, int sb) {
+  auto reverse_step = [&](const Recorded& r, const std::vector<TapeOp>& tape) {
+    auto saved = [&](int li, int mid) {
+      return SavedSources{r.mid(li, mid), reinterpret_cast<const int32_t*>(W + L.src_saved[li]),
+                          (int64_t)c->M.lv[li].gsrc_elem.size()};
+    };
+    // forward records of an interface from the tape's states: at t, and for
+    // the fill at t + 1/2 (kb >= 0) the means of those at t and t + 1
+    auto records = [&](int lc, int ka, int kb, int mid) {
       const HostLevel& Hc = c->M.lv[lc];
       MomentsArgs m{};
       m.force = force;
@@ -475,19 +475,20 @@ lbm_status lbm_adjoint(lbm_ctx* c, int64_t n, int32_t K, int32_t objective, void
       m.rx32 = make_relax32(Hc.omega);
       m.rho_off = c->rho_off;
       m.rho_off32 = (float)c->rho_off;
-      m.src = snap(sa);
+      m.src = r.state(lc, ka);
       m.mom = W + L.recA[lc];
-      m.prev = nullptr;
-      c->ops->source_moments(c->Q, m, st);
-      if (sb < 0) return static_cast<const void*>(W + L.recA[lc]);
-      m.src = snap(sb);
+      // LINEAR mode reverses the fill at t + 1/2 first, which has formed these
+      if (kb >= 0 || c->p.time_mode != LBM_TIME_LINEAR) c->ops->source_moments(c->Q, m, st);
+      if (kb < 0) return static_cast<const void*>(W + L.recA[lc]);
+      m.src = r.state(lc, kb);
+      m.saved = saved(lc, mid);
       m.mom = W + L.recB[lc];
       m.prev = W + L.recA[lc];
       c->ops->source_moments(c->Q, m, st);
       return static_cast<const void*>(W + L.recB[lc]);
     };
-    for (int k = (int)r.tape.size() - 1; k >= 0; --k) {
-      const TapeOp& t = r.tape[k];
+    for (int k = (int)tape.size() - 1; k >= 0; --k) {
+      const TapeOp& t = tape[k];
       const int li = t.level;
       const HostLevel& H = c->M.lv[li];
       if (t.op == OP_SC) {
@@ -495,11 +496,11 @@ lbm_status lbm_adjoint(lbm_ctx* c, int64_t n, int32_t K, int32_t objective, void
         const bool outlet = H.out_end > H.out_begin;
         if (outlet) {
           OutletArgs o = c->outlet_args(W + L.side_fwd);
-          c->add_outlet(o, li, snap(t.snap));
+          c->add_outlet(o, li, r.state(li, t.k));
           c->ops->outlet(c->Q, o, st);
         }
         AdjSCArgs a{};
-        a.c = common(snap(t.snap), lam_for(!p), lam_for(p), li);
+        a.c = common(r.state(li, t.k), lam_for(!p), lam_for(p), li);
         a.nbr = c->at<uint32_t>(c->oNbr);
         a.side_fwd = W + L.side_fwd;
         a.lam_side = W + L.lam_side;
@@ -540,7 +541,7 @@ lbm_status lbm_adjoint(lbm_ctx* c, int64_t n, int32_t K, int32_t objective, void
         if (outlet) {
           for (int which = 0; which < (c->p.bouzidi ? 6 : 3); ++which) {
             AdjOutletArgs o{};
-            o.c = common(snap(t.snap), nullptr, lam_for(p), li);
+            o.c = common(r.state(li, t.k), nullptr, lam_for(p), li);
             o.elem = c->at<int32_t>(c->oOutElem);
             o.a = c->at<int32_t>(c->oOutA);
             o.b = c->at<int32_t>(c->oOutB);
@@ -561,8 +562,9 @@ lbm_status lbm_adjoint(lbm_ctx* c, int64_t n, int32_t K, int32_t objective, void
         // the fill of the finer level's ghosts has just been reversed into contrib
         const bool half = t.op == OP_MOM_B;
         AdjMomArgs a{};
-        a.c = common(snap(t.snap), nullptr, lam_for(t.parity[li]), li);
+        a.c = common(r.state(li, t.k), nullptr, lam_for(t.parity[li]), li);
         a.elem = c->at<int32_t>(c->ld[li].src_elem);
+        if (half) a.saved = saved(li, t.mid);
         a.contrib = W + L.contrib;
         a.off = reinterpret_cast<const int32_t*>(W + L.csr_off[li]);
         a.item = reinterpret_cast<const int32_t*>(W + L.csr_item[li]);
@@ -574,7 +576,7 @@ lbm_status lbm_adjoint(lbm_ctx* c, int64_t n, int32_t K, int32_t objective, void
       } else if (t.op == OP_GFC_A || t.op == OP_GFC_B) {
         if (H.nC == 0) continue;
         const int lc = li - 1;
-        const void* rec = records(lc, t.snap_a, t.op == OP_GFC_B ? t.snap_b : -1);
+        const void* rec = records(lc, t.k, t.op == OP_GFC_B ? t.kb : -1, t.mid);
         AdjGfcArgs a{};
         a.c = common(nullptr, lam_for(t.parity[li]), nullptr, lc, li);
         a.rec = rec;
@@ -589,7 +591,7 @@ lbm_status lbm_adjoint(lbm_ctx* c, int64_t n, int32_t K, int32_t objective, void
       } else if (t.op == OP_GFF) {
         if (H.nG1 + H.nG2 == 0) continue;
         AdjGffArgs a{};
-        a.c = common(snap(t.snap), lam_for(t.parity[li]), lam_for(t.parity[li + 1]), li, li + 1);
+        a.c = common(r.state(li + 1, t.k), lam_for(t.parity[li]), lam_for(t.parity[li + 1]), li, li + 1);
         a.child0 = c->at<int32_t>(c->ld[li].gff_child0);
         a.ng = H.nG1 + H.nG2;
         a.n_inner = H.nG1;
@@ -604,41 +606,24 @@ lbm_status lbm_adjoint(lbm_ctx* c, int64_t n, int32_t K, int32_t objective, void
   };
   for (int seg = nseg - 1; seg >= 0 && s == LBM_OK; --seg) {
     const int64_t s0 = (int64_t)seg * K, s1 = std::min<int64_t>(s0 + K, n);
-    restore_state(W + L.ck + (size_t)seg * L.state_bytes, parity_at[s0]);
     if (L.tape_all) {
-      // record every step of the segment in one recompute; what a step's
-      // reverse would read in place is copied before the next step overwrites
-      // it (both buffers of a level can hold such a state)
-      std::vector<Recorder> recs;
-      recs.reserve((size_t)(s1 - s0));
-      for (int64_t t = s0; t < s1 && s == LBM_OK; ++t) {
-        recs.emplace_back(c);
-        Recorder& r = recs.back();
-        s = record_step(r, W + L.snaps + (size_t)(t - s0) * L.n_snaps * L.state_bytes);
-        if (s != LBM_OK || t + 1 == s1) continue;
-        char* ends = W + L.ends + (size_t)(t - s0) * 2 * L.state_bytes;
-        for (size_t id = 0; id < r.snap_key.size(); ++id) {
-          if (r.need_copy[id]) continue;
-          const int li = r.snap_key[id].first;
-          const int buf = r.snap_buf[id];
-          char* dst = ends + (size_t)buf * L.state_bytes;
-          copy_level(c, buf ? c->at(c->oB) : c->at(c->oA), dst, li);
-          r.where[id] = dst;
-        }
+      if (s1 < n) {
+        restore_state(W + L.ck + (size_t)seg * L.state_bytes, parity_at[s0]);
+        for (int64_t t = s0; t < s1; ++t) record_step(recs[t - s0], W + L.tape + (size_t)(t - s0) * L.step_bytes);
       }
-      for (int64_t t = s1 - 1; t >= s0 && s == LBM_OK; --t) s = reverse_step(recs[t - s0]);
+      for (int64_t t = s1 - 1; t >= s0 && s == LBM_OK; --t) s = reverse_step(recs[t - s0], plan(parity_at[t]));
     } else {
       // recompute the segment keeping each step's start state; the last step's
-      // is the live state, which its tape pass starts from directly
-      for (int64_t t = s0; t + 1 < s1; ++t) {
+      // is the live state, which its recording starts from directly
+      restore_state(W + L.ck + (size_t)seg * L.state_bytes, parity_at[s0]);
+      for (int64_t t = s0; t + 1 < s1 && s == LBM_OK; ++t) {
         save_state(W + L.steps + (size_t)(t - s0) * L.state_bytes);
-        c->coarse_step();
+        s = c->run_steps(1);
       }
       for (int64_t t = s1 - 1; t >= s0 && s == LBM_OK; --t) {
         if (t + 1 < s1) restore_state(W + L.steps + (size_t)(t - s0) * L.state_bytes, parity_at[t]);
-        Recorder r(c);
-        s = record_step(r, W + L.snaps);
-        if (s == LBM_OK) s = reverse_step(r);
+        record_step(recs[0], W + L.tape);
+        s = reverse_step(recs[0], plan(parity_at[t]));
       }
     }
   }

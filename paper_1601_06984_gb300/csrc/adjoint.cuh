@@ -789,8 +789,7 @@ __global__ void __launch_bounds__(sizeof(typename Sto<S>::R) == 8 ? 32 : 128) k_
     }
     const int64_t e = a.elem[k];
     R g[Q];
-#pragma unroll
-    for (int q = 0; q < Q; ++q) g[q] = Sto<S>::ld(x + (size_t)q * N + e);
+    load_source<Q, S>(a.saved, x, N, e, k, g);
     R F[3];
     load_force<S, R>(a.c.force, a.c.Ntot, e, F, D);
     R lg[Q], lF[3] = {R(0), R(0), R(0)}, lom = R(0);

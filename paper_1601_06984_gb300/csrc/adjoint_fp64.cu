@@ -34,6 +34,22 @@ __global__ void __launch_bounds__(256) k_copy_rows(const T* __restrict__ src, T*
     dst[base + k] = src[base + k];
 }
 
+template <class T>
+__global__ void k_gather_elements(const T* __restrict__ src, T* __restrict__ dst, const int32_t* __restrict__ elem,
+                                  int64_t n, int64_t pitch) {
+  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (k < n) dst[blockIdx.y * n + k] = src[blockIdx.y * pitch + elem[k]];
+}
+
+template <class T>
+__global__ void k_copy_ghosts(const T* __restrict__ inner, const T* __restrict__ outer, T* __restrict__ dst,
+                              const uint8_t* __restrict__ oct, int64_t first, int64_t ng, int64_t pitch) {
+  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= ng) return;
+  const int64_t at = blockIdx.y * pitch + first + k;
+  dst[at] = oct[k] & kGfcOuter ? outer[at] : inner[at];
+}
+
 __global__ void k_gather_force_user(const double* lam_force, const int32_t* uslot, double* stage, int64_t first,
                                     int64_t cnt, int64_t Ntot, int d) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -63,6 +79,33 @@ void launch_gather_lam_user(bool fp64, const void* lamA, const void* lamB, uint3
   const unsigned g = dev::blocks_for(cnt, 256);
   if (fp64) dev::k_gather_lam_user<double><<<g, 256, 0, st>>>(lamA, lamB, parity, uslot, ulev, stage, first, cnt, Ntot, Q);
   else dev::k_gather_lam_user<float><<<g, 256, 0, st>>>(lamA, lamB, parity, uslot, ulev, stage, first, cnt, Ntot, Q);
+}
+
+void launch_gather_elements(const void* src, void* dst, const int32_t* elem, int64_t n, int64_t pitch, int Q, size_t size,
+                            cudaStream_t st) {
+  if (n <= 0) return;
+  const dim3 grid(dev::blocks_for(n, 128), (unsigned)Q);
+  auto go = [&](auto zero) {
+    using T = decltype(zero);
+    dev::k_gather_elements<T><<<grid, 128, 0, st>>>(static_cast<const T*>(src), static_cast<T*>(dst), elem, n, pitch);
+  };
+  if (size == 8) go(uint64_t());
+  else if (size == 4) go(uint32_t());
+  else go(uint16_t());
+}
+
+void launch_copy_ghosts(const void* inner, const void* outer, void* dst, const uint8_t* oct, int64_t first, int64_t ng,
+                        int64_t pitch, int Q, size_t size, cudaStream_t st) {
+  if (ng <= 0) return;
+  const dim3 grid(dev::blocks_for(ng, 128), (unsigned)Q);
+  auto go = [&](auto zero) {
+    using T = decltype(zero);
+    dev::k_copy_ghosts<T><<<grid, 128, 0, st>>>(static_cast<const T*>(inner), static_cast<const T*>(outer),
+                                                static_cast<T*>(dst), oct, first, ng, pitch);
+  };
+  if (size == 8) go(uint64_t());
+  else if (size == 4) go(uint32_t());
+  else go(uint16_t());
 }
 
 void launch_accum(const AccumArgs& a, cudaStream_t st) { dev::k_accum<<<1, 256, 0, st>>>(a); }

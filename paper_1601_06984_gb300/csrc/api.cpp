@@ -293,6 +293,7 @@ int lbm_ctx::add_sc(ScArgs& a, int slot, int li, int kind) const {
 }
 
 void lbm_ctx::stream_collide(int li) {
+  if (new_state) state[li][parity[li] ^ 1] = new_state(li);
   OutletArgs o = outlet_args(at(oSide));
   add_outlet(o, li, cur(li));
   if (o.nlev) {
@@ -353,6 +354,8 @@ void lbm_ctx::tick_batched(int l0, int n) {
     cudaEventRecord(br.join[b], br.s[b]);
     cudaStreamWaitEvent(st, br.join[b], 0);
   };
+  if (new_state)
+    for (int l = l0; l < n; ++l) state[l][parity[l] ^ 1] = new_state(l);
   ScArgs in = sc_args(), rest = sc_args();
   OutletArgs out = outlet_args(at(oSide));
   int64_t elements = 0;
@@ -365,7 +368,7 @@ void lbm_ctx::tick_batched(int l0, int n) {
     add_outlet(out, l, cur(l));
     launches += out.nlev - no;
   }
-  const bool chain = elements <= (p.precision == LBM_FP64 ? kChainElements64 : kChainElements);
+  const bool chain = capturing && elements <= (p.precision == LBM_FP64 ? kChainElements64 : kChainElements);
   rest.chain = chain;
   const bool force = p.use_force != 0;
   // Interior bricks read no ghost.  At small instants they all run beside the
@@ -414,6 +417,7 @@ void lbm_ctx::tick_batched(int l0, int n) {
   GfcArgs gfc = gfc_args();
   gfc.chain = chain;
   if (p.time_mode == LBM_TIME_LINEAR && l0 > 0) {
+    if (at_mid_step) at_mid_step(l0 - 1);
     source_moments(l0 - 1, ld[l0 - 1].momA[parity[l0 - 1]], nullptr, SRC_GFF_OUTER);
     add_gfc(gfc, l0, true, false);
   }
@@ -467,7 +471,10 @@ void lbm_ctx::advance(int li) {
   if (has_finer) {
     advance(li + 1);
     if (linear) {
-      if (op(OP_MOM_B, li)) source_moments(li, ld[li].momA[parity[li]], nullptr, SRC_GFF_OUTER);
+      if (op(OP_MOM_B, li)) {
+        if (at_mid_step) at_mid_step(li);
+        source_moments(li, ld[li].momA[parity[li]], nullptr, SRC_GFF_OUTER);
+      }
       if (op(OP_GFC_B, li + 1)) fill_gfc(li + 1, true, false);
     }
     // the remaining substeps (one in acoustic scaling; three with diffusive
@@ -498,7 +505,7 @@ const lbm_ctx::StepGraph* lbm_ctx::step_graph(int nsteps) {
   }
   // levels batched by instant (up to kMaxBatch of them); without branch
   // streams, or with more levels, the captured steps are the recursion's
-  const bool batched = n_filled <= kMaxBatch && make_branches();
+  const bool batched = can_batch();
   // capture on a private stream (the bound stream may be the legacy default
   // stream, which cannot be captured); host bookkeeping is restored afterwards
   const std::vector<int> p0 = parity;
@@ -730,6 +737,7 @@ lbm_status lbm_bind(lbm_ctx* c, void* ws, uint64_t bytes, void* stream) {
   c->drop_graphs();  // captured steps point into the previous workspace
   c->ws = static_cast<char*>(ws);
   c->st = static_cast<cudaStream_t>(stream);
+  c->reset_state_buffers();
   const HostMesh& m = c->M;
   auto up = [&](size_t off, const void* src, size_t b) -> lbm_status {
     if (b == 0) return LBM_OK;

@@ -1029,6 +1029,23 @@ __global__ void k_outlet(const __grid_constant__ OutletArgs a) {
 #endif
 template <class S>
 constexpr int kMomBlock = sizeof(S) == 8 ? 32 : LBM_MOM_BLOCK;  // FP64: one warp, as kScBlock
+// pdfs of source k (element e): from the state, or as set aside
+template <int Q, class S>
+__device__ __forceinline__ void load_source(const SavedSources& sv, const S* src, size_t N, int64_t e, int64_t k,
+                                            typename Sto<S>::R (&g)[Q]) {
+  const S* p = src + e;
+  size_t pitch = N;
+  if (sv.values) {
+    const int32_t i = sv.index[k];
+    if (i >= 0) {
+      p = static_cast<const S*>(sv.values) + i;
+      pitch = (size_t)sv.n;
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < Q; ++q) g[q] = Sto<S>::ld(p + q * pitch);
+}
+
 template <int Q, class S, bool FORCE>
 __global__ void __launch_bounds__(kMomBlock<S>) k_source_moments(const __grid_constant__ MomentsArgs a) {
   using R = typename Sto<S>::R;
@@ -1041,8 +1058,7 @@ __global__ void __launch_bounds__(kMomBlock<S>) k_source_moments(const __grid_co
   const int64_t e = a.elem[k];
   const int64_t r = a.rec ? (int64_t)a.rec[k] : k;
   R g[Q];
-#pragma unroll
-  for (int q = 0; q < Q; ++q) g[q] = Sto<S>::ld(src + (size_t)q * N + e);
+  load_source<Q, S>(a.saved, src, N, e, k, g);
   R F[3] = {R(0), R(0), R(0)};
   if (FORCE)
 #pragma unroll

@@ -4,6 +4,7 @@
 
 #include <cuda_runtime_api.h>
 
+#include <array>
 #include <functional>
 #include <string>
 #include <vector>
@@ -65,6 +66,14 @@ struct lbm_ctx {
   char* ws = nullptr;
   cudaStream_t st = nullptr;
   std::vector<int> parity;
+  // the two buffers of every level's state, by parity: A and B of the
+  // workspace, except while the adjoint records steps into its tape
+  std::vector<std::array<void*, 2>> state;
+  void reset_state_buffers() { state.assign(nlev, {at(oA), at(oB)}); }
+  // recording (adjoint): where a level's next stream-collide writes its new
+  // state; and called when the fill at t + 1/2 reads a level's records at t + 1
+  std::function<void*(int level)> new_state;
+  std::function<void(int level)> at_mid_step;
   int64_t launches = 0;
   // optional mass check (params.check_every): coarse steps since the last
   // check, and the reference mass (taken at the first lbm_step after bind,
@@ -214,8 +223,8 @@ struct lbm_ctx {
   T* at(size_t off) const {
     return reinterpret_cast<T*>(ws + off);
   }
-  void* cur(int li) const { return parity[li] ? at(oB) : at(oA); }
-  void* nxt(int li) const { return parity[li] ? at(oA) : at(oB); }
+  void* cur(int li) const { return state[li][parity[li]]; }
+  void* nxt(int li) const { return state[li][parity[li] ^ 1]; }
   uint32_t parity_mask() const {
     uint32_t m = 0;
     for (int li = 0; li < nlev; ++li) m |= (uint32_t)(parity[li] & 1) << li;
@@ -260,8 +269,10 @@ struct lbm_ctx {
   enum { SRC_ALL = 0, SRC_GFF_OUTER = 1 };
   void fill_gfc(int li_fine, bool two_times, bool all_layers);
   void stream_collide(int li);
-  // one coarse step in a graph capture, the levels batched by instant
+  // one coarse step, the levels batched by instant (a graph capture, or
+  // launched at once where the adjoint records it)
   void step_batched();
+  bool can_batch() { return n_filled <= lbm::kMaxBatch && make_branches(); }
   void tick_batched(int l0, int n);
   int n_filled = 1;                  // levels up to the finest one with elements
   bool outlet_reads_ghosts = false;  // a boundary value reads a ghost's pdfs

@@ -299,12 +299,21 @@ struct OutletArgs {  // links begin .. end of the last level, levels in order
 // type): f^neq[Q] padded to a multiple of 4, rho - rho_off, u[d], S[nS], zero
 // padding.
 constexpr int mom_stride(int Q) { return Q == 27 ? 40 : 32; }
+// Pdfs of the GhostFromFiner sources set aside before their next fill (the
+// adjoint's tape): values[q n + index[k]] for record k, where index[k] >= 0.
+// values null: every source is read from the state.
+struct SavedSources {
+  const void* values;
+  const int32_t* index;
+  int64_t n;
+};
 struct MomentsArgs {
   const void* src;
   const void* force;
   const int32_t* elem;
   void* mom;         // [nsrc][mom_stride(Q)]
   const void* prev;  // if set: mom = (prev + moments now) / 2 (mean of two time levels)
+  SavedSources saved;
   const int32_t* rec;  // record index of elem[k] (null: k)
   int64_t Ntot, nsrc;
   double rho_off;
@@ -535,6 +544,7 @@ struct AdjOutletArgs {
 struct AdjMomArgs {  // reverse of the source records
   AdjCommon c;       // lam_b: adjoint of the coarse state
   const int32_t* elem;
+  SavedSources saved;
   const void* contrib;  // what k_adj_gfc left per ghost
   const int32_t* off;   // [nsrc+1] transposed source list
   const int32_t* item;  // ghost*4 + source slot
@@ -596,6 +606,12 @@ const AdjOps* adj_ops_fp64();
 const AdjOps* adj_ops_fp32dev();
 const AdjOps* adj_ops_bf16dev();
 void launch_accum(const AccumArgs&, cudaStream_t);
+// GhostFromCoarser slots first .. first + ng of dst: those of inner, or outer for the outer layer (oct & kGfcOuter)
+void launch_copy_ghosts(const void* inner, const void* outer, void* dst, const uint8_t* oct, int64_t first, int64_t ng,
+                        int64_t pitch, int Q, size_t size, cudaStream_t);
+// dst[q n + k] = src[q pitch + elem[k]] for q < Q, values of `size` bytes
+void launch_gather_elements(const void* src, void* dst, const int32_t* elem, int64_t n, int64_t pitch, int Q, size_t size,
+                            cudaStream_t);
 // Copies bytes [off, off + len) of each of `rows` rows of pitch `pitch` from
 // src to dst (same layout); elem is the element size the offsets are multiples of.
 void launch_copy_rows(const void* src, void* dst, size_t pitch, size_t off, size_t len, int rows, size_t elem,
