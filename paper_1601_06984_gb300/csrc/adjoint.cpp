@@ -219,6 +219,10 @@ lbm_status lbm_set_params(lbm_ctx* c, double omega_coarse, const double* u_in) {
   for (int li = 1; li < c->nlev; ++li) om[li] = finer_omega(om[li - 1], c->p.time_mode);
   for (int li = 0; li < c->nlev; ++li)
     if (std::fabs(1.0 - om[li]) < 1e-3) return c->fail(LBM_ERR_ARG, "omega too close to 1 on some level");
+  // the same values again (an optimisation loop over something else) change nothing
+  bool same = omega_coarse == c->p.omega_coarse;
+  for (int a = 0; u_in && a < 3; ++a) same = same && u_in[a] == c->p.u_in[a];
+  if (same) return LBM_OK;
   c->drop_graphs();  // captured steps carry the old omega and inlet values
   c->recs_valid = false;  // the source records depend on omega
   for (int li = 0; li < c->nlev; ++li) c->M.lv[li].omega = om[li];

@@ -703,14 +703,17 @@ template <int Q>
 constexpr int kGhostAdj = (Q + 3) / 4 * 4 + 4;
 
 // Reverse of the source records, one thread per source (64^3 two-level flow,
-// FP32: 16.1 us; the sum over four records' adjoints per ghost and the reverse
+// FP32: 12.5 us; the sum over four records' adjoints per ghost and the reverse
 // of the records as two kernels took 17.3 + 9.8 us): sums what its ghosts
 // leave for it (k_adj_gfc; fixed order: the transposed list), which is the
 // adjoint of its record, and takes it back to the source's pdfs.  LINEAR mode:
 // the record at t + 1/2 is the mean of those at t and t + 1; its reverse (half
 // set) applies half to the state at t + 1 and leaves half in rec_half, which
 // the reverse of the fill at t adds (rec_half without half).
-template <int Q, class S>
+// LANES consecutive lanes share a source's ghosts (about ten items, each a
+// chain of two loads), four where the sources alone would not fill the GPU:
+// 64^3 FP32 15.7 -> 12.5 us, D2Q9 FP64 with 450 sources 26 -> 17 us.
+template <int Q, class S, int LANES>
 __global__ void __launch_bounds__(sizeof(typename Sto<S>::R) == 8 ? 32 : 128) k_adj_moments(const __grid_constant__ AdjMomArgs a) {
   using R = typename Sto<S>::R;
   using RL = RecLayout<Q>;
@@ -721,14 +724,17 @@ __global__ void __launch_bounds__(sizeof(typename Sto<S>::R) == 8 ? 32 : 128) k_
   const size_t N = (size_t)a.c.Ntot;
   R part[1] = {R(0)};
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < a.nsrc; k += stride) {
+  // whole warps iterate together (the shuffles below)
+  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t - threadIdx.x % 32 < a.nsrc * LANES; t += stride) {
+    const int64_t k = t / LANES;
+    const bool active = k < a.nsrc;
     R lfn[Q], lS[NS], lu[3] = {R(0), R(0), R(0)}, lrp = R(0);
 #pragma unroll
     for (int q = 0; q < Q; ++q) lfn[q] = R(0);
 #pragma unroll
     for (int s = 0; s < NS; ++s) lS[s] = R(0);
-    const int j1 = a.off[k + 1];
-    for (int j = a.off[k]; j < j1; ++j) {
+    const int j1 = active ? a.off[k + 1] : 0;
+    for (int j = active ? a.off[k] + (int)(t % LANES) : 0; j < j1; j += LANES) {
       const int item = a.item[j], slot = item & 3, oct = (item >> 2) & ((1 << D) - 1);
       const R* __restrict__ v = ghosts + (size_t)(item >> 2) * CS;
       R h[CS];
@@ -760,6 +766,17 @@ __global__ void __launch_bounds__(sizeof(typename Sto<S>::R) == 8 ? 32 : 128) k_
         }
       }
     }
+#pragma unroll
+    for (int o = 1; o < LANES; o <<= 1) {
+#pragma unroll
+      for (int q = 0; q < Q; ++q) lfn[q] += __shfl_xor_sync(0xffffffffu, lfn[q], o);
+      lrp += __shfl_xor_sync(0xffffffffu, lrp, o);
+#pragma unroll
+      for (int b = 0; b < D; ++b) lu[b] += __shfl_xor_sync(0xffffffffu, lu[b], o);
+#pragma unroll
+      for (int s = 0; s < NS; ++s) lS[s] += __shfl_xor_sync(0xffffffffu, lS[s], o);
+    }
+    if (!active || t % LANES != 0) continue;
     if (a.rec_half) {
       R* __restrict__ half = static_cast<R*>(a.rec_half) + (size_t)k * RL::STRIDE;
       R rec[RL::STRIDE];
@@ -1030,8 +1047,13 @@ struct AdjLaunch {
   static constexpr int kGhostBlock = sizeof(typename Sto<S>::R) == 8 ? 32 : 128;
   static void moments(int Q, const AdjMomArgs& a, cudaStream_t st) {
     if (a.nsrc <= 0) return;
+    // four lanes a source up to a warp per SM (FP64, where the extra lanes are
+    // extra FP64 instructions) or four blocks per SM
+    const bool four = a.nsrc <= (kGhostBlock == 32 ? 152 * 32 : 152 * 4 * 128);
     with_q(Q, [&](auto q) {
-      k_adj_moments<decltype(q)::value, S><<<adj_grid(a.nsrc, kGhostBlock), kGhostBlock, 0, st>>>(a);
+      constexpr int QQ = decltype(q)::value;
+      if (four) k_adj_moments<QQ, S, 4><<<adj_grid(4 * a.nsrc, kGhostBlock), kGhostBlock, 0, st>>>(a);
+      else k_adj_moments<QQ, S, 1><<<adj_grid(a.nsrc, kGhostBlock), kGhostBlock, 0, st>>>(a);
     });
   }
   static void gfc(int Q, const AdjGfcArgs& a, cudaStream_t st) {
