@@ -3,6 +3,8 @@
 // transfers of the public calls.
 #include <cuda_runtime_api.h>
 
+#include <unistd.h>
+
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -1000,44 +1002,92 @@ lbm_status lbm_fill_ghosts(lbm_ctx* c) {
   return c->launched("fill_ghosts");
 }
 
+// Makes the pages of a large host output present, on all cores, while the GPU
+// works on the first chunk: a device-to-host copy into memory that was never
+// written stops at every page (64 KiB here) for the system to clear it, which
+// took 75 MB from 0.4 to 3.2 ms.  One byte of each page is written; the call
+// overwrites the whole array.
+static void touch_pages(void* p, size_t bytes) {
+  if (!p || bytes < ((size_t)4 << 20)) return;
+  const size_t page = (size_t)std::max(4096l, sysconf(_SC_PAGESIZE));
+  volatile char* b = static_cast<volatile char*>(p);
+  const int64_t n = (int64_t)((bytes + page - 1) / page);
+#pragma omp parallel for schedule(static)
+  for (int64_t k = 0; k < n; ++k) b[(size_t)k * page] = 0;
+}
+
 static lbm_status out_chunks(lbm_ctx* c, double* rho, double* u, double* S, double* f) {
-  const int64_t n = c->M.n_user, CH = c->chunk;
+  const int64_t n = c->M.n_user;
   const int d = c->d, nS = c->nS, Q = c->Q;
-  double* sr = c->at<double>(c->oStage);
-  double* su = sr + CH;
-  double* sS = su + CH * d;
-  double* sf = sS + CH * nS;
-  for (int64_t first = 0; first < n; first += CH) {
-    const int64_t cnt = std::min(CH, n - first);
-    OutArgs a{};
-    a.A = c->at(c->oA);
-    a.B = c->at(c->oB);
-    a.force = c->force_ptr();
-    a.uslot = c->at<int32_t>(c->oUslot);
-    a.ulev = c->at<uint8_t>(c->oUlev);
-    a.parity = c->parity_mask();
+  // Two halves of the staging area: the copy of one chunk to the host (on the
+  // copy stream) beside the kernel of the next, where the chunks' copies are
+  // long against the 10 us that each costs (moments of 1.5e5 D3Q19 elements in
+  // four chunks 268 us, in one 219; of 4.9e5 elements 424 and 609 us, of
+  // 1.08e7 5.4 ms in halves of the staging area and 12.5 in whole chunks, most
+  // of both from the kernel's fewer FP64 instructions).
+  const bool two = n >= (1 << 18) && c->copy_stream_ready();
+  const int64_t CH = two ? std::min((c->chunk + 1) / 2, std::max<int64_t>((n + 3) / 4, 1 << 17)) : c->chunk;
+  const int64_t per = 1 + d + nS + Q;  // staged doubles per element
+  cudaStream_t cs = two ? c->copy_st : c->st;
+  if (two) {
+    // the staging area may still be read by earlier work on the bound stream
+    cudaEventRecord(c->copy_ev[2], c->st);
+    cudaStreamWaitEvent(cs, c->copy_ev[2], 0);
+  }
+  OutArgs a{};
+  a.A = c->at(c->oA);
+  a.B = c->at(c->oB);
+  a.force = c->force_ptr();
+  a.uslot = c->at<int32_t>(c->oUslot);
+  a.ulev = c->at<uint8_t>(c->oUlev);
+  a.parity = c->parity_mask();
+  a.Ntot = c->M.Ntot;
+  for (int li = 0; li < c->nlev; ++li) a.rx[li] = make_relax(Q, c->M.lv[li].omega);
+  a.rho_off = c->rho_off;
+  lbm_status s = LBM_OK;
+  const int64_t chunks = (n + CH - 1) / CH;
+  auto stage = [&](int64_t i) { return c->at<double>(c->oStage) + (size_t)(two ? i & 1 : 0) * CH * per; };
+  auto compute = [&](int64_t i) {
+    // the half's previous copies are done
+    if (two && i >= 2) cudaStreamWaitEvent(c->st, c->copy_ev[i & 1], 0);
+    double* sr = stage(i);
     a.rho = rho ? sr : nullptr;
-    a.u = u ? su : nullptr;
-    a.S = S ? sS : nullptr;
-    a.f = f ? sf : nullptr;
-    a.first = first;
-    a.cnt = cnt;
-    a.Ntot = c->M.Ntot;
-    for (int li = 0; li < c->nlev; ++li) a.omega[li] = c->M.lv[li].omega;
-    a.rho_off = c->rho_off;
+    a.u = u ? sr + CH : nullptr;
+    a.S = S ? sr + CH * (1 + d) : nullptr;
+    a.f = f ? sr + CH * (1 + d + nS) : nullptr;
+    a.first = i * CH;
+    a.cnt = std::min(CH, n - a.first);
     c->ops->out(Q, a, c->st);
     ++c->launches;
-    lbm_status s = c->launched("output");
+    if (two) cudaEventRecord(c->copy_ev[2 + (i & 1)], c->st);
+  };
+  compute(0);
+  touch_pages(rho, (size_t)n * 8);
+  touch_pages(u, (size_t)n * d * 8);
+  touch_pages(S, (size_t)n * nS * 8);
+  touch_pages(f, (size_t)n * Q * 8);
+  for (int64_t i = 0; i < chunks && s == LBM_OK; ++i) {
+    // a copy to pageable memory may hold this thread, so the next chunk's
+    // kernel is launched before it
+    if (two && i + 1 < chunks) compute(i + 1);
+    if (two) cudaStreamWaitEvent(cs, c->copy_ev[2 + (i & 1)], 0);
+    const int64_t first = i * CH, cnt = std::min(CH, n - first);
+    const double* sr = stage(i);
     auto down = [&](double* dst, const double* src, size_t b) {
-      if (s == LBM_OK) s = c->cuda_check(cudaMemcpyAsync(dst, src, b, cudaMemcpyDeviceToHost, c->st), "output copy");
+      if (s == LBM_OK) s = c->cuda_check(cudaMemcpyAsync(dst, src, b, cudaMemcpyDeviceToHost, cs), "output copy");
     };
     if (rho) down(rho + first, sr, cnt * 8);
-    if (u) down(u + first * d, su, cnt * d * 8);
-    if (S) down(S + first * nS, sS, cnt * nS * 8);
-    if (f) down(f + first * Q, sf, cnt * Q * 8);
-    if (s != LBM_OK) return s;
+    if (u) down(u + first * d, sr + CH, cnt * d * 8);
+    if (S) down(S + first * nS, sr + CH * (1 + d), cnt * nS * 8);
+    if (f) down(f + first * Q, sr + CH * (1 + d + nS), cnt * Q * 8);
+    if (two) cudaEventRecord(c->copy_ev[i & 1], cs);
+    else if (i + 1 < chunks) compute(i + 1);
   }
-  return c->cuda_check(cudaStreamSynchronize(c->st), "output sync");
+  if (s == LBM_OK) s = c->launched("output");
+  // both streams idle: the staging area and the host arrays are free
+  const lbm_status e = c->cuda_check(cudaStreamSynchronize(c->st), "output sync");
+  const lbm_status e2 = c->cuda_check(cudaStreamSynchronize(cs), "output sync");
+  return s != LBM_OK ? s : e != LBM_OK ? e : e2;
 }
 
 lbm_status lbm_moments(lbm_ctx* c, double* rho, double* u, double* S) {

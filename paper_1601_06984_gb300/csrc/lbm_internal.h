@@ -423,7 +423,7 @@ struct OutArgs {  // moments / state to FP64 staging in user order
   uint32_t parity;
   double *rho, *u, *S, *f;  // staged chunk outputs (any may be null)
   int64_t first, cnt, Ntot;
-  double omega[16];
+  Relax rx[16];
   double rho_off;
 };
 
