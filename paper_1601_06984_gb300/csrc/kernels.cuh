@@ -1101,6 +1101,49 @@ __device__ __forceinline__ void compact_uloc(const R (&ul)[4][3], const R (&Sl)[
   }
 }
 
+// compact_uloc in FP64 with fewest instructions: the differences' factor 1/2
+// in the constants, two of the three differences of a component from the same
+// two half differences (3D: 83 instructions for 135).
+template <int Q>
+__device__ __forceinline__ void compact_uloc64(const double (&ul)[4][3], const double (&Sl)[4][Lat<Q>::NS],
+                                               double (&uloc)[3]) {
+  constexpr int D = Lat<Q>::D, NS = Lat<Q>::NS;
+  double x[NS], y[NS], z[NS];  // twice the differences
+#pragma unroll
+  for (int c = 0; c < NS; ++c) {
+    if (D == 3) {
+      const double a = Sl[1][c] - Sl[0][c], b = Sl[2][c] - Sl[3][c];
+      x[c] = a + b;
+      y[c] = a - b;
+      z[c] = (Sl[2][c] + Sl[3][c]) - (Sl[0][c] + Sl[1][c]);
+    } else {
+      const double a = Sl[1][c] - Sl[0][c], b = Sl[3][c] - Sl[2][c];
+      x[c] = b + a;
+      y[c] = (Sl[2][c] + Sl[3][c]) - (Sl[0][c] + Sl[1][c]);
+      z[c] = 0;
+    }
+  }
+  if (D == 3) {
+    constexpr int XX = 0, YY = 1, ZZ = 2, XY = 3, YZ = 4, XZ = NS - 1;
+    const double h = z[XY] + x[YZ] + y[XZ];
+    const double s1[3] = {x[XX] - x[YY] - x[ZZ], y[YY] - y[XX] - y[ZZ], z[ZZ] - z[XX] - z[YY]};
+    const double s2[3] = {y[XY] + z[XZ], x[XY] + z[YZ], x[XZ] + y[YZ]};
+    const double s3[3] = {fma(-2.0, x[YZ], y[XX] + z[XX] + h), fma(-2.0, y[XZ], x[YY] + z[YY] + h),
+                          fma(-2.0, z[XY], x[ZZ] + y[ZZ] + h)};
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      const double us = fma(5.0, ul[0][b], ul[1][b]) + (ul[2][b] + ul[3][b]);
+      uloc[b] = fma(-0.03125, s3[b], fma(-0.09375, s2[b], fma(-0.046875, s1[b], 0.125 * us)));
+    }
+  } else {
+    uloc[0] = fma(0.03125, y[0], fma(-0.09375, y[2], fma(-0.046875, x[0] - x[1],
+                  fma(0.5, ul[0][0], 0.25 * (ul[1][0] + ul[2][0])))));
+    uloc[1] = fma(0.03125, x[1], fma(-0.09375, x[2], fma(-0.046875, y[1] - y[0],
+                  fma(0.5, ul[0][1], 0.25 * (ul[1][1] + ul[2][1])))));
+    uloc[2] = 0;
+  }
+}
+
 // ----------------------------------------------------------------- GhostFromCoarser
 // Interpolation steps 2-5 (Sec. 2.2) for one fine ghost from its four coarse
 // sources.  The velocity is the compact quadratic interpolant evaluated at the
@@ -1145,7 +1188,7 @@ struct GfcGroup {
 // staged records (sg_base: NSLOT padded records), written into L.dst.
 template <int Q, class S>
 __device__ __forceinline__ void gfc_ghost(const GfcArgs& a, const GfcLevel& L, const typename Sto<S>::R* sg_base, int oct,
-                                          int64_t k) {
+                                          int64_t k, bool two) {
   using R = typename Sto<S>::R;
   using LT = Lat<Q>;
   using RL = RecLayout<Q>;
@@ -1184,11 +1227,17 @@ __device__ __forceinline__ void gfc_ghost(const GfcArgs& a, const GfcLevel& L, c
       }
   }
   R uloc[3];
-  compact_uloc<Q, R>(ul, Sl, uloc);
+  if constexpr (sizeof(R) == 8) compact_uloc64<Q>(ul, Sl, uloc);
+  else compact_uloc<Q, R>(ul, Sl, uloc);
   R u[3] = {R(0), R(0), R(0)};
   R usq = R(0);
   const auto& un = pick<R>(a.u64, a.u32);
-  const R us = un.u_scale;  // to fine lattice units (1 in acoustic scaling)
+  // FP64 at t + 1/2: the staged records are the sums of the two times';
+  // everything taken from them is linear, and the half goes, exactly, into
+  // its factors
+  [[maybe_unused]] const R half = two ? R(0.5) : R(1);
+  R us = un.u_scale;  // to fine lattice units (1 in acoustic scaling)
+  if constexpr (sizeof(R) == 8) us *= half;
 #pragma unroll
   for (int b = 0; b < D; ++b) {
     u[b] = sg[b] * uloc[b] * us;
@@ -1198,9 +1247,13 @@ __device__ __forceinline__ void gfc_ghost(const GfcArgs& a, const GfcLevel& L, c
   const R lw1 = D == 3 ? R(0.125) : R(0.1875);
   const R lw2 = D == 3 ? R(0.125) : R(0.1875);
   const R lw3 = D == 3 ? R(0.125) : R(0.0625);
-  const R rp = un.r_scale * (lw0 * rps[0] + lw1 * rps[1] + lw2 * rps[2] + lw3 * rps[3]) + un.r_shift;
+  R rs = un.r_scale, scale = pick<R>(L.scale, L.scale32);
+  if constexpr (sizeof(R) == 8) {
+    rs *= half;
+    scale *= D == 3 ? 0.125 * half : half;
+  }
+  const R rp = rs * (lw0 * rps[0] + lw1 * rps[1] + lw2 * rps[2] + lw3 * rps[3]) + un.r_shift;
   const R rho = un.rho_off + rp;
-  const R scale = pick<R>(L.scale, L.scale32);
   S* __restrict__ dst = static_cast<S*>(L.dst);
   const size_t N = (size_t)a.Ntot;
   const int64_t e = L.dest0 + k;
@@ -1215,7 +1268,11 @@ __device__ __forceinline__ void gfc_ghost(const GfcArgs& a, const GfcLevel& L, c
     ld4(rec[3] + RL::FN + q0, f3);
 #pragma unroll
     for (int c = 0; c < 4; ++c)
-      if (q0 + c < Q) fn[q0 + c] = lw0 * f0[c] + lw1 * f1[c] + lw2 * f2[c] + lw3 * f3[c];
+      if (q0 + c < Q) {
+        // FP64, 3D: 8 times the interpolated value, in three instructions
+        if constexpr (sizeof(R) == 8 && D == 3) fn[q0 + c] = fma(5.0, f0[c], f1[c]) + (f2[c] + f3[c]);
+        else fn[q0 + c] = lw0 * f0[c] + lw1 * f1[c] + lw2 * f2[c] + lw3 * f3[c];
+      }
   }
   const R base = rp - R(1.5) * rho * usq;
   dst[e] = Sto<S>::cv(R(LT::w(0)) * base + scale * fn[0]);
@@ -1230,17 +1287,22 @@ __device__ __forceinline__ void gfc_ghost(const GfcArgs& a, const GfcLevel& L, c
       if (LT::c(i, b) > 0) cu += u[b];
       if (LT::c(i, b) < 0) cu -= u[b];
     }
-    const R w = R(LT::w(i));
-    R even, odd;
     if constexpr (sizeof(R) == 8) {
-      // w base and w rho are shared by all directions of a weight
-      const double wr = w * rho, t = wr * cu;
-      odd = 3.0 * t;
-      even = fma(4.5 * t, cu, w * base);
-    } else {
-      even = w * (base + R(4.5) * rho * cu * cu);
-      odd = w * R(3) * rho * cu;
+      double fa = fn[i], fb = fn[i + 1];
+      if (odd_rescale) {
+        const double fe = 0.5 * (fa + fb), fo = 0.5 * (fa - fb) * ro;
+        fa = fe + fo;
+        fb = fe - fo;
+      }
+      // the products with a weight are shared by all its directions
+      const double w = LT::w(i), wr = 3.0 * w * rho, even = fma((4.5 * w * rho) * cu, cu, w * base);
+      dst[(size_t)i * N + e] = fma(scale, fa, fma(wr, cu, even));
+      dst[(size_t)(i + 1) * N + e] = fma(scale, fb, fma(-wr, cu, even));
+      continue;
     }
+    const R w = R(LT::w(i));
+    const R even = w * (base + R(4.5) * rho * cu * cu);
+    const R odd = w * R(3) * rho * cu;
     R fa = fn[i], fb = fn[i + 1];
     if (odd_rescale) {
       const R fe = R(0.5) * (fa + fb), fo = R(0.5) * (fa - fb) * ro;
@@ -1301,7 +1363,8 @@ __global__ void __launch_bounds__(kGfcBlock<S>) k_fill_gfc(const __grid_constant
           ld4(mom + (size_t)r[t - t0] * RL::STRIDE + 4 * (oct + c * G), v[t - t0][c]);
     }
     if (TWO && two) {
-      // the records at t + 1/2: mean of those at t and t + 1
+      // the records at t + 1/2: the means of those at t and t + 1 (FP64: the
+      // sums, gfc_ghost takes the half)
       R w[BATCH][CH][4];
 #pragma unroll
       for (int t = t0; t < t0 + BATCH && t < NSLOT; ++t)
@@ -1314,7 +1377,8 @@ __global__ void __launch_bounds__(kGfcBlock<S>) k_fill_gfc(const __grid_constant
 #pragma unroll
         for (int c = 0; c < CH; ++c)
 #pragma unroll
-          for (int j = 0; j < 4; ++j) v[t - t0][c][j] = R(0.5) * (v[t - t0][c][j] + w[t - t0][c][j]);
+          for (int j = 0; j < 4; ++j)
+            v[t - t0][c][j] = sizeof(R) == 8 ? v[t - t0][c][j] + w[t - t0][c][j] : R(0.5) * (v[t - t0][c][j] + w[t - t0][c][j]);
     }
 #pragma unroll
     for (int t = t0; t < t0 + BATCH && t < NSLOT; ++t)
@@ -1326,7 +1390,7 @@ __global__ void __launch_bounds__(kGfcBlock<S>) k_fill_gfc(const __grid_constant
   let_next_start();
   // outer-layer ghosts are staged with their group but, when skipped, not written
   if (!active || (L.skip_outer && (L.oct[k] & kGfcOuter))) return;
-  gfc_ghost<Q, S>(a, L, sg_base, oct, k);
+  gfc_ghost<Q, S>(a, L, sg_base, oct, k, TWO && two);
 }
 
 // ----------------------------------------------------------------- GhostFromFiner
