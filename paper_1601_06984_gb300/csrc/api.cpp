@@ -941,11 +941,13 @@ static lbm_status step_run(lbm_ctx* c, int64_t n_coarse) {
   int64_t k = 0;
   if (n_coarse > 0) c->ensure_records();  // outside any capture
   // pairs of coarse steps replay a captured two-step graph and a remaining
-  // single step a one-step graph; timed steps (mode 1) and the adjoint's
-  // recorded steps are issued one kernel at a time
+  // single step a one-step graph (small meshes, later, longer ones); timed
+  // steps (mode 1) are issued one kernel at a time
   if (c->graphs_on && c->timing != 1 && !c->hook && !c->dry) {
     while (k < n_coarse) {
-      const lbm_ctx::StepGraph* g = c->step_graph(n_coarse - k >= 2 ? 2 : 1);
+      const int64_t left = n_coarse - k;
+      const bool longer = left >= kLongGraphSteps && c->long_graphs();
+      const lbm_ctx::StepGraph* g = c->step_graph(longer ? kLongGraphSteps : left >= 2 ? 2 : 1);
       if (!g) break;
       lbm_status s = c->cuda_check(cudaGraphLaunch(g->exec, c->st), "graph launch");
       if (s != LBM_OK) return s;
@@ -953,6 +955,7 @@ static lbm_status step_run(lbm_ctx* c, int64_t n_coarse) {
       c->parity = g->end;
       c->last_graph = (int)(g - c->graphs.data());
       c->graph_unread = true;
+      c->graph_steps += g->steps;
       k += g->steps;
     }
   }

@@ -30,6 +30,15 @@ constexpr int64_t kChainElements = 1 << 20, kChainElements64 = 1 << 12;
 // 57.3, two-level 64^3 44.9 / 45.7, D3Q27 9e5 elements 131 / 132; beyond it the
 // sphere of 1.1e7 elements took 7.4 against 4.94 ms).
 constexpr int64_t kBesideElements = 1 << 20;
+// A graph launch costs about 3.5 us between two replays, 4 to 5% of a step of a
+// small mesh with two steps a graph.  Once a context has replayed
+// kLongGraphAfter steps (so that a short run pays for no longer capture) and
+// has at most kLongGraphUpdates updates a coarse step, it replays graphs of
+// kLongGraphSteps: us per call, with its output, D2Q9 channel FP64, 50 steps
+// 2003 -> 1879, cylinder, 50 steps 2745 -> 2601, two-level 64^3, 200 steps 8870
+// -> 8620, D2Q9 32x32 FP64, 20 steps 811 -> 792.
+constexpr int kLongGraphSteps = 16;
+constexpr int64_t kLongGraphAfter = 64, kLongGraphUpdates = 1 << 21;
 // Kernel kinds of the per-launch timing (lbm_timing_read row kTimedKinds * L + kind)
 enum TimedKind { TK_INTERIOR = 0, TK_LIST = 1, TK_BOUNDARY = 2, TK_GFF = 3, TK_MOM = 4, TK_GFC = 5, TK_OUTLET = 6,
                  TK_SC_SPAN = 7 };
@@ -190,6 +199,12 @@ struct lbm_ctx {
     return copy_st != nullptr;
   }
   bool graphs_on = true;
+  int64_t graph_steps = 0;  // replayed since the graphs were last dropped
+  bool long_graphs() const {
+    int64_t updates = 0, per = 1;
+    for (int li = 0; li < nlev; ++li, per *= lbm::time_ratio(p.time_mode)) updates += M.lv[li].nF * per;
+    return timing == 0 && graph_steps >= lbm::kLongGraphAfter && updates <= lbm::kLongGraphUpdates;
+  }
   int last_graph = -1;        // graph of the most recent replay
   bool graph_unread = false;  // its events hold a replay not yet read
   void drop_graphs() {
@@ -201,6 +216,7 @@ struct lbm_ctx {
       }
     }
     graphs.clear();
+    graph_steps = 0;
     last_graph = -1;
     graph_unread = false;
   }
@@ -283,7 +299,7 @@ struct lbm_ctx {
     ensure_records();
     advance(0);
   }
-  // graph of nsteps (1 or 2) coarse steps from the current parity state,
+  // graph of nsteps (1, or an even number) coarse steps from the current parity state,
   // captured on first use; null when capture is unavailable (the caller
   // steps eagerly)
   const StepGraph* step_graph(int nsteps);
