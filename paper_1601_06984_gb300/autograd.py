@@ -26,7 +26,7 @@ class MultilevelLBM(torch.autograd.Function):
     def forward(ctx, force, omega_c, u_in, sim, init, n_coarse, K, objective):
         sim.set_params(float(omega_c), [float(x) for x in u_in.detach().cpu().tolist()])
         sim.init(*init)
-        sim.set_force(force.detach().cpu().numpy())
+        sim.set_force(force.detach().to("cpu", torch.float64).numpy())
         needs = any(ctx.needs_input_grad[:3])
         if needs:
             J, dF, dw, du = sim.adjoint(n_coarse, K, objective)

@@ -75,6 +75,11 @@ struct lbm_ctx {
   char* ws = nullptr;
   cudaStream_t st = nullptr;
   std::vector<int> parity;
+  // per level, built by the first lbm_adjoint (build_source_lists)
+  struct SourceLists {
+    std::vector<int32_t> off, item, saved;
+  };
+  std::vector<SourceLists> source_lists;
   // the two buffers of every level's state, by parity: A and B of the
   // workspace, except while the adjoint records steps into its tape
   std::vector<std::array<void*, 2>> state;
