@@ -325,7 +325,7 @@ def run_gpu(mesh, Q, om, uin, fields, prec, K, W_, device, dist=None, want_momen
     step_bytes = float(sum(msub ** li * (brick_units[li] * bytes_per_update(Q, prec, brick=True)
                                         + (info[li, 1] - brick_units[li]) * bytes_per_update(Q, prec))
                            for li in range(nlev)))
-    # the finest level's stream-collide as one op: its three kernels run as
+    # the finest level's stream-collide as one op: its two kernels run as
     # parallel graph branches, timed from fork to join (timing kind 7)
     span_ms = kms[finest, 7] / nl[finest, 7] if timing == 2 and nl[finest, 7] > 0 else None
     sc_bytes = (units * bpu + bnd_units * bytes_per_update(Q, prec, brick=True)
@@ -334,7 +334,7 @@ def run_gpu(mesh, Q, om, uin, fields, prec, K, W_, device, dist=None, want_momen
               "gbs": sc_bytes / (span_ms * 1e-3) / 1e9 if span_ms else None}
     res = {"ms_total": ms, "ms_per_step": ms / K, "mlups": K * U / (ms * 1e-3) / 1e6, "launches": launches,
            "finest_sc": res_sc,
-           "finest_kernel": "k_stream_collide_brick" if kb == 0 else "k_stream_collide",
+           "finest_kernel": "k_sc_interior" if kb == 0 else "k_sc_rest",
            "finest_launch_ms": avg_ms, "finest_launches": int(nl[finest, kb]), "finest_units": units,
            "finest_bytes": units * bpu, "finest_gbs": units * bpu / (avg_ms * 1e-3) / 1e9 if timed else None,
            "finest_list_units": list_units, "finest_list_launch_ms": list_ms,
@@ -769,11 +769,12 @@ def main():
         "roofline": {"bound": "hbm", "achieved": sc["gbs"], "peak": peak, "unit": "GB/s",
                      "frac": sc["gbs"] / peak,
                      "traffic": traffic,
-                     "traffic_source": "ncu DRAM bytes per unit of each of the three kernels (half-scale sphere "
+                     "traffic_source": "ncu DRAM bytes per unit of each kind of element (half-scale sphere "
                                        "capture, profiles/stream_collide_brick_fp32_sphere.md) times its units",
-                     "kernel": "finest-level stream-collide: k_stream_collide_brick<19,float> on the interior and "
-                               "boundary bricks and k_stream_collide<19,float> on the other elements, run as "
-                               "parallel branches of the captured step graph",
+                     "kernel": "finest-level stream-collide: k_sc_interior<19,float> on the interior bricks and "
+                               "k_sc_rest<19,float> on the boundary bricks and the other elements, run as "
+                               "parallel branches of the captured step graph (timed where the finest level "
+                               "advances alone)",
                      "units_per_launch": sc["units"], "bytes_per_unit": sc["bytes"] / sc["units"],
                      "avg_launch_ms": sc["span_ms"], "launches_averaged": r["finest_launches"],
                      "interior_kernel": {"units": r["finest_units"], "bytes_per_unit": r["bytes_per_update"],

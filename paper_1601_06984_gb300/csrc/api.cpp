@@ -488,8 +488,11 @@ void lbm_ctx::advance(int li) {
 bool lbm_ctx::make_branches() {
   if (br.s[0]) return br.ok;
   br.ok = true;
+  int least = 0, greatest = 0;
+  cudaDeviceGetStreamPriorityRange(&least, &greatest);
   for (int b = 0; b < 2; ++b) {
-    br.ok = br.ok && cudaStreamCreateWithFlags(&br.s[b], cudaStreamNonBlocking) == cudaSuccess;
+    br.ok = br.ok &&
+            cudaStreamCreateWithPriority(&br.s[b], cudaStreamNonBlocking, b == 0 ? least : greatest) == cudaSuccess;
     for (cudaEvent_t* e : {&br.fork[b], &br.join[b]})
       br.ok = br.ok && cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess;
   }
@@ -500,7 +503,9 @@ bool lbm_ctx::make_branches() {
 const lbm_ctx::StepGraph* lbm_ctx::step_graph(int nsteps) {
   for (const StepGraph& g : graphs)
     if (g.parity == parity && g.steps == nsteps) return &g;
-  if (!cap_stream && cudaStreamCreateWithFlags(&cap_stream, cudaStreamNonBlocking) != cudaSuccess) {
+  int least = 0, greatest = 0;
+  cudaDeviceGetStreamPriorityRange(&least, &greatest);
+  if (!cap_stream && cudaStreamCreateWithPriority(&cap_stream, cudaStreamNonBlocking, greatest) != cudaSuccess) {
     cudaGetLastError();
     graphs_on = false;
     return nullptr;
@@ -548,7 +553,7 @@ const lbm_ctx::StepGraph* lbm_ctx::step_graph(int nsteps) {
   const bool same = p1 == expect;
   parity = p0;
   cudaGraphExec_t exec = nullptr;
-  if (e == cudaSuccess && graph && same) e = cudaGraphInstantiate(&exec, graph, 0);
+  if (e == cudaSuccess && graph && same) e = cudaGraphInstantiate(&exec, graph, batched && prioritised() ? cudaGraphInstantiateFlagUseNodePriority : 0);
   if (graph) cudaGraphDestroy(graph);
   if (e != cudaSuccess || !exec || !same) {
     cudaGetLastError();

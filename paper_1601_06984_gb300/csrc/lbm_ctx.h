@@ -30,6 +30,12 @@ constexpr int64_t kChainElements = 1 << 20, kChainElements64 = 1 << 12;
 // 57.3, two-level 64^3 44.9 / 45.7, D3Q27 9e5 elements 131 / 132; beyond it the
 // sphere of 1.1e7 elements took 7.4 against 4.94 ms).
 constexpr int64_t kBesideElements = 1 << 20;
+// Graphs of meshes within kBesideElements give the interior bricks the least
+// priority and the chain of fills and the rest the greatest: its blocks, on
+// the critical path, start before the waiting bricks' (two-level 64^3 FP32 8510
+// -> 7930 us for 200 steps; others within 0.5%).  Beyond it the mixture slows
+// the bricks (sphere of 1.1e7 elements 4.97 -> 5.38 ms a step).
+//
 // A graph launch costs about 3.5 us between two replays, 4 to 5% of a step of a
 // small mesh with two steps a graph.  Once a context has replayed
 // kLongGraphAfter steps (so that a short run pays for no longer capture) and
@@ -202,6 +208,11 @@ struct lbm_ctx {
       }
     }
     return copy_st != nullptr;
+  }
+  bool prioritised() const {
+    int64_t n = 0;
+    for (const lbm::HostLevel& H : M.lv) n += H.nF;
+    return n <= lbm::kBesideElements;
   }
   bool graphs_on = true;
   int64_t graph_steps = 0;  // replayed since the graphs were last dropped
