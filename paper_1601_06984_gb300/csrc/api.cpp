@@ -578,37 +578,35 @@ lbm_status reduce_plan(lbm_ctx* c, ReducePlan* plan) {
   plan->Q = c->Q;
   plan->stream = c->st;
   plan->workspace = c->ws;
-  plan->levels.clear();
+  ReduceArgs& a = plan->args;
+  a = ReduceArgs{};
+  a.force = c->force_ptr();
+  a.Ntot = c->M.Ntot;
+  a.rho_off = c->rho_off;
+  a.rho0 = c->p.rho0;
+  a.nseg = c->nlev;
   const int d = c->d;
   for (int li = 0; li < c->nlev; ++li) {
     const HostLevel& H = c->M.lv[li];
-    ReduceArgs a{};
-    a.pdf = c->cur(li);
-    a.force = c->force_ptr();
-    a.Ntot = c->M.Ntot;
-    a.begin = H.base + H.oF;
-    a.end = H.base + H.oF + H.nF;
-    a.omega = H.omega;
-    a.rho_off = c->rho_off;
-    a.vol = std::ldexp(1.0, -d * li);
+    ReduceLevel& l = a.lev[li];
+    l.pdf = c->cur(li);
+    l.begin = H.base + H.oF;
+    l.end = H.base + H.oF + H.nF;
+    l.vol = std::ldexp(1.0, -d * li);
     // diffusive scaling: mass, momentum and kinetic energy in the coarsest
     // level's units (a lattice velocity of level li is 2^li of the
     // coarsest's), forces in the finest level's (a force unit goes with
     // dx^(d+1) / dt^2)
     const double us = 1.0 / level_velocity_ratio(li, c->p.time_mode);
-    a.vol_m = a.vol * us;
-    a.vol_k = a.vol * us * us;
-    a.r_scale = us * us;
-    a.rho0 = c->p.rho0;
-    a.partial = nullptr;
-    a.nblocks = kReduceBlocks;
-    a.obs_elem = c->at<int32_t>(c->oObsElem) + H.obs_begin;
-    a.obs_dir = c->at<int8_t>(c->oObsDir) + H.obs_begin;
-    a.obs_a = c->at<int32_t>(c->oObsA) + H.obs_begin;
-    a.obs_q = c->at<double>(c->oObsQ) + H.obs_begin;
-    a.obs_n = H.obs_end - H.obs_begin;
-    a.fscale = std::ldexp(1.0, (c->p.time_mode == LBM_TIME_DIFFUSIVE ? d - 3 : d - 1) * (c->nlev - 1 - li));
-    plan->levels.push_back(a);
+    l.vol_m = l.vol * us;
+    l.vol_k = l.vol * us * us;
+    l.r_scale = us * us;
+    l.obs_elem = c->at<int32_t>(c->oObsElem) + H.obs_begin;
+    l.obs_dir = c->at<int8_t>(c->oObsDir) + H.obs_begin;
+    l.obs_a = c->at<int32_t>(c->oObsA) + H.obs_begin;
+    l.obs_q = c->at<double>(c->oObsQ) + H.obs_begin;
+    l.obs_n = H.obs_end - H.obs_begin;
+    l.fscale = std::ldexp(1.0, (c->p.time_mode == LBM_TIME_DIFFUSIVE ? d - 3 : d - 1) * (c->nlev - 1 - li));
   }
   return LBM_OK;
 }
@@ -745,6 +743,7 @@ lbm_status lbm_bind(lbm_ctx* c, void* ws, uint64_t bytes, void* stream) {
   c->ws = static_cast<char*>(ws);
   c->st = static_cast<cudaStream_t>(stream);
   c->reset_state_buffers();
+  c->pinned_result();
   const HostMesh& m = c->M;
   auto up = [&](size_t off, const void* src, size_t b) -> lbm_status {
     if (b == 0) return LBM_OK;
@@ -898,18 +897,19 @@ static lbm_status reduce_to_host(lbm_ctx* c, double out[8]) {
   ReducePlan plan;
   lbm_status ps = reduce_plan(c, &plan);
   if (ps != LBM_OK) return ps;
-  for (int li = 0; li < c->nlev; ++li) {
-    ReduceArgs a = plan.levels[li];
-    a.partial = c->at<double>(c->oPartial) + (size_t)li * kReduceBlocks * 8;
-    c->ops->reduce(c->Q, a, c->st);
-    ++c->launches;
-  }
-  FinalArgs fa{c->at<double>(c->oPartial), (int64_t)c->nlev * kReduceBlocks, c->at<double>(c->oRed)};
+  plan.args.partial = c->at<double>(c->oPartial);
+  const unsigned rows = c->ops->reduce(c->Q, plan.args, c->st);
+  // the result goes straight to pinned host memory (a copy of 64 bytes costs
+  // about 8 us more), or through the workspace where there is none
+  double* pinned = c->result_host;
+  FinalArgs fa{c->at<double>(c->oPartial), (int64_t)rows, pinned ? pinned : c->at<double>(c->oRed)};
   launch_final_reduce(fa, c->st);
-  ++c->launches;
+  c->launches += c->nlev + 1;  // a level's reduction counts as a kernel
   lbm_status s = c->launched("reduce");
-  if (s == LBM_OK) s = c->cuda_check(cudaMemcpyAsync(out, c->at(c->oRed), 64, cudaMemcpyDeviceToHost, c->st), "reduce copy");
+  if (s == LBM_OK && !pinned)
+    s = c->cuda_check(cudaMemcpyAsync(out, c->at(c->oRed), 64, cudaMemcpyDeviceToHost, c->st), "reduce copy");
   if (s == LBM_OK) s = c->cuda_check(cudaStreamSynchronize(c->st), "reduce sync");
+  if (s == LBM_OK && pinned) std::memcpy(out, pinned, 64);
   return s;
 }
 

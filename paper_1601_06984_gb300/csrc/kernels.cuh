@@ -15,6 +15,7 @@
 #pragma once
 
 #include <cuda_bf16.h>
+#include <algorithm>
 #include <type_traits>
 #include <cuda_runtime.h>
 
@@ -1718,23 +1719,26 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-template <int NV>
-__device__ __forceinline__ void block_sum_store(double (&v)[NV], double* out) {
-  __shared__ double sh[NV][32];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+// Block sums of the threads' values v[0..NV) where bit k of `used` is set
+// (uniform), out[k] = 0 elsewhere: one warp per value, NV (threads / 32 + 5)
+// FP64 instructions a block (in every warp: 4 times as many, on the narrow
+// FP64 pipe, 11 us for a launch of 512 blocks of 256 threads).
+template <int NV, int BLOCK>
+__device__ __forceinline__ void block_sum_store(const double (&v)[NV], double* out, unsigned used) {
+  __shared__ double sh[NV][BLOCK];
 #pragma unroll
-  for (int c = 0; c < NV; ++c) {
-    const double s = warp_sum(v[c]);
-    if (lane == 0) sh[c][wid] = s;
-  }
+  for (int k = 0; k < NV; ++k)
+    if ((used >> k) & 1u) sh[k][threadIdx.x] = v[k];
   __syncthreads();
-  if (wid == 0) {
+  const int lane = threadIdx.x & 31;
+  for (int k = threadIdx.x >> 5; k < NV; k += BLOCK / 32) {
+    double s = 0.0;
+    if ((used >> k) & 1u) {
 #pragma unroll
-    for (int c = 0; c < NV; ++c) {
-      double s = lane < nw ? sh[c][lane] : 0.0;
+      for (int t = 0; t < BLOCK; t += 32) s += sh[k][t + lane];
       s = warp_sum(s);
-      if (lane == 0) out[c] = s;
     }
+    if (lane == 0) out[k] = s;
   }
 }
 
@@ -1754,18 +1758,27 @@ struct SumF2 {
 };
 
 // mass, momentum, obstacle force (momentum exchange, Sec. 2.3) and kinetic energy
-// of one level; one partial row per block, fixed grid -> deterministic order.
+// of all levels; one partial row per block, grid fixed by the mesh ->
+// deterministic order.  One launch with blocks for the elements there are (one
+// of 512 blocks per level before: 50 us of kernels for the four-level D2Q9
+// cylinder, where the blocks' sums alone bound it).
 // A thread sums its elements' moments (FP32 compute type: as two-float sums,
 // which keeps the FP64 pipe, GB300's narrow one, out of the per-element work;
 // FP64 storage: in FP64), then the block and grid sums are FP64.
+template <class S>
+constexpr int kRedBlock = sizeof(S) == 8 ? 128 : 256;
 template <int Q, class S>
-__global__ void __launch_bounds__(256) k_reduce(const ReduceArgs a) {
+__global__ void __launch_bounds__(kRedBlock<S>) k_reduce(const __grid_constant__ ReduceArgs a) {
   using LT = Lat<Q>;
   constexpr int D = LT::D;
   double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  const S* p = static_cast<const S*>(a.pdf);
+  const int seg = segment_of(a.first, a.nseg, blockIdx.x);
+  const ReduceLevel& L = a.lev[seg];
+  const unsigned blocks = (seg + 1 < a.nseg ? a.first[seg + 1] : gridDim.x) - a.first[seg];
+  const int64_t t0 = (int64_t)(blockIdx.x - a.first[seg]) * kRedBlock<S> + threadIdx.x;
+  const S* p = static_cast<const S*>(L.pdf);
   const size_t N = (size_t)a.Ntot;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  const int64_t stride = (int64_t)blocks * kRedBlock<S>;
   // each element's moments in the storage's compute type (the sums of its Q
   // stored values); the accumulation over elements in FP64
   // (the level volume and rho_off are applied once per thread below)
@@ -1773,12 +1786,13 @@ __global__ void __launch_bounds__(256) k_reduce(const ReduceArgs a) {
   constexpr bool F2 = sizeof(R) == 4;
   SumF2 sf[5];  // rp, rho u, kinetic energy (FP32 compute type)
   int64_t cnt = 0;
-  for (int64_t e = a.begin + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < a.end; e += stride) {
+  for (int64_t e = L.begin + t0; e < L.end; e += stride) {
     R g[Q];
 #pragma unroll
     for (int q = 0; q < Q; ++q) g[q] = Sto<S>::ld(p + (size_t)q * N + e);
     R rp, j[3];
-    raw_moments<Q, R>(g, rp, j);
+    if constexpr (F2) raw_moments<Q, R>(g, rp, j);
+    else raw_moments64<Q>(g, rp, j);
     R F[3] = {R(0), R(0), R(0)};
     if (a.force)
       for (int b = 0; b < D; ++b) F[b] = static_cast<const R*>(a.force)[(size_t)b * N + e];
@@ -1810,34 +1824,37 @@ __global__ void __launch_bounds__(256) k_reduce(const ReduceArgs a) {
     for (int b = 0; b < 3; ++b) acc[1 + b] = sf[1 + b].value();
     acc[7] = sf[4].value();
   }
-  if (a.r_scale == 1.0)
-    acc[0] = a.vol * (acc[0] + (double)cnt * a.rho_off);
+  if (L.r_scale == 1.0)
+    acc[0] = L.vol * (acc[0] + (double)cnt * a.rho_off);
   else  // density deviations in another level's units
-    acc[0] = a.vol * ((double)cnt * a.rho0 + a.r_scale * (acc[0] + (double)cnt * (a.rho_off - a.rho0)));
+    acc[0] = L.vol * ((double)cnt * a.rho0 + L.r_scale * (acc[0] + (double)cnt * (a.rho_off - a.rho0)));
 #pragma unroll
-  for (int b = 0; b < 3; ++b) acc[1 + b] *= a.vol_m;
-  acc[7] *= a.vol_k;
+  for (int b = 0; b < 3; ++b) acc[1 + b] *= L.vol_m;
+  acc[7] *= L.vol_k;
   // momentum exchange (Sec. 2.3): the link carries c_ib (f*_ib(x) + f_i(x)) to
   // the body, f_i the bounce-back value of the next step (interpolated with
   // the wall distance q; q = 1/2 gives 2 c_ib f*_ib)
-  for (int64_t l = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; l < a.obs_n; l += stride) {
-    const int i = a.obs_dir[l];
+  for (int64_t l = t0; l < L.obs_n; l += stride) {
+    const int i = L.obs_dir[l];
     const int ib = opp(i);
-    const int64_t e = a.obs_elem[l];
-    const double q = a.obs_q ? a.obs_q[l] : 0.5;
+    const int64_t e = L.obs_elem[l];
+    const double q = L.obs_q ? L.obs_q[l] : 0.5;
     const double go = (double)Sto<S>::ld(p + (size_t)ib * N + e);
     double gb;
     if (q < 0.5) {
-      const int32_t a2 = a.obs_a ? a.obs_a[l] : -1;
+      const int32_t a2 = L.obs_a ? L.obs_a[l] : -1;
       gb = a2 < 0 ? go : 2.0 * q * go + (1.0 - 2.0 * q) * (double)Sto<S>::ld(p + (size_t)ib * N + a2);
     } else {
       gb = go / (2.0 * q) + (2.0 * q - 1.0) / (2.0 * q) * (double)Sto<S>::ld(p + (size_t)i * N + e);
     }
     const double sum = go + gb + 2.0 * LT::w(ib) * a.rho_off;
 #pragma unroll
-    for (int b = 0; b < D; ++b) acc[4 + b] += a.fscale * LT::c(ib, b) * sum;
+    for (int b = 0; b < D; ++b) acc[4 + b] += L.fscale * LT::c(ib, b) * sum;
   }
-  block_sum_store<8>(acc, a.partial + (size_t)blockIdx.x * 8);
+  // mass, kinetic energy, momentum, and forces where there are obstacle links
+  const unsigned axes = (1u << D) - 1u;
+  block_sum_store<8, kRedBlock<S>>(acc, a.partial + (size_t)blockIdx.x * 8,
+                                   0x81u | axes << 1 | (L.obs_n > 0 ? axes << 4 : 0u));
 }
 
 // ----------------------------------------------------------------- launchers
@@ -1995,8 +2012,14 @@ struct Launch {
     if (a.cnt <= 0) return;
     with_q(Q, [&](auto q) { k_gather_ghosts<decltype(q)::value, S><<<blocks_for(a.cnt, 128), 128, 0, st>>>(a); });
   }
-  static void reduce(int Q, const ReduceArgs& a, cudaStream_t st) {
-    with_q(Q, [&](auto q) { k_reduce<decltype(q)::value, S><<<a.nblocks, 256, 0, st>>>(a); });
+  static unsigned reduce(int Q, ReduceArgs& a, cudaStream_t st) {
+    const unsigned g = assign_blocks(a, 1, [&](int k) {
+      const ReduceLevel& l = a.lev[k];
+      const int64_t n = std::max(l.end - l.begin, l.obs_n);
+      return std::min<int64_t>(std::max<int64_t>((n + kRedBlock<S> - 1) / kRedBlock<S>, 1), kReduceBlocks);
+    });
+    with_q(Q, [&](auto q) { k_reduce<decltype(q)::value, S><<<g, kRedBlock<S>, 0, st>>>(a); });
+    return g;
   }
 };
 

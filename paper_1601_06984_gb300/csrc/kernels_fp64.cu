@@ -18,13 +18,17 @@ __global__ void k_scatter_force(const ForceArgs a) {
   for (int b = 0; b < D; ++b) F[(size_t)b * a.Ntot + e] = R(a.stage[t * D + b]);
 }
 
-// Sum of the partial rows in a fixed order (one block): deterministic.
+// Sum of the partial rows in a fixed order (one block, a warp per column):
+// deterministic.
 __global__ void __launch_bounds__(256) k_final_reduce(const FinalArgs a) {
-  double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  for (int64_t r = threadIdx.x; r < a.n; r += blockDim.x)
+  const int col = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double acc[4] = {0, 0, 0, 0};
+  for (int64_t r = lane; r < a.n; r += 128)
 #pragma unroll
-    for (int c = 0; c < 8; ++c) acc[c] += a.partial[r * 8 + c];
-  block_sum_store<8>(acc, a.out);
+    for (int k = 0; k < 4; ++k)
+      if (r + 32 * k < a.n) acc[k] += a.partial[(r + 32 * k) * 8 + col];
+  const double s = warp_sum((acc[0] + acc[1]) + (acc[2] + acc[3]));
+  if (lane == 0) a.out[col] = s;
 }
 
 }  // namespace dev

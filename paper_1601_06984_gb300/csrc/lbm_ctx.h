@@ -214,6 +214,19 @@ struct lbm_ctx {
     for (const lbm::HostLevel& H : M.lv) n += H.nF;
     return n <= lbm::kBesideElements;
   }
+  // 64 bytes of pinned host memory that kernels can write (made by lbm_bind;
+  // null if unavailable)
+  double* result_host = nullptr;
+  bool result_tried = false;
+  double* pinned_result() {
+    if (!result_tried) {
+      result_tried = true;
+      void* q = nullptr;
+      if (cudaHostAlloc(&q, 64, cudaHostAllocMapped | cudaHostAllocPortable) == cudaSuccess) result_host = static_cast<double*>(q);
+      else cudaGetLastError();
+    }
+    return result_host;
+  }
   bool graphs_on = true;
   int64_t graph_steps = 0;  // replayed since the graphs were last dropped
   bool long_graphs() const {
@@ -241,6 +254,7 @@ struct lbm_ctx {
     recycle_timed();
     for (cudaEvent_t e : event_pool) cudaEventDestroy(e);
     if (cap_stream) cudaStreamDestroy(cap_stream);
+    if (result_host) cudaFreeHost(result_host);
     if (copy_st) cudaStreamDestroy(copy_st);
     for (cudaEvent_t e : copy_ev)
       if (e) cudaEventDestroy(e);

@@ -442,13 +442,13 @@ struct GatherGhostArgs {  // ghost pdfs -> FP64 [cnt][Q]
   double rho_off;
 };
 
-struct ReduceArgs {
+// Reductions of all levels in one launch, one partial row per block; a level
+// takes at most kReduceBlocks of them, by its size, so the order of the sums
+// is fixed by the mesh.
+struct ReduceLevel {
   const void* pdf;       // current state of the level
-  const void* force;
-  int64_t Ntot, begin, end;  // fluid range of the level
-  double omega, rho_off, vol;
-  double* partial;       // [nblocks][8]
-  int nblocks;
+  int64_t begin, end;    // fluid range of the level
+  double vol;
   // obstacle links of the level
   const int32_t* obs_elem;
   const int8_t* obs_dir;
@@ -458,7 +458,16 @@ struct ReduceArgs {
   double fscale;
   // mass vol (cnt rho0 + r_scale sum (rho - rho0)) (r_scale 1: vol sum rho),
   // momentum vol_m sum rho u, kinetic energy vol_k sum rho |u|^2 / 2
-  double vol_m, vol_k, r_scale, rho0;
+  double vol_m, vol_k, r_scale;
+};
+struct ReduceArgs {
+  uint32_t first[16];     // first block of each level (set by the launcher)
+  int nseg;               // levels
+  const void* force;
+  int64_t Ntot;
+  double rho_off, rho0;
+  double* partial;        // [blocks][8]
+  ReduceLevel lev[16];
 };
 
 struct FinalArgs {
@@ -482,7 +491,7 @@ struct Ops {
   void (*out)(int Q, const OutArgs&, cudaStream_t);
   void (*set_state)(int Q, const SetStateArgs&, cudaStream_t);
   void (*gather_ghosts)(int Q, const GatherGhostArgs&, cudaStream_t);
-  void (*reduce)(int Q, const ReduceArgs&, cudaStream_t);
+  unsigned (*reduce)(int Q, ReduceArgs&, cudaStream_t);  // returns the partial rows written
   size_t storage_bytes;  // bytes per stored pdf
   size_t compute_bytes;  // bytes of the compute type
 };
@@ -627,7 +636,7 @@ const Ops* ops_fp32dev();
 const Ops* ops_bf16dev();
 void launch_scatter_force(bool fp64, const ForceArgs&, cudaStream_t);
 void launch_final_reduce(const FinalArgs&, cudaStream_t);
-constexpr int kReduceBlocks = 512;  // blocks per reduce launch (fixed: deterministic order)
+constexpr int kReduceBlocks = 512;  // most blocks (partial rows) a level takes in a reduction
 
 // What a reduction over a bound context needs, without the scratch pointers
 // (used by the entry point that keeps its scratch in a static device array).
@@ -636,7 +645,7 @@ struct ReducePlan {
   int Q = 0;
   cudaStream_t stream = nullptr;
   const void* workspace = nullptr;
-  std::vector<ReduceArgs> levels;  // partial == nullptr; filled in by the caller
+  ReduceArgs args{};  // partial == nullptr; filled in by the caller
 };
 lbm_status reduce_plan(lbm_ctx* ctx, ReducePlan* plan);
 lbm_status set_error(lbm_ctx* ctx, lbm_status s, const std::string& msg);

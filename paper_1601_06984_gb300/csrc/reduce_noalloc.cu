@@ -75,10 +75,10 @@ extern "C" lbm_status lbm_reduce_noalloc(lbm_ctx* ctx, double out[8]) {
   lbm::ReducePlan plan;
   lbm_status s = lbm::reduce_plan(ctx, &plan);
   if (s != LBM_OK) return s;
-  const int64_t rows = (int64_t)plan.levels.size() * lbm::kReduceBlocks;
-  if (rows > kRows)
+  const int levels = plan.args.nseg;
+  if ((int64_t)levels * lbm::kReduceBlocks > kRows)
     return lbm::set_error(ctx, LBM_ERR_ARG,
-                          "lbm_reduce_noalloc: mesh has " + std::to_string(plan.levels.size()) +
+                          "lbm_reduce_noalloc: mesh has " + std::to_string(levels) +
                               " levels; the static scratch holds at most " +
                               std::to_string(kRows / lbm::kReduceBlocks) + " (use lbm_reduce)");
   double* scratch = nullptr;
@@ -88,15 +88,12 @@ extern "C" lbm_status lbm_reduce_noalloc(lbm_ctx* ctx, double out[8]) {
   // Every partial row read by the final sum is written by this call's level
   // kernels first, and the final kernel overwrites the result slot, so nothing
   // has to be cleared between calls.
-  for (size_t li = 0; li < plan.levels.size(); ++li) {
-    lbm::ReduceArgs a = plan.levels[li];
-    a.partial = scratch + li * lbm::kReduceBlocks * 8;
-    plan.ops->reduce(plan.Q, a, plan.stream);
-  }
+  plan.args.partial = scratch;
+  const unsigned rows = plan.ops->reduce(plan.Q, plan.args, plan.stream);
   double* result = scratch + kRows * 8;
-  lbm::FinalArgs fa{scratch, rows, result};
+  lbm::FinalArgs fa{scratch, (int64_t)rows, result};
   lbm::launch_final_reduce(fa, plan.stream);
-  lbm::count_launches(ctx, (int64_t)plan.levels.size() + 1);
+  lbm::count_launches(ctx, levels + 1);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaMemcpyAsync(out, result, 8 * sizeof(double), cudaMemcpyDeviceToHost, plan.stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(plan.stream);
