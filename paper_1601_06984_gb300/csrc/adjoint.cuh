@@ -3,10 +3,11 @@
 // Every forward kernel of the path has a reverse here: pull stream + BGK
 // collide (Sec. 2.1), the outlet values (Sec. 2.3), the GhostFromCoarser
 // source moments and compact interpolation and the GhostFromFiner restriction
-// (Sec. 2.2).  A reverse kernel reads the forward state the op saw (a snapshot),
-// consumes the adjoint of the op's outputs (and zeroes it: those slots were
-// overwritten by the op), and adds the transposed Jacobian times that adjoint
-// to the adjoint of the op's inputs.  Scatter targets are unique within one
+// (Sec. 2.2).  A reverse kernel reads the forward state the op saw (from the
+// tape) and applies the transposed Jacobian to the adjoint of the op's
+// outputs.  The reverse stream-collide stores the adjoint of its inputs, whose
+// rows hold nothing yet; the ghosts' adjoints go to compact arrays and are
+// added to their sources afterwards.  Scatter targets are unique within one
 // launch (each pdf slot is pulled by exactly one element; each ghost has its
 // own children; each source element appears once), so plain read-modify-write
 // is race-free; the ghost-to-source sums of GhostFromCoarser go through a

@@ -358,14 +358,17 @@ void lbm_ctx::tick_batched(int l0, int n) {
   };
   if (new_state)
     for (int l = l0; l < n; ++l) state[l][parity[l] ^ 1] = new_state(l);
-  ScArgs in = sc_args(), rest = sc_args();
+  ScArgs in = sc_args(), rest = sc_args(), rest_fin = sc_args();
   OutletArgs out = outlet_args(at(oSide));
   int64_t elements = 0;
   for (int l = l0; l < n; ++l) elements += M.lv[l].nF;
+  const bool beside = elements <= kBesideElements;
   for (int l = l0; l < n; ++l) {
+    // large instants: the finest level's rest apart, without record epilogue
+    ScArgs& r = beside || finest_only || l + 1 < n ? rest : rest_fin;
     launches += add_sc(in, l - l0, l, TK_INTERIOR);
-    launches += add_sc(rest, l - l0, l, TK_BOUNDARY);
-    launches += add_sc(rest, l - l0, l, TK_LIST);
+    launches += add_sc(r, l - l0, l, TK_BOUNDARY);
+    launches += add_sc(r, l - l0, l, TK_LIST);
     const int no = out.nlev;
     add_outlet(out, l, cur(l));
     launches += out.nlev - no;
@@ -373,12 +376,14 @@ void lbm_ctx::tick_batched(int l0, int n) {
   const bool chain = capturing && elements <= (p.precision == LBM_FP64 ? kChainElements64 : kChainElements);
   rest.chain = chain;
   const bool force = p.use_force != 0;
-  // Interior bricks read no ghost.  At small instants they all run beside the
-  // GhostFromCoarser fill; beyond kBesideElements the finest level's, which
-  // fill the GPU by themselves, only after it, apart from the coarser ones'
-  // (and so with BF16 storage, whose two-element kernel has no record
-  // epilogue).
-  const bool beside = elements <= kBesideElements;
+  // Interior bricks read no ghost.  At small instants they run beside the
+  // GhostFromCoarser fill; beyond kBesideElements only after it: the fill
+  // leaves an SM little L1 beside its shared memory, bricks that start there
+  // keep that split for as long as blocks follow one another, and in which
+  // order a graph starts two branches is not ours to say (sphere of 8.6e7
+  // elements, FP32, ms a step: after 33.1, beside 33.2 or 43.2).  The finest
+  // level's bricks are a launch of their own there (and with BF16 storage,
+  // whose two-element kernel has no record epilogue).
   ScArgs fin = in;
   int coarse_segs = 0;
   if (in.nseg > 1 && !in.seg[in.nseg - 1].rec_out && (!beside || p.precision == LBM_BF16DEV)) {
@@ -401,15 +406,13 @@ void lbm_ctx::tick_batched(int l0, int n) {
     if (gff.nseg > k) launches += 1 + (gff.lev[k].rec_out != nullptr);
   }
   if (gff.nseg) ops->fill_gff(Q, gff, st);
-  // Interior bricks beside the GhostFromCoarser fill: queued before it (the
-  // other way round, blocks of the bricks start on SMs set up for the fill's
-  // shared memory, with little L1: sphere 6.26 against 4.94 ms a step), but
+  // Interior bricks beside the GhostFromCoarser fill: queued before it, but
   // after it in FP64, where one-warp blocks of the bricks would fill the slots
   // the fill needs (D2Q9 channel 52 against 40 us)
-  const bool early = fin.nseg && (beside || coarse_segs);
+  const bool early = fin.nseg && beside;
   auto run_early = [&] {
     if (coarse_segs) ops->sc_interior(Q, force, in, br.s[0]);
-    if (beside) timed_launch(timed_level, TK_INTERIOR, [&] { ops->sc_interior(Q, force, fin, br.s[0]); }, br.s[0]);
+    timed_launch(timed_level, TK_INTERIOR, [&] { ops->sc_interior(Q, force, fin, br.s[0]); }, br.s[0]);
   };
   const bool fill_first = p.precision == LBM_FP64;
   if (early) {
@@ -432,9 +435,11 @@ void lbm_ctx::tick_batched(int l0, int n) {
   timed_launch(timed_level, TK_SC_SPAN, [&] {
     if (fin.nseg && !beside) {
       fork(0);
+      if (coarse_segs) ops->sc_interior(Q, force, in, br.s[0]);
       timed_launch(timed_level, TK_INTERIOR, [&] { ops->sc_interior(Q, force, fin, br.s[0]); }, br.s[0]);
     }
     if (rest.nseg) timed_launch(timed_level, TK_BOUNDARY, [&] { ops->sc_rest(Q, force, rest, st); });
+    if (rest_fin.nseg) ops->sc_rest(Q, force, rest_fin, st);
     if (fin.nseg) join(0);
   });
   for (int l = l0; l < n; ++l) parity[l] ^= 1;
@@ -1017,6 +1022,10 @@ lbm_status lbm_fill_ghosts(lbm_ctx* c) {
 // overwrites the whole array.
 static void touch_pages(void* p, size_t bytes) {
   if (!p || bytes < ((size_t)4 << 20)) return;
+  // pinned memory has its pages; device memory is for the copy to refuse
+  cudaPointerAttributes at{};
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) cudaGetLastError();
+  else if (at.type != cudaMemoryTypeUnregistered) return;
   const size_t page = (size_t)std::max(4096l, sysconf(_SC_PAGESIZE));
   volatile char* b = static_cast<volatile char*>(p);
   const int64_t n = (int64_t)((bytes + page - 1) / page);
