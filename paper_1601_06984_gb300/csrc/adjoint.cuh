@@ -972,8 +972,10 @@ __global__ void __launch_bounds__(kAdjBlock<S>, adj_minb<S>(2)) k_adj_gff(const 
 #pragma unroll
       for (int c = 0; c < D; ++c) uP[c] += __shfl_xor_sync(0xffffffffu, uP[c], o);
     }
-    // every lane of the group has read the ghost's adjoints (the shuffles are
-    // warp barriers); each clears its share
+    // every lane of the group reads all of the ghost's adjoints, and each
+    // clears its share of them: the shuffles order no memory accesses, so the
+    // warp waits here, inactive lanes too
+    __syncwarp();
     if (!active) continue;
 #pragma unroll
     for (int q = 0; q < Q; ++q)
