@@ -371,6 +371,12 @@ lbm_status lbm_adjoint(lbm_ctx* ctx, int64_t n_coarse, int32_t K, int32_t object
  * mode 1, or shares one with other levels, as in the captured steps. */
 lbm_status lbm_kernel_launches(const lbm_ctx* ctx, int64_t* count);
 
+/* Kernel launches that this context issued since it was bound (a replayed
+ * graph's kernel nodes among them), for the same work as lbm_kernel_launches:
+ * levels that share a launch count once.  The reverse kernels of lbm_adjoint
+ * are in neither count. */
+lbm_status lbm_launches(const lbm_ctx* ctx, int64_t* count);
+
 /* Device timing of the step's kernels with CUDA events on the bound stream.
  *  mode 0: off.
  *  mode 1: every launch of lbm_step is bracketed by events, and the steps are

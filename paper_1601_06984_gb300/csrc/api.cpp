@@ -143,7 +143,7 @@ void lbm_ctx::fill_gff(int li) {
   GffArgs a = gff_args();
   add_gff(a, li);
   if (!a.nseg) return;
-  timed_launch(li, TK_GFF, [&] { ops->fill_gff(Q, a, st); });
+  timed_launch(li, TK_GFF, [&] { issued += ops->fill_gff(Q, a, st); });
   ++launches;
 }
 
@@ -170,7 +170,7 @@ void lbm_ctx::source_moments(int li, size_t mom_off, cudaStream_t s, int subset)
   a.rx32 = make_relax32(M.lv[li].omega);
   a.rho_off = rho_off;
   a.rho_off32 = (float)rho_off;
-  timed_launch(li, TK_MOM, [&] { ops->source_moments(Q, a, s); }, s);
+  timed_launch(li, TK_MOM, [&] { issued += ops->source_moments(Q, a, s); }, s);
   ++launches;
 }
 
@@ -205,7 +205,7 @@ void lbm_ctx::fill_gfc(int lf, bool two_times, bool all_layers) {
   GfcArgs a = gfc_args();
   add_gfc(a, lf, two_times, all_layers);
   if (!a.nseg) return;
-  timed_launch(lf, TK_GFC, [&] { ops->fill_gfc(Q, a, st); });
+  timed_launch(lf, TK_GFC, [&] { issued += ops->fill_gfc(Q, a, st); });
   ++launches;
 }
 
@@ -299,13 +299,13 @@ void lbm_ctx::stream_collide(int li) {
   OutletArgs o = outlet_args(at(oSide));
   add_outlet(o, li, cur(li));
   if (o.nlev) {
-    timed_launch(li, TK_OUTLET, [&] { ops->outlet(Q, o, st); });
+    timed_launch(li, TK_OUTLET, [&] { issued += ops->outlet(Q, o, st); });
     ++launches;
   }
   for (int kind : {TK_INTERIOR, TK_BOUNDARY, TK_LIST}) {
     ScArgs a = sc_args();
     if (!add_sc(a, 0, li, kind)) continue;
-    timed_launch(li, kind, [&] { (kind == TK_INTERIOR ? ops->sc_interior : ops->sc_rest)(Q, p.use_force != 0, a, st); });
+    timed_launch(li, kind, [&] { issued += (kind == TK_INTERIOR ? ops->sc_interior : ops->sc_rest)(Q, p.use_force != 0, a, st); });
     ++launches;
   }
   parity[li] ^= 1;
@@ -392,7 +392,7 @@ void lbm_ctx::tick_batched(int l0, int n) {
     fin.seg[0] = in.seg[in.nseg - 1];
     in.nseg = coarse_segs;
   }
-  auto run_outlet = [&](cudaStream_t s) { ops->outlet(Q, out, s); };
+  auto run_outlet = [&](cudaStream_t s) { issued += ops->outlet(Q, out, s); };
   const bool out_branch = out.nlev && !outlet_reads_ghosts;
   if (out_branch) {
     fork(1);
@@ -405,14 +405,14 @@ void lbm_ctx::tick_batched(int l0, int n) {
     add_gff(gff, l);
     if (gff.nseg > k) launches += 1 + (gff.lev[k].rec_out != nullptr);
   }
-  if (gff.nseg) ops->fill_gff(Q, gff, st);
+  if (gff.nseg) issued += ops->fill_gff(Q, gff, st);
   // Interior bricks beside the GhostFromCoarser fill: queued before it, but
   // after it in FP64, where one-warp blocks of the bricks would fill the slots
   // the fill needs (D2Q9 channel 52 against 40 us)
   const bool early = fin.nseg && beside;
   auto run_early = [&] {
-    if (coarse_segs) ops->sc_interior(Q, force, in, br.s[0]);
-    timed_launch(timed_level, TK_INTERIOR, [&] { ops->sc_interior(Q, force, fin, br.s[0]); }, br.s[0]);
+    if (coarse_segs) issued += ops->sc_interior(Q, force, in, br.s[0]);
+    timed_launch(timed_level, TK_INTERIOR, [&] { issued += ops->sc_interior(Q, force, fin, br.s[0]); }, br.s[0]);
   };
   const bool fill_first = p.precision == LBM_FP64;
   if (early) {
@@ -428,18 +428,18 @@ void lbm_ctx::tick_batched(int l0, int n) {
   }
   for (int l = l0 + 1; l < n; ++l) add_gfc(gfc, l, false, false);
   launches += gfc.nseg;
-  if (gfc.nseg) ops->fill_gfc(Q, gfc, st);
+  if (gfc.nseg) issued += ops->fill_gfc(Q, gfc, st);
   if (early && fill_first) run_early();
   if (out.nlev && !out_branch) run_outlet(st);
   if (out_branch) join(1);
   timed_launch(timed_level, TK_SC_SPAN, [&] {
     if (fin.nseg && !beside) {
       fork(0);
-      if (coarse_segs) ops->sc_interior(Q, force, in, br.s[0]);
-      timed_launch(timed_level, TK_INTERIOR, [&] { ops->sc_interior(Q, force, fin, br.s[0]); }, br.s[0]);
+      if (coarse_segs) issued += ops->sc_interior(Q, force, in, br.s[0]);
+      timed_launch(timed_level, TK_INTERIOR, [&] { issued += ops->sc_interior(Q, force, fin, br.s[0]); }, br.s[0]);
     }
-    if (rest.nseg) timed_launch(timed_level, TK_BOUNDARY, [&] { ops->sc_rest(Q, force, rest, st); });
-    if (rest_fin.nseg) ops->sc_rest(Q, force, rest_fin, st);
+    if (rest.nseg) timed_launch(timed_level, TK_BOUNDARY, [&] { issued += ops->sc_rest(Q, force, rest, st); });
+    if (rest_fin.nseg) issued += ops->sc_rest(Q, force, rest_fin, st);
     if (fin.nseg) join(0);
   });
   for (int l = l0; l < n; ++l) parity[l] ^= 1;
@@ -521,7 +521,7 @@ const lbm_ctx::StepGraph* lbm_ctx::step_graph(int nsteps) {
   // capture on a private stream (the bound stream may be the legacy default
   // stream, which cannot be captured); host bookkeeping is restored afterwards
   const std::vector<int> p0 = parity;
-  const int64_t l0 = launches;
+  const int64_t l0 = launches, i0 = issued;
   if (timing == 2) {
     // events for the finest level's stream-collide launches and their span
     // (up to four pairs per substep, m^(nlev-1) substeps per coarse step, m
@@ -548,8 +548,9 @@ const lbm_ctx::StepGraph* lbm_ctx::step_graph(int nsteps) {
   st = user;
   std::vector<Timed> gt(timed.begin() + t0, timed.end());
   timed.resize(t0);
-  const int64_t nl = launches - l0;
+  const int64_t nl = launches - l0, ni = issued - i0;
   launches = l0;
+  issued = i0;
   // two steps bring every level back to its buffer; one step flips the
   // coarsest level's (the finer levels take an even number of substeps)
   std::vector<int> expect = p0;
@@ -569,7 +570,7 @@ const lbm_ctx::StepGraph* lbm_ctx::step_graph(int nsteps) {
     graphs_on = false;
     return nullptr;
   }
-  graphs.push_back({p0, p1, nsteps, exec, nl, std::move(gt)});
+  graphs.push_back({p0, p1, nsteps, exec, nl, ni, std::move(gt)});
   return &graphs.back();
 }
 
@@ -618,7 +619,10 @@ lbm_status reduce_plan(lbm_ctx* c, ReducePlan* plan) {
 
 lbm_status set_error(lbm_ctx* c, lbm_status s, const std::string& msg) { return c->fail(s, msg); }
 
-void count_launches(lbm_ctx* c, int64_t n) { c->launches += n; }
+void count_launches(lbm_ctx* c, int64_t level_kernels, int64_t issued) {
+  c->launches += level_kernels;
+  c->issued += issued;
+}
 
 }  // namespace lbm
 
@@ -791,7 +795,7 @@ lbm_status lbm_bind(lbm_ctx* c, void* ws, uint64_t bytes, void* stream) {
   for (size_t off : {c->oA, c->oB}) {
     FillArgs f{c->ws + off, m.Ntot, c->p.rho0, c->rho_off};
     c->ops->fill_rest(c->Q, f, c->st);
-    ++c->launches;
+    count_launches(c, 1, 1);
   }
   s = c->launched("bind");
   if (s == LBM_OK) s = c->cuda_check(cudaStreamSynchronize(c->st), "bind sync");
@@ -858,15 +862,15 @@ lbm_status lbm_init(lbm_ctx* c, const double* rho, const double* u, const double
     for (int li = 0; li < c->nlev; ++li) a.omega[li] = c->M.lv[li].omega;
     a.rho_off = c->rho_off;
     c->ops->init(Q, a, c->st);
-    ++c->launches;
+    count_launches(c, 1, 1);
     if (two) cudaEventRecord(c->copy_ev[half], c->st);
   }
   PlaceArgs pl{c->at(c->oB), c->at(c->oA), c->at<int32_t>(c->oSlotUser), n, c->M.Ntot};
   c->ops->init_place(Q, pl, c->st);
-  ++c->launches;
+  count_launches(c, 1, 1);
   FillArgs f{c->at(c->oB), c->M.Ntot, c->p.rho0, c->rho_off};
   c->ops->fill_rest(Q, f, c->st);
-  ++c->launches;
+  count_launches(c, 1, 1);
   lbm_status s = c->launched("init");
   if (s == LBM_OK) s = c->cuda_check(cudaStreamSynchronize(c->st), "init sync");
   return s;
@@ -885,7 +889,7 @@ lbm_status lbm_set_force(lbm_ctx* c, const double* F) {
     if (s != LBM_OK) return s;
     ForceArgs a{c->at(c->oF), c->at<int32_t>(c->oUslot), sf, first, cnt, c->M.Ntot, c->d};
     launch_scatter_force(c->p.precision == LBM_FP64, a, c->st);
-    ++c->launches;
+    count_launches(c, 1, 1);
   }
   c->recs_valid = false;
   lbm_status s = c->launched("set_force");
@@ -909,7 +913,7 @@ static lbm_status reduce_to_host(lbm_ctx* c, double out[8]) {
   double* pinned = c->result_host;
   FinalArgs fa{c->at<double>(c->oPartial), (int64_t)rows, pinned ? pinned : c->at<double>(c->oRed)};
   launch_final_reduce(fa, c->st);
-  c->launches += c->nlev + 1;  // a level's reduction counts as a kernel
+  count_launches(c, c->nlev + 1, 2);  // a level's reduction counts as a level kernel
   lbm_status s = c->launched("reduce");
   if (s == LBM_OK && !pinned)
     s = c->cuda_check(cudaMemcpyAsync(out, c->at(c->oRed), 64, cudaMemcpyDeviceToHost, c->st), "reduce copy");
@@ -961,7 +965,7 @@ static lbm_status step_run(lbm_ctx* c, int64_t n_coarse) {
       if (!g) break;
       lbm_status s = c->cuda_check(cudaGraphLaunch(g->exec, c->st), "graph launch");
       if (s != LBM_OK) return s;
-      c->launches += g->launches;
+      count_launches(c, g->launches, g->issued);
       c->parity = g->end;
       c->last_graph = (int)(g - c->graphs.data());
       c->graph_unread = true;
@@ -1075,7 +1079,7 @@ static lbm_status out_chunks(lbm_ctx* c, double* rho, double* u, double* S, doub
     a.first = i * CH;
     a.cnt = std::min(CH, n - a.first);
     c->ops->out(Q, a, c->st);
-    ++c->launches;
+    count_launches(c, 1, 1);
     if (two) cudaEventRecord(c->copy_ev[2 + (i & 1)], c->st);
   };
   compute(0);
@@ -1133,7 +1137,7 @@ lbm_status lbm_set_state(lbm_ctx* c, const double* f) {
     SetStateArgs a{c->at(c->oA), c->at(c->oB), c->at<int32_t>(c->oUslot), c->at<uint8_t>(c->oUlev),
                    c->parity_mask(), sf, first, cnt, c->M.Ntot, c->rho_off};
     c->ops->set_state(c->Q, a, c->st);
-    ++c->launches;
+    count_launches(c, 1, 1);
   }
   lbm_status s = c->launched("set_state");
   if (s == LBM_OK) s = c->cuda_check(cudaStreamSynchronize(c->st), "state sync");
@@ -1177,7 +1181,7 @@ lbm_status lbm_get_ghosts(lbm_ctx* c, int64_t* info, double* f) {
         const int64_t cnt = std::min<int64_t>(c->chunk, seg_cnt[sgi] - done);
         GatherGhostArgs a{c->cur(li), seg_first[sgi] + done, cnt, c->M.Ntot, stage, c->rho_off};
         c->ops->gather_ghosts(Q, a, c->st);
-        ++c->launches;
+        count_launches(c, 1, 1);
         lbm_status s = c->launched("ghosts");
         if (s == LBM_OK)
           s = c->cuda_check(cudaMemcpyAsync(f + (row + done) * Q, stage, cnt * Q * 8, cudaMemcpyDeviceToHost, c->st),
@@ -1200,6 +1204,12 @@ lbm_status lbm_sfc_partition(const int64_t* tree_ids, int64_t n, int32_t d, int3
 lbm_status lbm_kernel_launches(const lbm_ctx* c, int64_t* count) {
   if (!c || !count) return LBM_ERR_ARG;
   *count = c->launches;
+  return LBM_OK;
+}
+
+lbm_status lbm_launches(const lbm_ctx* c, int64_t* count) {
+  if (!c || !count) return LBM_ERR_ARG;
+  *count = c->issued;
   return LBM_OK;
 }
 

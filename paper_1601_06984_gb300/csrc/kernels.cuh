@@ -1903,8 +1903,9 @@ struct Launch {
       if (a.seg[k].rec_out) return true;
     return false;
   }
-  static void sc_interior(int Q, bool force, ScArgs& a, cudaStream_t st) {
+  static int sc_interior(int Q, bool force, ScArgs& a, cudaStream_t st) {
     const bool moms = any_records(a);
+    int n = 0;
     with_q(Q, [&](auto q) {
       constexpr int QQ = decltype(q)::value;
       if constexpr (std::is_same<S, __nv_bfloat16>::value) {
@@ -1920,11 +1921,13 @@ struct Launch {
             if (force) launch(k_sc_interior_pair<QQ, true>, g, LBM_BR_PAIR_BLOCK, st, one);
             else launch(k_sc_interior_pair<QQ, false>, g, LBM_BR_PAIR_BLOCK, st, one);
           }
+          n = a.nseg;
           return;
         }
       }
       const unsigned g = assign_blocks(a, kScBlock<S>, [&](int k) { return 64ll * a.seg[k].n; });
       if (!g) return;
+      n = 1;
       if (force) {
         if (moms) launch(k_sc_interior<QQ, S, true, true>, g, kScBlock<S>, st, a);
         else launch(k_sc_interior<QQ, S, true, false>, g, kScBlock<S>, st, a);
@@ -1933,12 +1936,13 @@ struct Launch {
         else launch(k_sc_interior<QQ, S, false, false>, g, kScBlock<S>, st, a);
       }
     });
+    return n;
   }
-  static void sc_rest(int Q, bool force, ScArgs& a, cudaStream_t st) {
+  static int sc_rest(int Q, bool force, ScArgs& a, cudaStream_t st) {
     const bool moms = any_records(a);
     const unsigned g =
         assign_blocks(a, kScBlock<S>, [&](int k) { return (a.seg[k].list ? 1ll : 64ll) * a.seg[k].n; });
-    if (!g) return;
+    if (!g) return 0;
     bool list = false;
     for (int k = 0; k < a.nseg; ++k) list |= a.seg[k].list != 0;
     with_q(Q, [&](auto q) {
@@ -1952,24 +1956,27 @@ struct Launch {
       if (force) moms ? by_list(T{}, T{}) : by_list(T{}, U{});
       else moms ? by_list(U{}, T{}) : by_list(U{}, U{});
     });
+    return 1;
   }
-  static void outlet(int Q, const OutletArgs& a, cudaStream_t st) {
-    if (!a.nlev) return;
+  static int outlet(int Q, const OutletArgs& a, cudaStream_t st) {
+    if (!a.nlev) return 0;
     const int64_t n = a.lev[a.nlev - 1].end - a.begin;
     with_q(Q, [&](auto q) { launch(k_outlet<decltype(q)::value, S>, blocks_for(n, kMomBlock<S>), kMomBlock<S>, st, a); });
+    return 1;
   }
-  static void source_moments(int Q, const MomentsArgs& a, cudaStream_t st) {
-    if (a.nsrc <= 0) return;
+  static int source_moments(int Q, const MomentsArgs& a, cudaStream_t st) {
+    if (a.nsrc <= 0) return 0;
     with_q(Q, [&](auto q) {
       constexpr int QQ = decltype(q)::value;
       const unsigned g = blocks_for(a.nsrc, kMomBlock<S>);
       if (a.force) k_source_moments<QQ, S, true><<<g, kMomBlock<S>, 0, st>>>(a);
       else k_source_moments<QQ, S, false><<<g, kMomBlock<S>, 0, st>>>(a);
     });
+    return 1;
   }
-  static void fill_gfc(int Q, GfcArgs& a, cudaStream_t st) {
+  static int fill_gfc(int Q, GfcArgs& a, cudaStream_t st) {
     const unsigned g = assign_blocks(a, kGfcBlock<S>, [&](int k) { return (int64_t)a.lev[k].ng; });
-    if (!g) return;
+    if (!g) return 0;
     bool two = false;
     for (int k = 0; k < a.nseg; ++k) two |= a.lev[k].mom2 != nullptr;
     with_q(Q, [&](auto q) {
@@ -1977,16 +1984,20 @@ struct Launch {
       else if (two) launch(k_fill_gfc<decltype(q)::value, S, true>, g, kGfcBlock<S>, st, a);
       else launch(k_fill_gfc<decltype(q)::value, S, false>, g, kGfcBlock<S>, st, a);
     });
+    return 1;
   }
-  static void fill_gff(int Q, GffArgs& a, cudaStream_t st) {
+  static int fill_gff(int Q, GffArgs& a, cudaStream_t st) {
+    int n = 0;
     with_q(Q, [&](auto q) {
       constexpr int QQ = decltype(q)::value;
       const unsigned g =
           assign_blocks(a, kGffBlock<S>, [&](int k) { return (int64_t)a.lev[k].ng << Lat<QQ>::D; });
       if (!g) return;
+      n = 1;
       if (a.force) launch(k_fill_gff<QQ, S, true>, g, kGffBlock<S>, st, a);
       else launch(k_fill_gff<QQ, S, false>, g, kGffBlock<S>, st, a);
     });
+    return n;
   }
   static void fill_rest(int Q, const FillArgs& a, cudaStream_t st) {
     with_q(Q, [&](auto q) { k_fill_rest<decltype(q)::value, S><<<blocks_for(a.Ntot, 256), 256, 0, st>>>(a); });

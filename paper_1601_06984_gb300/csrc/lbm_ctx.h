@@ -94,7 +94,8 @@ struct lbm_ctx {
   // state; and called when the fill at t + 1/2 reads a level's records at t + 1
   std::function<void*(int level)> new_state;
   std::function<void(int level)> at_mid_step;
-  int64_t launches = 0;
+  // level kernels (lbm_kernel_launches) and the launches that carried them (lbm_launches)
+  int64_t launches = 0, issued = 0;
   // optional mass check (params.check_every): coarse steps since the last
   // check, and the reference mass (taken at the first lbm_step after bind,
   // init or set_state)
@@ -174,7 +175,7 @@ struct lbm_ctx {
     std::vector<int> end;     // after the replay
     int steps;
     cudaGraphExec_t exec;
-    int64_t launches;
+    int64_t launches, issued;
     std::vector<Timed> timed;  // event pairs recorded by the graph (timing mode 2)
   };
   std::vector<StepGraph> graphs;

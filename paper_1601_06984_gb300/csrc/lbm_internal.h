@@ -477,14 +477,15 @@ struct FinalArgs {
 };
 
 struct Ops {
+  // The ops of a step return the kernels they launched.
   // interior bricks of the segments' levels (record epilogue where a level has sources)
-  void (*sc_interior)(int Q, bool force, ScArgs&, cudaStream_t);
+  int (*sc_interior)(int Q, bool force, ScArgs&, cudaStream_t);
   // boundary bricks and neighbour-list elements
-  void (*sc_rest)(int Q, bool force, ScArgs&, cudaStream_t);
-  void (*outlet)(int Q, const OutletArgs&, cudaStream_t);
-  void (*source_moments)(int Q, const MomentsArgs&, cudaStream_t);
-  void (*fill_gfc)(int Q, GfcArgs&, cudaStream_t);
-  void (*fill_gff)(int Q, GffArgs&, cudaStream_t);
+  int (*sc_rest)(int Q, bool force, ScArgs&, cudaStream_t);
+  int (*outlet)(int Q, const OutletArgs&, cudaStream_t);
+  int (*source_moments)(int Q, const MomentsArgs&, cudaStream_t);
+  int (*fill_gfc)(int Q, GfcArgs&, cudaStream_t);
+  int (*fill_gff)(int Q, GffArgs&, cudaStream_t);
   void (*fill_rest)(int Q, const FillArgs&, cudaStream_t);
   void (*init)(int Q, const InitArgs&, cudaStream_t);
   void (*init_place)(int Q, const PlaceArgs&, cudaStream_t);
@@ -649,6 +650,6 @@ struct ReducePlan {
 };
 lbm_status reduce_plan(lbm_ctx* ctx, ReducePlan* plan);
 lbm_status set_error(lbm_ctx* ctx, lbm_status s, const std::string& msg);
-void count_launches(lbm_ctx* ctx, int64_t n);
+void count_launches(lbm_ctx* ctx, int64_t level_kernels, int64_t issued);
 
 }  // namespace lbm

@@ -93,7 +93,7 @@ extern "C" lbm_status lbm_reduce_noalloc(lbm_ctx* ctx, double out[8]) {
   double* result = scratch + kRows * 8;
   lbm::FinalArgs fa{scratch, (int64_t)rows, result};
   lbm::launch_final_reduce(fa, plan.stream);
-  lbm::count_launches(ctx, levels + 1);
+  lbm::count_launches(ctx, levels + 1, 2);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaMemcpyAsync(out, result, 8 * sizeof(double), cudaMemcpyDeviceToHost, plan.stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(plan.stream);

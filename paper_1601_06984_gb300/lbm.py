@@ -24,7 +24,7 @@ OUTLET_LINEAR, OUTLET_ZERO_GRADIENT = 0, 1
 INLET_UNIFORM, INLET_PARABOLIC = 0, 1
 EXPORTS = ["lbm_build_mesh", "lbm_mesh_info", "lbm_device_bytes", "lbm_bind", "lbm_init", "lbm_set_force",
            "lbm_step", "lbm_fill_ghosts", "lbm_moments", "lbm_reduce", "lbm_get_state", "lbm_set_state", "lbm_ghost_count",
-           "lbm_get_ghosts", "lbm_sfc_partition", "lbm_kernel_launches", "lbm_timing_enable", "lbm_timing_read",
+           "lbm_get_ghosts", "lbm_sfc_partition", "lbm_kernel_launches", "lbm_launches", "lbm_timing_enable", "lbm_timing_read",
            "lbm_reduce_noalloc", "lbm_set_params", "lbm_adjoint_bytes", "lbm_adjoint", "lbm_last_error",
            "lbm_destroy", "lbm_obstacle_links", "lbm_set_link_q", "lbm_alu_peak", "lbm_halo_plan"]
 
@@ -73,6 +73,7 @@ def lib():
             "lbm_get_ghosts": [P, P, P],
             "lbm_sfc_partition": [P, I64, I32, I32, P, P, P, P],
             "lbm_kernel_launches": [P, C.POINTER(I64)],
+            "lbm_launches": [P, C.POINTER(I64)],
             "lbm_timing_enable": [P, I32],
             "lbm_timing_read": [P, P, P, I32],
             "lbm_reduce_noalloc": [P, P],
@@ -260,8 +261,15 @@ class Sim:
         return int(nbytes.value)
 
     def kernel_launches(self):
+        """Level kernels since bind: one per kernel and level, shared launch or not."""
         n = C.c_int64()
         _check(self.ctx, lib().lbm_kernel_launches(self.ctx, C.byref(n)))
+        return int(n.value)
+
+    def launches(self):
+        """Kernel launches issued since bind (levels that share one count once)."""
+        n = C.c_int64()
+        _check(self.ctx, lib().lbm_launches(self.ctx, C.byref(n)))
         return int(n.value)
 
     def timing_enable(self, mode=1):
