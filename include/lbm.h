@@ -219,8 +219,10 @@ lbm_status lbm_set_force(lbm_ctx* ctx, const double* F);
  * two substeps of the next finer level).  Pairs of coarse steps replay a CUDA
  * graph captured on first use, a remaining single step a one-step graph (one
  * of each per A/B parity state; dropped by lbm_set_params and lbm_bind), on
- * the bound stream; in timing mode 1 every step is launched kernel by kernel
- * (the adjoint's recomputed steps too).  Both paths do the same ops with the
+ * the bound stream.  A small mesh (at most 2^21 updates and 16 instants a
+ * coarse step) that has replayed 64 steps takes graphs of 16 steps where that
+ * many are left, also captured on first use.  In timing mode 1 every step is
+ * launched kernel by kernel (the adjoint's recomputed steps too).  Both paths do the same ops with the
  * same kernels; in the graphs one launch takes all levels that advance at the
  * same instant, and the interior bricks run beside the other elements, which
  * leaves every result bitwise the same.  With params.check_every = M

@@ -42,9 +42,14 @@ constexpr int64_t kBesideElements = 1 << 20;
 // has at most kLongGraphUpdates updates a coarse step, it replays graphs of
 // kLongGraphSteps: us per call, with its output, D2Q9 channel FP64, 50 steps
 // 2003 -> 1879, cylinder, 50 steps 2745 -> 2601, two-level 64^3, 200 steps 8870
-// -> 8620, D2Q9 32x32 FP64, 20 steps 811 -> 792.
+// -> 8620, D2Q9 32x32 FP64, 20 steps 811 -> 792.  A step of many instants is
+// long against the gap, and its graph large: kLongGraphInstants instants a step
+// (five levels, or three in diffusive scaling) keep a long graph to about a
+// thousand nodes.  (16 steps in FP32, a long graph against short ones: 16
+// instants 1.33 / 1.35 ms, 64 instants 3.02 / 3.04 ms, 1,024 instants, six
+// levels in diffusive scaling, 55 / 50 ms and 240 ms to make its 4.1e4 nodes.)
 constexpr int kLongGraphSteps = 16;
-constexpr int64_t kLongGraphAfter = 64, kLongGraphUpdates = 1 << 21;
+constexpr int64_t kLongGraphAfter = 64, kLongGraphUpdates = 1 << 21, kLongGraphInstants = 16;
 // Kernel kinds of the per-launch timing (lbm_timing_read row kTimedKinds * L + kind)
 enum TimedKind { TK_INTERIOR = 0, TK_LIST = 1, TK_BOUNDARY = 2, TK_GFF = 3, TK_MOM = 4, TK_GFC = 5, TK_OUTLET = 6,
                  TK_SC_SPAN = 7 };
@@ -229,11 +234,15 @@ struct lbm_ctx {
     return result_host;
   }
   bool graphs_on = true;
-  int64_t graph_steps = 0;  // replayed since the graphs were last dropped
+  int64_t graph_steps = 0;     // replayed since the graphs were last dropped
   bool long_graphs() const {
-    int64_t updates = 0, per = 1;
-    for (int li = 0; li < nlev; ++li, per *= lbm::time_ratio(p.time_mode)) updates += M.lv[li].nF * per;
-    return timing == 0 && graph_steps >= lbm::kLongGraphAfter && updates <= lbm::kLongGraphUpdates;
+    int64_t updates = 0, instants = 1;
+    for (int li = 0; li < n_filled; ++li) {
+      if (li) instants *= lbm::time_ratio(p.time_mode);
+      updates += M.lv[li].nF * instants;
+    }
+    return timing == 0 && graph_steps >= lbm::kLongGraphAfter && updates <= lbm::kLongGraphUpdates &&
+           instants <= lbm::kLongGraphInstants;
   }
   int last_graph = -1;        // graph of the most recent replay
   bool graph_unread = false;  // its events hold a replay not yet read
