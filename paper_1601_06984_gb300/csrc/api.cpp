@@ -567,7 +567,7 @@ const lbm_ctx::StepGraph* lbm_ctx::step_graph(int nsteps) {
       event_pool.push_back(t.a);
       event_pool.push_back(t.b);
     }
-    graphs_on = false;
+    (nsteps > 2 ? long_graphs_on : graphs_on) = false;
     return nullptr;
   }
   graphs.push_back({p0, p1, nsteps, exec, nl, ni, std::move(gt)});
@@ -961,7 +961,8 @@ static lbm_status step_run(lbm_ctx* c, int64_t n_coarse) {
     while (k < n_coarse) {
       const int64_t left = n_coarse - k;
       const bool longer = left >= kLongGraphSteps && c->long_graphs();
-      const lbm_ctx::StepGraph* g = c->step_graph(longer ? kLongGraphSteps : left >= 2 ? 2 : 1);
+      const lbm_ctx::StepGraph* g = longer ? c->step_graph(kLongGraphSteps) : nullptr;
+      if (!g) g = c->step_graph(left >= 2 ? 2 : 1);
       if (!g) break;
       lbm_status s = c->cuda_check(cudaGraphLaunch(g->exec, c->st), "graph launch");
       if (s != LBM_OK) return s;

@@ -234,6 +234,7 @@ struct lbm_ctx {
     return result_host;
   }
   bool graphs_on = true;
+  bool long_graphs_on = true;  // false once a long graph could not be made
   int64_t graph_steps = 0;     // replayed since the graphs were last dropped
   bool long_graphs() const {
     int64_t updates = 0, instants = 1;
@@ -241,7 +242,7 @@ struct lbm_ctx {
       if (li) instants *= lbm::time_ratio(p.time_mode);
       updates += M.lv[li].nF * instants;
     }
-    return timing == 0 && graph_steps >= lbm::kLongGraphAfter && updates <= lbm::kLongGraphUpdates &&
+    return long_graphs_on && timing == 0 && graph_steps >= lbm::kLongGraphAfter && updates <= lbm::kLongGraphUpdates &&
            instants <= lbm::kLongGraphInstants;
   }
   int last_graph = -1;        // graph of the most recent replay
@@ -340,8 +341,9 @@ struct lbm_ctx {
     advance(0);
   }
   // graph of nsteps (1, or an even number) coarse steps from the current parity state,
-  // captured on first use; null when capture is unavailable (the caller
-  // steps eagerly)
+  // captured on first use; null when capture is unavailable: the caller steps
+  // eagerly (graphs_on cleared) or, of a long graph, with shorter ones
+  // (long_graphs_on cleared)
   const StepGraph* step_graph(int nsteps);
   // n coarse steps as lbm_step issues them (graph replay unless timing mode 1)
   lbm_status run_steps(int64_t n_coarse);

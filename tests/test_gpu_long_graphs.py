@@ -1,5 +1,6 @@
 """Graphs of several coarse steps: the same results as the steps one by one,
-and no graph of a size beyond its use."""
+no graph of a size beyond its use, and a graph that cannot be made leaves the
+shorter ones in use."""
 import os
 import subprocess
 import sys
@@ -42,8 +43,8 @@ def test_long_graphs_equal_level_by_level(levels, mode, precision):
     assert np.array_equal(a.ghosts()[1], b.ghosts()[1])
 
 
-# cudaGraphInstantiate in front of the runtime's: writes down the most nodes that
-# were asked for
+# cudaGraphInstantiate in front of the runtime's: refuses graphs of more than
+# MAX_NODES nodes and writes down the most that were asked for
 SHIM = r"""
 #define _GNU_SOURCE
 #include <dlfcn.h>
@@ -59,6 +60,7 @@ int cudaGraphInstantiate(void** exec, void* graph, unsigned long long flags) {
   FILE* f = fopen(getenv("NODES_FILE"), "w");
   fprintf(f, "%zu", most);
   fclose(f);
+  if (n > (size_t)atol(getenv("MAX_NODES"))) return 2; /* cudaErrorMemoryAllocation */
   return ((inst_t)dlsym(RTLD_NEXT, "cudaGraphInstantiate"))(exec, graph, flags);
 }
 """
@@ -77,14 +79,14 @@ print("launches", s.launches() - n)
 """
 
 
-def run_child(tmp_path, levels, mode):
+def run_child(tmp_path, levels, mode, max_nodes):
     """Launches of 32 coarse steps after 64 of them, and the largest graph asked for."""
     src, so, nodes = tmp_path / "shim.c", tmp_path / "shim.so", tmp_path / "nodes"
     src.write_text(SHIM)
     subprocess.run(["gcc", "-shared", "-fPIC", "-O1", str(src), "-o", str(so), "-ldl"], check=True)
     om = 1.6 if mode == 2 else W.omega_coarse_from_finest(1.6, levels)
     code = CHILD.format(root=ROOT, tests=os.path.join(ROOT, "tests"), levels=levels, mode=mode, omega=repr(om))
-    env = dict(os.environ, LD_PRELOAD=str(so), NODES_FILE=str(nodes))
+    env = dict(os.environ, LD_PRELOAD=str(so), NODES_FILE=str(nodes), MAX_NODES=str(max_nodes))
     r = subprocess.run([sys.executable, "-c", code], env=env, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stderr
     return int(r.stdout.split("launches")[1]), int(nodes.read_text())
@@ -93,5 +95,13 @@ def run_child(tmp_path, levels, mode):
 def test_long_graphs_stay_small(tmp_path):
     """Six levels of diffusive scaling advance at 1,024 instants a coarse step:
     the two-step graph is the largest that is made."""
-    _, most = run_child(tmp_path, 6, 2)
+    _, most = run_child(tmp_path, 6, 2, 10**9)
     assert most <= 2 * 1024 * 8  # at most eight nodes an instant
+
+
+def test_a_long_graph_that_cannot_be_made_leaves_the_short_ones(tmp_path):
+    """Two levels: 7 launches a replayed step (9 launched level by level)."""
+    assert run_child(tmp_path, 2, 0, 10**9)[0] == 32 * 7
+    launches, most = run_child(tmp_path, 2, 0, 40)
+    assert most > 40  # a long graph was refused
+    assert launches == 32 * 7
