@@ -225,7 +225,11 @@ lbm_status lbm_set_force(lbm_ctx* ctx, const double* F);
  * launched kernel by kernel (the adjoint's recomputed steps too).  Both paths do the same ops with the
  * same kernels; in the graphs one launch takes all levels that advance at the
  * same instant, and the interior bricks run beside the other elements, which
- * leaves every result bitwise the same.  With params.check_every = M
+ * leaves every result bitwise the same.  The interior bricks have the bound
+ * stream's priority; on meshes of at most 2^20 elements the replayed steps'
+ * other kernels, on the critical path, have one level more (if there is one):
+ * they go before work on other streams of the bound stream's priority, and
+ * never before streams of a greater one.  With params.check_every = M
  * the mass is checked after every M-th coarse step (see lbm_params); a failed
  * check returns LBM_ERR_NUMERIC right after that step, with the state left as
  * it was then (the context stays usable, e.g. for lbm_set_state). */

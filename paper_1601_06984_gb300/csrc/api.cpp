@@ -490,14 +490,23 @@ void lbm_ctx::advance(int li) {
   }
 }
 
+void lbm_ctx::set_priority() {
+  int bound = 0, least = 0, greatest = 0;
+  if (cudaStreamGetPriority(st, &bound) != cudaSuccess || cudaDeviceGetStreamPriorityRange(&least, &greatest) != cudaSuccess) {
+    cudaGetLastError();
+    bound = greatest = 0;
+  }
+  const StepPriority p = step_priority(bound, greatest);
+  if (p.bricks != prio.bricks || p.chain != prio.chain) drop_streams();
+  prio = p;
+}
+
 bool lbm_ctx::make_branches() {
   if (br.s[0]) return br.ok;
   br.ok = true;
-  int least = 0, greatest = 0;
-  cudaDeviceGetStreamPriorityRange(&least, &greatest);
   for (int b = 0; b < 2; ++b) {
-    br.ok = br.ok &&
-            cudaStreamCreateWithPriority(&br.s[b], cudaStreamNonBlocking, b == 0 ? least : greatest) == cudaSuccess;
+    br.ok = br.ok && cudaStreamCreateWithPriority(&br.s[b], cudaStreamNonBlocking,
+                                                  b == 0 ? prio.bricks : prio.chain) == cudaSuccess;
     for (cudaEvent_t* e : {&br.fork[b], &br.join[b]})
       br.ok = br.ok && cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess;
   }
@@ -508,9 +517,7 @@ bool lbm_ctx::make_branches() {
 const lbm_ctx::StepGraph* lbm_ctx::step_graph(int nsteps) {
   for (const StepGraph& g : graphs)
     if (g.parity == parity && g.steps == nsteps) return &g;
-  int least = 0, greatest = 0;
-  cudaDeviceGetStreamPriorityRange(&least, &greatest);
-  if (!cap_stream && cudaStreamCreateWithPriority(&cap_stream, cudaStreamNonBlocking, greatest) != cudaSuccess) {
+  if (!cap_stream && cudaStreamCreateWithPriority(&cap_stream, cudaStreamNonBlocking, prio.chain) != cudaSuccess) {
     cudaGetLastError();
     graphs_on = false;
     return nullptr;
@@ -559,7 +566,8 @@ const lbm_ctx::StepGraph* lbm_ctx::step_graph(int nsteps) {
   const bool same = p1 == expect;
   parity = p0;
   cudaGraphExec_t exec = nullptr;
-  if (e == cudaSuccess && graph && same) e = cudaGraphInstantiate(&exec, graph, batched && prioritised() ? cudaGraphInstantiateFlagUseNodePriority : 0);
+  if (e == cudaSuccess && graph && same)
+    e = cudaGraphInstantiate(&exec, graph, batched && prioritised() ? cudaGraphInstantiateFlagUseNodePriority : 0);
   if (graph) cudaGraphDestroy(graph);
   if (e != cudaSuccess || !exec || !same) {
     cudaGetLastError();
@@ -751,6 +759,7 @@ lbm_status lbm_bind(lbm_ctx* c, void* ws, uint64_t bytes, void* stream) {
   c->drop_graphs();  // captured steps point into the previous workspace
   c->ws = static_cast<char*>(ws);
   c->st = static_cast<cudaStream_t>(stream);
+  c->set_priority();
   c->reset_state_buffers();
   c->pinned_result();
   const HostMesh& m = c->M;

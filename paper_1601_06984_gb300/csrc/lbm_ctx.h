@@ -30,11 +30,19 @@ constexpr int64_t kChainElements = 1 << 20, kChainElements64 = 1 << 12;
 // 57.3, two-level 64^3 44.9 / 45.7, D3Q27 9e5 elements 131 / 132; beyond it the
 // sphere of 1.1e7 elements took 7.4 against 4.94 ms).
 constexpr int64_t kBesideElements = 1 << 20;
-// Graphs of meshes within kBesideElements give the interior bricks the least
-// priority and the chain of fills and the rest the greatest: its blocks, on
-// the critical path, start before the waiting bricks' (two-level 64^3 FP32 8510
-// -> 7930 us for 200 steps; others within 0.5%).  Beyond it the mixture slows
-// the bricks (sphere of 1.1e7 elements 4.97 -> 5.38 ms a step).
+// Graphs of meshes within kBesideElements give the chain of fills and the rest
+// one level of priority more than the interior bricks: its blocks, on the
+// critical path, start before the waiting bricks' (two-level 64^3 FP32 7450 ->
+// 6730 us for 200 steps, D3Q27 96x80x64 4408 -> 4366 for 50; others within
+// 0.5%).  Beyond it the mixture slows the bricks (sphere of 1.1e7 elements 4.97
+// -> 5.38 ms a step).  The bricks keep the bound stream's priority, so that the
+// steps never pass a stream that the caller ranks above it; on a stream of the
+// greatest priority all kernels have that one.  (The least and the greatest
+// priority of the device instead: 6728 us.)
+struct StepPriority {
+  int bricks, chain;
+};
+inline StepPriority step_priority(int bound, int greatest) { return {bound, bound > greatest ? bound - 1 : bound}; }
 //
 // A graph launch costs about 3.5 us between two replays, 4 to 5% of a step of a
 // small mesh with two steps a graph.  Once a context has replayed
@@ -185,6 +193,9 @@ struct lbm_ctx {
   };
   std::vector<StepGraph> graphs;
   cudaStream_t cap_stream = nullptr;
+  // of the kernels in the captured steps (lbm_bind: by the bound stream's)
+  lbm::StepPriority prio{0, 0};
+  void set_priority();
   // branch streams and fork/join events of the captured graphs: [0] the
   // interior bricks, [1] the boundary values
   struct Branches {
@@ -264,16 +275,22 @@ struct lbm_ctx {
     drop_graphs();
     recycle_timed();
     for (cudaEvent_t e : event_pool) cudaEventDestroy(e);
-    if (cap_stream) cudaStreamDestroy(cap_stream);
+    drop_streams();
     if (result_host) cudaFreeHost(result_host);
     if (copy_st) cudaStreamDestroy(copy_st);
     for (cudaEvent_t e : copy_ev)
       if (e) cudaEventDestroy(e);
+  }
+  // the capture and branch streams, made again when they are next needed
+  void drop_streams() {
+    if (cap_stream) cudaStreamDestroy(cap_stream);
+    cap_stream = nullptr;
     for (int b = 0; b < 2; ++b) {
       if (br.s[b]) cudaStreamDestroy(br.s[b]);
       for (cudaEvent_t e : {br.fork[b], br.join[b]})
         if (e) cudaEventDestroy(e);
     }
+    br = Branches{};
   }
 
   template <class T = void>
