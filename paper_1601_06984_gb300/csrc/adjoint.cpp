@@ -130,11 +130,16 @@ AdjLayout adj_layout(lbm_ctx* c, int64_t n, int K) {
   L.lamF = take((size_t)c->d * N * 8);
   L.side_fwd = take(c->M.out_elem.size() * lb);
   L.lam_side = take(c->M.out_elem.size() * lb);
-  const int64_t block = adj_ops_for(c->p.precision)->sc_block;
-  int64_t interior = kAdjBlocks, rest = 0;
+  const AdjOps* aops = adj_ops_for(c->p.precision);
+  const int64_t block = aops->sc_block;
+  int64_t interior = 1, rest = 0;
   for (int li = 0; li < c->nlev; ++li) {
     const HostLevel& H = c->M.lv[li];
-    interior = std::max(interior, (64 * H.nB + block - 1) / block);
+    // four lanes a source at most, 2^d a ghost of the GhostFromFiner fill
+    const int64_t ghosts =
+        std::max({adj_grid(4 * (int64_t)H.src_elem.size(), aops->ghost_block), adj_grid(H.nC, aops->ghost_block),
+                  adj_grid((H.nG1 + H.nG2) << c->d, aops->sc_block), adj_grid(H.out_end - H.out_begin, kAdjLinkBlock)});
+    interior = std::max({interior, ghosts, (64 * H.nB + block - 1) / block});
     rest = std::max(rest, (64 * H.nBb + block - 1) / block + (H.N - 64 * (H.nB + H.nBb)) / block + 2);
   }
   // the rest of the reverse stream-collide runs beside the interior bricks',

@@ -1018,11 +1018,6 @@ __global__ void __launch_bounds__(kAdjBlock<S>, adj_minb<S>(2)) k_adj_gff(const 
 }
 
 // ----------------------------------------------------------------- launchers
-inline unsigned adj_grid(int64_t n, int threads) {
-  const int64_t b = (n + threads - 1) / threads;
-  return (unsigned)(b < 1 ? 1 : (b > kAdjBlocks ? kAdjBlocks : b));
-}
-
 template <class S>
 struct AdjLaunch {
   static void seed(int Q, const AdjSeedArgs& a, cudaStream_t st) {
@@ -1044,7 +1039,7 @@ struct AdjLaunch {
   static void outlet(int Q, const AdjOutletArgs& a, cudaStream_t st) {
     if (a.end <= a.begin) return;
     with_q(Q, [&](auto q) {
-      k_adj_outlet<decltype(q)::value, S><<<adj_grid(a.end - a.begin, 64), 64, 0, st>>>(a);
+      k_adj_outlet<decltype(q)::value, S><<<adj_grid(a.end - a.begin, kAdjLinkBlock), kAdjLinkBlock, 0, st>>>(a);
     });
   }
   static constexpr int kGhostBlock = sizeof(typename Sto<S>::R) == 8 ? 32 : 128;
@@ -1078,7 +1073,7 @@ template <class S>
 const AdjOps* make_adj_ops() {
   static const AdjOps ops = {&AdjLaunch<S>::seed,    &AdjLaunch<S>::sc_interior, &AdjLaunch<S>::sc_rest,
                              &AdjLaunch<S>::outlet,  &AdjLaunch<S>::moments, &AdjLaunch<S>::gfc,
-                             &AdjLaunch<S>::gff,     sizeof(typename Sto<S>::R), kAdjBlock<S>};
+                             &AdjLaunch<S>::gff,     sizeof(typename Sto<S>::R), kAdjBlock<S>, AdjLaunch<S>::kGhostBlock};
   return &ops;
 }
 

@@ -502,7 +502,17 @@ struct Ops {
 // [d][Ntot] FP64; partial holds one running row of parameter derivatives per
 // block (cols 0..15 d/d omega of each level, 16..18 d/d u_in): block b of
 // every launch adds its sums to row b, so the totals are deterministic.
-constexpr int kAdjBlocks = 1024;  // largest grid of the reverse ghost and boundary kernels
+// Grid of a reverse ghost or boundary kernel over n items: at most kAdjThreads
+// threads, whatever the block, which then stride.  (At most 1,024 blocks left
+// the one- and two-warp blocks of FP64 at 7 and 13 warps an SM.  FP64 two-level
+// D3Q19: 64^3, per launch, GhostFromCoarser 51 -> 44 us; 96^3 GhostFromFiner
+// 514 -> 463, records 224 -> 181 us, gradient of 8 steps 33.9 -> 32.8 ms.)
+constexpr int64_t kAdjThreads = 1 << 18;
+inline unsigned adj_grid(int64_t n, int threads) {
+  const int64_t b = (n + threads - 1) / threads, most = kAdjThreads / threads;
+  return (unsigned)(b < 1 ? 1 : b > most ? most : b);
+}
+constexpr int kAdjLinkBlock = 64;  // threads per block of the reverse boundary values
 constexpr int kAccCols = 32;
 
 struct AdjCommon {
@@ -610,7 +620,9 @@ struct AdjOps {
   void (*gfc)(int Q, const AdjGfcArgs&, cudaStream_t);
   void (*gff)(int Q, const AdjGffArgs&, cudaStream_t);
   size_t lam_bytes;  // bytes per adjoint value (compute type)
-  int sc_block;      // threads per block of the reverse stream-collide (one running row per block)
+  // threads per block of the reverse stream-collide and GhostFromFiner fill,
+  // and of the reverse records and GhostFromCoarser fill (one running row per block)
+  int sc_block, ghost_block;
 };
 const AdjOps* adj_ops_fp64();
 const AdjOps* adj_ops_fp32dev();
