@@ -656,8 +656,9 @@ __device__ __forceinline__ void bgk_collide(R (&g)[Q], const RelaxOf<R>& rx, R r
 // FP64 storage: one warp per block.  A warp holds its SM's FP64 pipe for about
 // 120 x 19 cycles, so a launch takes as long as the SM with the most warps,
 // and small blocks spread a small level over all SMs (D2Q9, 1,800 elements:
-// 7 blocks of 256 on 7 SMs before).  Registers are not capped: 12 to 24 warps
-// per SM keep the pipe busy, and the caps of 64 and 80 registers spilled.
+// 7 blocks of 256 on 7 SMs before).  12 to 24 warps per SM keep the pipe busy,
+// and bounds of 24, 16 and 12 blocks (D2Q9, D3Q19, D3Q27) leave every kernel
+// the registers it takes, 64, 114 and 148 at most; 80 for D3Q19 spilled.
 template <class S>
 constexpr int kScBlock = sizeof(S) == 8 ? 32 : 256;
 template <int Q>
@@ -958,7 +959,6 @@ __global__ void k_outlet(const __grid_constant__ OutletArgs a) {
   const size_t N = (size_t)a.Ntot;
   const int i = a.dir[k];
   R* side = static_cast<R*>(a.side);
-  wait_for_previous();
   if (a.kind[k] == OUT_EXTRAP) {
     const R fa = Sto<S>::ld(src + (size_t)i * N + a.a[k]);
     side[k] = a.zero_gradient ? fa : R(2) * fa - Sto<S>::ld(src + (size_t)i * N + a.b[k]);
@@ -1961,7 +1961,7 @@ struct Launch {
   static int outlet(int Q, const OutletArgs& a, cudaStream_t st) {
     if (!a.nlev) return 0;
     const int64_t n = a.lev[a.nlev - 1].end - a.begin;
-    with_q(Q, [&](auto q) { launch(k_outlet<decltype(q)::value, S>, blocks_for(n, kMomBlock<S>), kMomBlock<S>, st, a); });
+    with_q(Q, [&](auto q) { k_outlet<decltype(q)::value, S><<<blocks_for(n, kMomBlock<S>), kMomBlock<S>, 0, st>>>(a); });
     return 1;
   }
   static int source_moments(int Q, const MomentsArgs& a, cudaStream_t st) {

@@ -292,7 +292,6 @@ struct OutletArgs {  // links begin .. end of the last level, levels in order
   int64_t Ntot, begin;
   double rho_off, rho0;
   const double* q;    // wall distance of interpolated bounce-back links
-  int chain;          // host: launch as a programmatic dependent
 };
 
 // GFC source moments: one record of mom_stride(Q) values per source (compute
