@@ -258,6 +258,36 @@ def oracle_timings(seconds_each):
 OUTLETS = {"linear": 0, "zero-gradient": 1}
 
 
+def finest_stream_collide(row, launches, ms, Q, prec):
+    """The finest level's stream-collide as the captured steps time it (timing
+    mode 2).  row: the level's lbm_mesh_info; launches, ms: its counts and times
+    per kind: 0 the interior bricks, 2 the launch of the boundary bricks and the
+    neighbour-list elements, 7 the span of both, which run as parallel graph
+    branches.  The kernel reported is that of the interior bricks, or the other
+    one where the level has none."""
+    interior, boundary = int(64 * row[8]), int(64 * row[9])
+    in_list = int(row[1]) - interior - boundary
+    brick, through_list = bytes_per_update(Q, prec, brick=True), bytes_per_update(Q, prec)
+    rest_bytes = boundary * brick + in_list * through_list
+    kind = 0 if interior else 2
+    units, nbytes = (interior, interior * brick) if interior else (boundary + in_list, rest_bytes)
+
+    def mean(k):
+        return float(ms[k] / launches[k]) if launches[k] > 0 else None
+
+    def rate(b, t):
+        return b / (t * 1e-3) / 1e9 if t else None
+
+    t, span = mean(kind), mean(7)
+    return {"finest_sc": {"span_ms": span, "bytes": interior * brick + rest_bytes, "units": int(row[1]),
+                          "gbs": rate(interior * brick + rest_bytes, span)},
+            "finest_kernel": "k_sc_interior" if interior else "k_sc_rest", "finest_launches": int(launches[kind]),
+            "finest_units": units, "finest_bytes": nbytes, "bytes_per_update": nbytes / units if units else brick,
+            "finest_launch_ms": t, "finest_gbs": rate(nbytes, t),
+            "finest_boundary_units": boundary, "finest_list_units": in_list,
+            "finest_rest_launch_ms": mean(2), "finest_rest_gbs": rate(rest_bytes, mean(2))}
+
+
 def run_gpu(mesh, Q, om, uin, fields, prec, K, W_, device, dist=None, want_moments=False, outlet=0,
             timing=2, breakdown=True, state=None, time_mode=0):
     """Time K coarse steps after W_ warm-up steps, the way a caller's
@@ -307,17 +337,7 @@ def run_gpu(mesh, Q, om, uin, fields, prec, K, W_, device, dist=None, want_momen
     ms = max_over_ranks(ms, dist, device)
     finest = len(info) - 1
     nlev = len(info)
-    # dominant kernel: the interior-brick stream-collide of the finest level
-    # (the neighbour-list kernel when the level has no interior bricks)
-    kb = 0 if info[finest, 8] > 0 else 1
-    units = int(64 * info[finest, 8]) if kb == 0 else int(info[finest, 1])
-    timed = timing == 2 and nl[finest, kb] > 0
-    avg_ms = kms[finest, kb] / nl[finest, kb] if timed else float("nan")
-    bpu = bytes_per_update(Q, prec, brick=kb == 0)
-    list_units = int(info[finest, 1] - 64 * (info[finest, 8] + info[finest, 9]))
-    list_ms = kms[finest, 1] / max(nl[finest, 1], 1)
-    bnd_units = int(64 * info[finest, 9])
-    bnd_ms = kms[finest, 2] / max(nl[finest, 2], 1)
+    fin = finest_stream_collide(info[finest], nl[finest], kms[finest], Q, prec)
     # algorithmic bytes of one coarse step: every level's interior and boundary
     # bricks at the brick rate, the rest at the neighbour-list rate, times its
     # substeps per coarse step
@@ -325,27 +345,10 @@ def run_gpu(mesh, Q, om, uin, fields, prec, K, W_, device, dist=None, want_momen
     step_bytes = float(sum(msub ** li * (brick_units[li] * bytes_per_update(Q, prec, brick=True)
                                         + (info[li, 1] - brick_units[li]) * bytes_per_update(Q, prec))
                            for li in range(nlev)))
-    # the finest level's stream-collide as one op: its two kernels run as
-    # parallel graph branches, timed from fork to join (timing kind 7)
-    span_ms = kms[finest, 7] / nl[finest, 7] if timing == 2 and nl[finest, 7] > 0 else None
-    sc_bytes = (units * bpu + bnd_units * bytes_per_update(Q, prec, brick=True)
-                + list_units * bytes_per_update(Q, prec)) if kb == 0 else units * bpu
-    res_sc = {"span_ms": span_ms, "bytes": sc_bytes, "units": int(info[finest, 1]),
-              "gbs": sc_bytes / (span_ms * 1e-3) / 1e9 if span_ms else None}
-    res = {"ms_total": ms, "ms_per_step": ms / K, "mlups": K * U / (ms * 1e-3) / 1e6, "launches": launches,
-           "finest_sc": res_sc,
-           "finest_kernel": "k_sc_interior" if kb == 0 else "k_sc_rest",
-           "finest_launch_ms": avg_ms, "finest_launches": int(nl[finest, kb]), "finest_units": units,
-           "finest_bytes": units * bpu, "finest_gbs": units * bpu / (avg_ms * 1e-3) / 1e9 if timed else None,
-           "finest_list_units": list_units, "finest_list_launch_ms": list_ms,
-           "finest_boundary_units": bnd_units, "finest_boundary_launch_ms": bnd_ms,
-           "finest_boundary_gbs": (bnd_units * bytes_per_update(Q, prec, brick=True) / (bnd_ms * 1e-3) / 1e9
-                                   if nl[finest, 2] > 0 and bnd_ms > 0 else None),
-           "finest_list_gbs": (list_units * bytes_per_update(Q, prec) / (list_ms * 1e-3) / 1e9
-                               if nl[finest, 1] > 0 and list_ms > 0 else None),
+    res = {"ms_total": ms, "ms_per_step": ms / K, "mlups": K * U / (ms * 1e-3) / 1e6, "launches": launches, **fin,
            "interior_fraction": float(64 * info[:, 8].sum() / info[:, 1].sum()),
            "brick_fraction": float(64 * (info[:, 8] + info[:, 9]).sum() / info[:, 1].sum()),
-           "step_bytes": step_bytes, "bytes_per_update": bpu, "build_s": t_build,
+           "step_bytes": step_bytes, "build_s": t_build,
            "device_gb": sim.device_bytes() / 1e9}
     if breakdown:
         sim.timing_enable(1)
@@ -366,14 +369,12 @@ def run_gpu(mesh, Q, om, uin, fields, prec, K, W_, device, dist=None, want_momen
                                                             for i, k in enumerate(KINDS) if nl1[li, i] > 0}
                                     for li in range(nlev)}
         # the finest level's boundary-brick and neighbour-list kernels launched
-        # alone (in the graph they run beside the interior bricks, and their
-        # events there span the shared time)
+        # alone (in the graph one launch takes both, beside the interior bricks)
         for kind, key, brick in ((2, "boundary", True), (1, "list", False)):
-            n_ = bnd_units if kind == 2 else list_units
-            if nl1[finest, kind] > 0 and n_ > 0:
-                t_ = kms1[finest, kind] / nl1[finest, kind]
-                res[f"finest_{key}_launch_ms"] = float(t_)
-                res[f"finest_{key}_gbs"] = n_ * bytes_per_update(Q, prec, brick=brick) / (t_ * 1e-3) / 1e9
+            n_ = res[f"finest_{key}_units"]
+            t_ = float(kms1[finest, kind] / nl1[finest, kind]) if nl1[finest, kind] > 0 and n_ > 0 else None
+            res[f"finest_{key}_launch_ms"] = t_
+            res[f"finest_{key}_gbs"] = n_ * bytes_per_update(Q, prec, brick=brick) / (t_ * 1e-3) / 1e9 if t_ else None
         # every level's brick stream-collide against the HBM roofline
         res["level_brick_gbs"] = {}
         for li in range(nlev):
@@ -668,8 +669,8 @@ def main():
                "how": "lbm_alu_peak: register-only multiply-add chains on every SM, CUDA events, 2 flop per FMA"}
         irec = fp64_instruction_record()
         v = rec["fp64"]
-        # element updates / s of the finest level's stream-collide (all three
-        # kernels, fork to join; they share the FP64 pipe)
+        # element updates / s of the finest level's stream-collide (both kernels,
+        # fork to join; they share the FP64 pipe)
         fsc = v["finest_sc"]
         rate = (fsc["units"] / (fsc["span_ms"] * 1e-3) if fsc["span_ms"]
                 else v["finest_units"] / (v["finest_launch_ms"] * 1e-3))
@@ -765,7 +766,8 @@ def main():
                        l2="inputs larger than L2 (%.1f GB workspace)" % r["device_gb"],
                        timing="K coarse steps through lbm_step's captured two-step CUDA graphs, CUDA events on the "
                               "bound stream around the region; the graphs also record events around the finest "
-                              "level's stream-collide (roofline: the last replay's 32 finest-level spans)"),
+                              "level's stream-collide (roofline: the last replay's instants at which that "
+                              "level advances alone)"),
         "roofline": {"bound": "hbm", "achieved": sc["gbs"], "peak": peak, "unit": "GB/s",
                      "frac": sc["gbs"] / peak,
                      "traffic": traffic,

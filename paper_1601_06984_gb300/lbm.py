@@ -284,7 +284,10 @@ class Sim:
         """Launches and summed device ms since enabled, arrays [level, kind]
         with kind 0 = interior-brick stream-collide, 1 = neighbour-list
         stream-collide, 2 = boundary-brick stream-collide, 3 = GhostFromFiner,
-        4 = source moments, 5 = GhostFromCoarser, 6 = outlet values."""
+        4 = source moments, 5 = GhostFromCoarser, 6 = outlet values, 7 = span of
+        a level's stream-collide.  Mode 2 gives kinds 0, 2 and 7 of the finest
+        level, from the most recent replay and where it advances alone; its kind
+        2 is the launch of the boundary bricks and the neighbour-list elements."""
         k = len(self.TIMED_KINDS)
         n = np.zeros(16 * k, np.int64)
         ms = np.zeros(16 * k)
