@@ -27,8 +27,9 @@ enum StepOp { OP_GFF = 0, OP_MOM_A = 1, OP_GFC_A = 2, OP_SC = 3, OP_MOM_B = 4, O
 constexpr int64_t kChainElements = 1 << 20, kChainElements64 = 1 << 12;
 // Instants of at most this many elements run all interior bricks beside the
 // GhostFromCoarser fill (us per coarse step, beside / after: cylinder 54.5 /
-// 57.3, two-level 64^3 44.9 / 45.7, D3Q27 9e5 elements 131 / 132; beyond it the
-// sphere of 1.1e7 elements took 7.4 against 4.94 ms).
+// 57.3, two-level 64^3 44.9 / 45.7, D3Q27 9e5 elements 131 / 132; four-level
+// sphere of 3.6e6 elements BF16 915 / 750, FP32 1022 / 992, two-level 160^3 372 /
+// 367; the sphere of 1.1e7 elements took 7.4 against 4.94 ms).
 constexpr int64_t kBesideElements = 1 << 20;
 // Graphs of meshes within kBesideElements give the chain of fills and the rest
 // one level of priority more than the interior bricks: its blocks, on the
