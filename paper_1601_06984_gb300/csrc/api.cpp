@@ -1036,10 +1036,13 @@ lbm_status lbm_fill_ghosts(lbm_ctx* c) {
 // overwrites the whole array.
 static void touch_pages(void* p, size_t bytes) {
   if (!p || bytes < ((size_t)4 << 20)) return;
-  // pinned memory has its pages; device memory is for the copy to refuse
+  // pinned memory has its pages; device memory, or memory that the runtime
+  // cannot tell (the context is lost), is for the copy to refuse
   cudaPointerAttributes at{};
-  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) cudaGetLastError();
-  else if (at.type != cudaMemoryTypeUnregistered) return;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess || at.type != cudaMemoryTypeUnregistered) {
+    cudaGetLastError();
+    return;
+  }
   const size_t page = (size_t)std::max(4096l, sysconf(_SC_PAGESIZE));
   volatile char* b = static_cast<volatile char*>(p);
   const int64_t n = (int64_t)((bytes + page - 1) / page);
